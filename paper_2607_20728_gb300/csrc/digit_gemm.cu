@@ -1,0 +1,420 @@
+// FP64 GEMM on the BF16 tensor pipe by exact digit products (the error-free splitting of Ozaki, Ogita,
+// Oishi and Rump, Numer. Algorithms 59, 95 (2012)).
+//
+// GB300 issues two FP64 multiply-adds per clock and SM (0.53e12/s on the chip, measured) but 1024 BF16
+// ones through mma.sync, so a product that is spelled out in small integers is the faster FP64 product.
+// Every row of op(A) and column of op(B) is scaled by its own power of two and rounded to a fixed-point
+// number X of 56 bits, |X| <= 2^55; X is written in 8 balanced digits of base 128, each a BF16 integer
+// in [-64, 64].  Digit products are at most 2^12, so 128 of them for up to eight digit pairs sum exactly
+// in an FP32 accumulator (2^22 at most); the pairs (s, t) with s + t = g share one accumulator, g <= 8,
+// and the pairs with s + t > 8 (below 2^-62 of the largest product) are left out.  Every 128 k the
+// accumulators are read as integers (adding 1.5 * 2^23 leaves the integer in the mantissa) and summed
+// in two 64-bit integers, which nothing rounds; one rounding to FP64 per K slice is the only one after
+// the rounding of X.  What comes here instead of to the streaming kernels, with times, stands
+// at dgemm in linalg.cu.
+//
+// With ND = 4 digits (28 bits, groups s + t <= 4) the same kernel serves the products whose contract is
+// FP32 arithmetic on FP64 operands: finer operands than FP32's 24 bits and exact sums, 13 products
+// instead of 43.
+#include <algorithm>
+#include <cstdint>
+
+#include <cuda_bf16.h>
+
+#include "internal.cuh"
+
+namespace bse {
+namespace {
+
+constexpr int kKC = 32;             // k per staged chunk
+constexpr int kRawStride = kKC + 2;  // doubles per staged row (16-byte aligned, rows off the same banks)
+constexpr int kDigStride = kKC + 8;  // bf16 per digit row: ldmatrix reads 8 rows without bank conflicts
+constexpr int kMaxStrips = 10;      // 16-row strips of A and B per CTA
+constexpr int kRows = 16 * kMaxStrips;
+constexpr int kWarps = 16;
+constexpr int kFlush = 4;           // chunks between reads of the FP32 accumulators (128 k)
+constexpr int kBadExp = 1 << 28;    // row holds a non-finite value
+constexpr int kMaxSlice = 1 << 19;  // longest K slice
+
+// |x| < 2^e  ->  round(x 2^(kBits - e)), kBits = 7 ND - 1
+template <int ND>
+__device__ __forceinline__ long long to_fixed(double x, int e) {
+  const long long b = __double_as_longlong(x);
+  const int E = (int)((b >> 52) & 0x7ff);
+  unsigned long long m = (unsigned long long)b & 0xfffffffffffffull;
+  if (E) m |= 1ull << 52;
+  const int s = max(E, 1) - 1075 + (7 * ND - 1) - e;  // at most 2 for ND = 8
+  const int l = min(max(s, 0), 63), r = min(max(-s, 0), 63);  // (above 2: rows of denormals, or with infinities)
+  m <<= l;
+  m = (m + ((1ull << r) >> 1)) >> r;
+  return b < 0 ? -(long long)m : (long long)m;
+}
+// sum over all digits of 64 * 128^j: makes every balanced digit a plain 7-bit field
+template <int ND>
+__device__ __forceinline__ constexpr unsigned long long digit_bias() {
+  unsigned long long c = 0;
+  for (int j = 0; j < ND; ++j) c = c * 128 + 64;
+  return c;
+}
+
+__device__ __forceinline__ unsigned smem_addr(const void *p) {
+  return static_cast<unsigned>(__cvta_generic_to_shared(p));
+}
+__device__ __forceinline__ void cp_async8(void *dst, const void *src, bool valid) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_addr(dst)), "l"(src), "r"(valid ? 8 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void ldmatrix4(unsigned (&r)[4], unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+__device__ __forceinline__ void mma16816(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// smallest e with |x| < 2^e for a row whose largest |x| has the bits m (0: any e)
+__device__ __forceinline__ int exponent_of(unsigned long long m) {
+  const int E = (int)(m >> 52);
+  if (E == 0x7ff) return kBadExp;
+  return E ? E - 1022 : m ? 64 - __clzll(m) - 1074 : 0;
+}
+
+// Exponents of the rows of op(A) and the columns of op(B): the smallest e with |x| < 2^e over the row,
+// kBadExp when a value is not finite.  Rows that are contiguous in k take one CTA each; rows that lie
+// across the memory (k strides by ld) go 32 to a CTA, 8 k at a time, coalesced over the rows.
+__global__ void __launch_bounds__(256) row_exponents(int M, int N, int K, bool a_across, const double *__restrict__ A,
+                                                     int lda, bool b_across, const double *__restrict__ B, int ldb,
+                                                     int nblk_a, int *__restrict__ ex) {
+  __shared__ unsigned long long red[8][32];
+  const bool isb = (int)blockIdx.x >= nblk_a;
+  const int blk = isb ? blockIdx.x - nblk_a : blockIdx.x;
+  const bool across = isb ? b_across : a_across;
+  const double *X = isb ? B : A;
+  const int ld = isb ? ldb : lda, rows = isb ? N : M;
+  int *out = ex + (isb ? M : 0);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned long long m = 0;
+  auto bits = [](double x) { return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull; };
+  if (across) {
+    const int row = blk * 32 + lane;
+    if (row < rows)
+#pragma unroll 4
+      for (int k = warp; k < K; k += 8) m = max(m, bits(__ldg(&X[(long)k * ld + row])));
+    red[warp][lane] = m;
+    __syncthreads();
+    if (warp == 0 && row < rows) {
+      for (int w = 1; w < 8; ++w) m = max(m, red[w][lane]);
+      out[row] = exponent_of(m);
+    }
+  } else {
+    const double *x = X + (long)blk * ld;
+#pragma unroll 4
+    for (int k = threadIdx.x; k < K; k += 256) m = max(m, bits(__ldg(&x[k])));
+    for (int w = 16; w > 0; w >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, w));
+    if (lane == 0) red[0][warp] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < 8; ++w) m = max(m, red[0][w]);
+      out[blk] = exponent_of(m);
+    }
+  }
+}
+
+template <int ND>
+constexpr size_t digit_smem() {
+  return (size_t)kRows * kRawStride * 8 + (size_t)ND * kRows * kDigStride * 2 +
+         (ND == 8 ? (size_t)kWarps * 32 * 8 * 16 : 0) + kRows * 4;
+}
+
+// One CTA: SM x SN warps (at most 16), each a 16 x 16 block of C over k in its K slice; the SM strips of
+// A and SN strips of B (16 rows each) are staged as FP64 by cp.async, rewritten as digits by all threads
+// and multiplied from the digit planes.  The next chunk's FP64 rows arrive while this one is multiplied.
+// Bound by the tensor pipe (86 mma.sync of 2 clocks per warp and 16 k) and, beside it, the integer work
+// of the rewriting (about 40 instructions per value).  Strips past the end of C skip their products.
+template <bool TA, bool TB, int ND>
+__global__ void __launch_bounds__(kWarps * 32, 1)
+    digit_gemm_kernel(int M, int N, int K, int kslice, int SM, int SN, const double *__restrict__ A, int lda,
+                      const double *__restrict__ B, int ldb, const int *__restrict__ ex, double alpha, double beta,
+                      double *__restrict__ C, int ldc, double *__restrict__ part) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  double *raw = reinterpret_cast<double *>(smem);                                          // [rows][kRawStride]
+  __nv_bfloat16 *dig = reinterpret_cast<__nv_bfloat16 *>(raw + kRows * kRawStride);        // [ND][rows][kDigStride]
+  longlong2 *sums = reinterpret_cast<longlong2 *>(dig + (size_t)ND * kRows * kDigStride);  // [8][512] (ND = 8)
+  int *rexp = reinterpret_cast<int *>(reinterpret_cast<unsigned char *>(sums) +
+                                      (ND == 8 ? (size_t)kWarps * 32 * 8 * 16 : 0));
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rows_a = 16 * SM, rows = 16 * (SM + SN);
+  const int m0 = blockIdx.y * rows_a, n0 = blockIdx.x * 16 * SN;
+  const int kbeg = blockIdx.z * kslice, kend = min(K, kbeg + kslice);
+  for (int r = tid; r < rows; r += blockDim.x) {
+    const bool a = r < rows_a;
+    const int g = a ? m0 + r : n0 + r - rows_a;
+    int e = 0;
+    if (g < (a ? M : N)) e = ex[a ? g : M + g];
+    rexp[r] = e == kBadExp ? 0 : e;
+  }
+  auto load = [&](int k0) {
+    // 8-byte copies, consecutive threads along the contiguous direction of each operand
+    const int na = rows_a * kKC, nt = rows * kKC;
+    for (int i = tid; i < nt; i += kWarps * 32) {
+      const bool a = i < na;
+      const int j = a ? i : i - na;
+      int r, k;
+      if (a ? TA : !TB) {
+        const int nr = a ? rows_a : rows - rows_a;
+        k = j / nr;
+        r = j - k * nr;
+      } else {
+        r = j / kKC;
+        k = j % kKC;
+      }
+      const int g = (a ? m0 : n0) + r, gk = k0 + k;
+      const bool ok = g < (a ? M : N) && gk < kend;
+      const double *src = a ? A : B;
+      if (ok) src += a ? (TA ? (long)gk * lda + g : (long)g * lda + gk) : (TB ? (long)g * ldb + gk : (long)gk * ldb + g);
+      cp_async8(&raw[(a ? r : rows_a + r) * kRawStride + k], src, ok);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  const int wm = warp / SN, wn = warp - wm * SN;
+  const bool active = wm < SM && m0 + 16 * wm < M && n0 + 16 * wn < N;
+  const unsigned a_addr = smem_addr(dig + (16 * wm + (lane & 15)) * kDigStride + (lane >> 4) * 8);
+  const unsigned b_addr =
+      smem_addr(dig + (rows_a + 16 * wn + ((lane >> 4) << 3) + (lane & 7)) * kDigStride + ((lane >> 3) & 1) * 8);
+  constexpr unsigned kPlane = kRows * kDigStride * 2;
+  constexpr int NG = ND + 1;  // digit-pair groups s + t = 0 .. ND
+  float acc[NG][2][4];
+#pragma unroll
+  for (int g = 0; g < NG; ++g)
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[g][t][i] = 0.f;
+  long long one[ND == 8 ? 1 : 8];  // ND = 4: a single 64-bit sum per output, in registers
+  if constexpr (ND == 8) {
+#pragma unroll
+    for (int o = 0; o < 8; ++o) sums[o * (kWarps * 32) + tid] = make_longlong2(0, 0);
+  } else {
+#pragma unroll
+    for (int o = 0; o < 8; ++o) one[o] = 0;
+  }
+  load(kbeg);
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  int held = 0;
+  for (int k0 = kbeg; k0 < kend; k0 += kKC) {
+    // FP64 -> digits, two k per thread and step
+    for (int i = tid; i < rows * (kKC / 2); i += kWarps * 32) {
+      const int r = i / (kKC / 2), kp = i % (kKC / 2);
+      const double2 x = *reinterpret_cast<const double2 *>(&raw[r * kRawStride + 2 * kp]);
+      const int e = rexp[r];
+      const unsigned long long y0 = (unsigned long long)to_fixed<ND>(x.x, e) + digit_bias<ND>();
+      const unsigned long long y1 = (unsigned long long)to_fixed<ND>(x.y, e) + digit_bias<ND>();
+      unsigned *d = reinterpret_cast<unsigned *>(dig + r * kDigStride + 2 * kp);
+#pragma unroll
+      for (int s = 0; s < ND; ++s) {
+        const int sh = 7 * (ND - 1 - s);
+        // the leading field reaches 128; a 7-bit field u next to the BF16 bits of 128 reads 128 + u
+        const unsigned msk = s == 0 ? 0xffu : 0x7fu;
+        const unsigned u = ((unsigned)(y0 >> sh) & msk) + (((unsigned)(y1 >> sh) & msk) << 16) + 0x43004300u;
+        __nv_bfloat162 w = __hsub2(*reinterpret_cast<const __nv_bfloat162 *>(&u), __float2bfloat162_rn(192.f));
+        d[s * (kPlane / 4)] = *reinterpret_cast<const unsigned *>(&w);
+      }
+    }
+    __syncthreads();
+    if (k0 + kKC < kend) load(k0 + kKC);
+    if (active) {
+#pragma unroll
+      for (int kk = 0; kk < kKC / 16; ++kk) {
+        unsigned a[ND][4];
+#pragma unroll
+        for (int s = 0; s < ND; ++s) ldmatrix4(a[s], a_addr + s * kPlane + kk * 32);
+#pragma unroll
+        for (int t = 0; t < ND; ++t) {
+          unsigned b[4];
+          ldmatrix4(b, b_addr + t * kPlane + kk * 32);
+#pragma unroll
+          for (int s = 0; s < ND && s + t < NG; ++s) {
+            mma16816(acc[s + t][0], a[s], b[0], b[1]);
+            mma16816(acc[s + t][1], a[s], b[2], b[3]);
+          }
+        }
+      }
+      if (++held == kFlush || k0 + kKC >= kend) {
+        held = 0;
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            int v[NG];
+#pragma unroll
+            for (int g = 0; g < NG; ++g) {
+              v[g] = __float_as_int(acc[g][t][i] + 12582912.f) - 0x4B400000;
+              acc[g][t][i] = 0.f;
+            }
+            if constexpr (ND == 8) {
+              longlong2 &s = sums[(t * 4 + i) * (kWarps * 32) + tid];
+              longlong2 x = s;
+              x.x += (((long long)v[0] * 128 + v[1]) * 128 + v[2]) * 128 + v[3];
+              x.y += ((((long long)v[4] * 128 + v[5]) * 128 + v[6]) * 128 + v[7]) * 128 + v[8];
+              s = x;
+            } else {
+              one[t * 4 + i] += ((((long long)v[0] * 128 + v[1]) * 128 + v[2]) * 128 + v[3]) * 128 + v[4];
+            }
+          }
+      }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+  }
+  if (!active) return;
+  if (part) part += (long)blockIdx.z * M * N;
+#pragma unroll
+  for (int t = 0; t < 2; ++t)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int m = m0 + 16 * wm + (lane >> 2) + (i >> 1) * 8;
+      const int n = n0 + 16 * wn + t * 8 + (lane & 3) * 2 + (i & 1);
+      if (m >= M || n >= N) continue;
+      const int ea = ex[m], eb = ex[M + n];
+      double v;
+      if (ea == kBadExp || eb == kBadExp) {
+        // infinities and NaN follow the plain FP64 sum
+        v = 0.0;
+        for (int k = kbeg; k < kend; ++k)
+          v = fma(TA ? A[(long)k * lda + m] : A[(long)m * lda + k], TB ? B[(long)n * ldb + k] : B[(long)k * ldb + n], v);
+      } else if constexpr (ND == 8) {
+        // group g weighs 128^(14 - g) of 2^(ea + eb - 110)
+        const longlong2 s = sums[(t * 4 + i) * (kWarps * 32) + tid];
+        v = ldexp(fma((double)s.x, 34359738368.0, (double)s.y), ea + eb - 110 + 42);
+      } else {
+        // group g weighs 128^(6 - g) of 2^(ea + eb - 54)
+        v = ldexp((double)one[t * 4 + i], ea + eb - 54 + 14);
+      }
+      if (part) {
+        part[(long)m * N + n] = v;
+      } else {
+        double *c = C + (long)m * ldc + n;
+        *c = beta == 0.0 ? alpha * v : alpha * v + beta * (*c);
+      }
+    }
+}
+
+// C = alpha sum_z part[z] + beta C, four slices in flight per thread
+__global__ void __launch_bounds__(128) digit_reduce(int M, int N, int nsplit, const double *__restrict__ part,
+                                                    double alpha, double beta, double *__restrict__ C, int ldc) {
+  const long total = (long)M * N;
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
+    double s0 = 0, s1 = 0, s2 = 0, s3 = 0;
+    int z = 0;
+    for (; z + 4 <= nsplit; z += 4) {
+      s0 += part[(long)z * total + i];
+      s1 += part[(long)(z + 1) * total + i];
+      s2 += part[(long)(z + 2) * total + i];
+      s3 += part[(long)(z + 3) * total + i];
+    }
+    for (; z < nsplit; ++z) s0 += part[(long)z * total + i];
+    const double s = (s0 + s1) + (s2 + s3);
+    double *c = C + (i / N) * ldc + (i % N);
+    *c = beta == 0.0 ? alpha * s : alpha * s + beta * (*c);
+  }
+}
+
+// Strips per CTA and K slices: the fewest clocks by a model of one CTA per SM, a chunk costing 1900
+// clocks of staging and rewriting plus 344 (ND = 8; 104 for ND = 4) per active warp, a CTA 8000 more.
+struct Shape {
+  int sm, sn, kslice, nsplit;
+};
+Shape choose(int M, int N, int K, int nd, size_t part_cap) {
+  static const int opts[][2] = {{4, 4}, {5, 3}, {3, 5}, {2, 8}, {8, 2}, {6, 2}, {2, 6}, {3, 3}, {2, 4}, {4, 2}, {2, 2},
+                                {1, 9}, {9, 1}, {1, 4}, {4, 1}, {1, 1}};
+  const int ms = (M + 15) / 16, ns = (N + 15) / 16;
+  const double per_warp = nd == 8 ? 344.0 : 104.0;
+  Shape best{4, 4, K, 1};
+  double bc = 1e300;
+  for (auto &o : opts) {
+    const int sm = o[0], sn = o[1];
+    if (sm > ms + 1 || sn > ns + 1) continue;
+    const long tiles = (long)((ms + sm - 1) / sm) * ((ns + sn - 1) / sn);
+    const double load = 1900.0 * (sm + sn) / 8.0 + per_warp * std::min(sm, ms) * std::min(sn, ns);
+    // a slice of at most kMaxSlice k keeps the 64-bit sums in range (2^50 per 128 k)
+    const int mins = (K + kMaxSlice - 1) / kMaxSlice;
+    const int maxs = (int)std::max(mins, std::min(K / 64, 128));
+    for (int s = mins; s <= maxs; ++s) {
+      if (s > mins && (size_t)s * M * N > part_cap) break;
+      const int chunks = (K + kKC - 1) / kKC;
+      const int per = (chunks + s - 1) / s;
+      const int sr = (chunks + per - 1) / per;
+      if (sr != s) continue;
+      const double waves = (double)((tiles * s + 151) / 152);
+      const double cost = waves * (per * load + 8000.0) + (s > 1 ? 4000.0 + 0.01 * s * M * N / 152.0 * 8 : 0.0);
+      if (cost < bc) {
+        bc = cost;
+        best = {sm, sn, per * kKC, sr};
+      }
+    }
+  }
+  return best;
+}
+
+template <bool TA, bool TB, int ND>
+void go(dim3 grid, cudaStream_t s, int M, int N, int K, const Shape &h, const double *A, int lda, const double *B,
+        int ldb, const int *ex, double alpha, double beta, double *C, int ldc, double *part) {
+  BSE_CUDA(cudaFuncSetAttribute(digit_gemm_kernel<TA, TB, ND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)digit_smem<ND>()));
+  digit_gemm_kernel<TA, TB, ND><<<grid, kWarps * 32, digit_smem<ND>(), s>>>(M, N, K, h.kslice, h.sm, h.sn, A, lda, B,
+                                                                           ldb, ex, alpha, beta, C, ldc, part);
+  BSE_CHECK_LAUNCH();
+}
+
+template <int ND>
+void run(char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda, const double *B, int ldb,
+         double beta, double *C, int ldc, cudaStream_t s, DevBuf<double> &scratch, bool fixed, int split_pct) {
+  const size_t nex = ((size_t)M + N + 1) / 2;  // exponents, in doubles, ahead of the partial sums
+  const size_t cap = fixed ? (scratch.n > nex ? scratch.n - nex : 0) : (size_t)1 << 26;
+  Shape h = choose(M, N, K, ND, cap);
+  if (split_pct != 100) {
+    // the autotuner's variation of the number of K slices
+    const int chunks = (K + kKC - 1) / kKC;
+    int ns = std::max(1, std::min(chunks, h.nsplit * split_pct / 100));
+    if (ns > 1) ns = (int)std::max<size_t>(1, std::min<size_t>(ns, cap / ((size_t)M * N)));
+    ns = std::max(ns, (K + kMaxSlice - 1) / kMaxSlice);
+    const int per = (chunks + ns - 1) / ns;
+    h.kslice = per * kKC;
+    h.nsplit = (chunks + per - 1) / per;
+  }
+  if (!fixed) scratch.alloc(nex + (h.nsplit > 1 ? (size_t)h.nsplit * M * N : 0));
+  int *ex = reinterpret_cast<int *>(scratch.get());
+  double *part = h.nsplit > 1 ? scratch.get() + nex : nullptr;
+  const bool TA = ta == 'T', TB = tb == 'T';
+  const int ba = TA ? (M + 31) / 32 : M, bb = TB ? N : (N + 31) / 32;
+  row_exponents<<<ba + bb, 256, 0, s>>>(M, N, K, TA, A, lda, !TB, B, ldb, ba, ex);
+  BSE_CHECK_LAUNCH();
+  const dim3 grid((unsigned)((N + 16 * h.sn - 1) / (16 * h.sn)), (unsigned)((M + 16 * h.sm - 1) / (16 * h.sm)),
+                  (unsigned)h.nsplit);
+  if (!TA && !TB) go<false, false, ND>(grid, s, M, N, K, h, A, lda, B, ldb, ex, alpha, beta, C, ldc, part);
+  else if (!TA && TB) go<false, true, ND>(grid, s, M, N, K, h, A, lda, B, ldb, ex, alpha, beta, C, ldc, part);
+  else if (TA && !TB) go<true, false, ND>(grid, s, M, N, K, h, A, lda, B, ldb, ex, alpha, beta, C, ldc, part);
+  else go<true, true, ND>(grid, s, M, N, K, h, A, lda, B, ldb, ex, alpha, beta, C, ldc, part);
+  if (part) {
+    const long total = (long)M * N;
+    digit_reduce<<<(int)std::min<long>(152 * 16, (total + 127) / 128), 128, 0, s>>>(M, N, h.nsplit, part, alpha, beta, C,
+                                                                                  ldc);
+    BSE_CHECK_LAUNCH();
+  }
+}
+
+}  // namespace
+
+void digit_gemm(int digits, char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda,
+                const double *B, int ldb, double beta, double *C, int ldc, cudaStream_t s, DevBuf<double> &scratch,
+                bool fixed, int split_pct) {
+  if (digits == 8) run<8>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, scratch, fixed, split_pct);
+  else run<4>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, scratch, fixed, split_pct);
+}
+
+}  // namespace bse

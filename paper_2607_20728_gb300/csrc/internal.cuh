@@ -125,6 +125,12 @@ void sgemm(char ta, char tb, int M, int N, int K, float alpha, const float *A, i
 // are rounded to FP32 as they are staged, alpha, beta and the sum over K slices are applied in FP64
 void mgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda, const double *B, int ldb,
            double beta, double *C, int ldc, cudaStream_t s, int split_pct = 100);
+// the same product from exact BF16 digit products on the tensor pipe (digit_gemm.cu): digits = 8 for
+// FP64 results, 4 where dgemm's callers ask for FP32 arithmetic.  scratch: row exponents and split-K
+// partial sums, grown on demand unless fixed
+void digit_gemm(int digits, char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda,
+                const double *B, int ldb, double beta, double *C, int ldc, cudaStream_t s, DevBuf<double> &scratch,
+                bool fixed, int split_pct = 100);
 // out[i] = sum_j X[i][j] * Y[i][j] for i < rows (part: scratch of the partial sums; the default is
 // a per-thread buffer)
 void rowdot(int rows, long len, const double *X, const double *Y, double *out, cudaStream_t s,

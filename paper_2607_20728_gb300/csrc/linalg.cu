@@ -24,13 +24,12 @@ constexpr int BM = 64, BN = 64, BK = 16;
 
 // C = alpha op(A) op(B) + beta C over k in [kz * kchunk, min(K, (kz + 1) kchunk)), kz = blockIdx.z.
 // With split-K (gridDim.z > 1) each slice writes its own partial matrix C + kz * M * ldc.
-// T: the arithmetic type of the products and sums; TI: the operands' type in memory (rounded to
-// T as the tiles are staged); TO: the output's type (alpha and beta applied in TO)
-template <bool TA, bool TB, class T, class TI = T, class TO = T>
-__global__ void __launch_bounds__(256) dgemm_kernel(int M, int N, int K, int kchunk, TO alpha,
-                                                    const TI *__restrict__ A, int lda,
-                                                    const TI *__restrict__ B, int ldb,
-                                                    TO beta, TO *__restrict__ C, int ldc) {
+// The FP32 products of the mixed form's operators (FP64 products go through digit_gemm.cu).
+template <bool TA, bool TB, class T>
+__global__ void __launch_bounds__(256) sgemm_kernel(int M, int N, int K, int kchunk, T alpha,
+                                                    const T *__restrict__ A, int lda,
+                                                    const T *__restrict__ B, int ldb,
+                                                    T beta, T *__restrict__ C, int ldc) {
   __shared__ T As[BK][BM + 2];
   __shared__ T Bs[BK][BN + 2];
   const int tid = threadIdx.x;
@@ -52,7 +51,7 @@ __global__ void __launch_bounds__(256) dgemm_kernel(int M, int N, int K, int kch
       if (!TA) { k = e % BK; m = e / BK; } else { m = e % BM; k = e / BM; }
       const int gm = m0 + m, gk = k0 + k;
       T v = 0;
-      if (gm < M && gk < kend) v = (T)(TA ? A[(long)gk * lda + gm] : A[(long)gm * lda + gk]);
+      if (gm < M && gk < kend) v = TA ? A[(long)gk * lda + gm] : A[(long)gm * lda + gk];
       As[k][m] = v;
     }
 #pragma unroll
@@ -62,7 +61,7 @@ __global__ void __launch_bounds__(256) dgemm_kernel(int M, int N, int K, int kch
       if (!TB) { n = e % BN; k = e / BN; } else { k = e % BK; n = e / BK; }
       const int gn = n0 + n, gk = k0 + k;
       T v = 0;
-      if (gn < N && gk < kend) v = (T)(TB ? B[(long)gn * ldb + gk] : B[(long)gk * ldb + gn]);
+      if (gn < N && gk < kend) v = TB ? B[(long)gn * ldb + gk] : B[(long)gk * ldb + gn];
       Bs[k][n] = v;
     }
     __syncthreads();
@@ -88,20 +87,12 @@ __global__ void __launch_bounds__(256) dgemm_kernel(int M, int N, int K, int kch
     for (int j = 0; j < 4; ++j) {
       const int gn = n0 + tx + 16 * j;
       if (gn >= N) continue;
-      TO *c = C + (long)gm * ldc + gn;
-      const TO v = (TO)acc[i][j];
-      *c = beta == (TO)0 ? alpha * v : alpha * v + beta * (*c);
+      T *c = C + (long)gm * ldc + gn;
+      const T v = acc[i][j];
+      *c = beta == (T)0 ? alpha * v : alpha * v + beta * (*c);
     }
   }
 }
-
-// Small-output NT product: C[i][j] = sum_k A[i][k] B[j][k] for M*N <= 4096 outputs and long K.
-// Each CTA stages K-chunks of the M + N rows in shared memory; every output is owned by a group
-// of tpo adjacent lanes (tpo a power of two <= 32, so that small outputs still occupy the CTA)
-// which accumulate interleaved k in registers over the CTA's chunks and are summed by shuffles;
-// part[cta][M][N] is reduced afterwards.
-constexpr int kSmallOut = 4096;
-constexpr int kSmallPerThread = kSmallOut / 256;
 
 // Skinny inner products for at most four rows of A: part[z][i][j] = sum over the z-th K slice of
 // A[i][k] B[j][k] for i < MM and the kSkinnyRows rows j of B this block takes.  Threads stream
@@ -175,56 +166,6 @@ __global__ void __launch_bounds__(256) gemm_nt_skinny_kernel(int N, int K, int k
   }
 }
 
-__global__ void __launch_bounds__(256) gemm_nt_small_kernel(int M, int N, int K, int L, int tpo,
-                                                            const double *__restrict__ A, int lda,
-                                                            const double *__restrict__ B, int ldb,
-                                                            double *__restrict__ part) {
-  extern __shared__ double sh[];
-  const int Lp = L + 1;  // padded row stride against bank conflicts
-  double *As = sh;
-  double *Bs = sh + (size_t)M * Lp;
-  const int MN = M * N;
-  const int slots = MN * tpo;
-  const int j = threadIdx.x & (tpo - 1);
-  double acc[kSmallPerThread];
-#pragma unroll
-  for (int q = 0; q < kSmallPerThread; ++q) acc[q] = 0.0;
-  const int nchunk = (K + L - 1) / L;
-  for (int ch = blockIdx.x; ch < nchunk; ch += gridDim.x) {
-    const int k0 = ch * L;
-    const int len = min(L, K - k0);
-    for (int e = threadIdx.x; e < (M + N) * L; e += blockDim.x) {
-      const int row = e / L, l = e - row * L;
-      double v = 0.0;
-      if (l < len) v = row < M ? A[(long)row * lda + k0 + l] : B[(long)(row - M) * ldb + k0 + l];
-      sh[(size_t)row * Lp + l] = v;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < kSmallPerThread; ++q) {
-      const int idx = threadIdx.x + q * 256;
-      if (idx < slots) {
-        const int o = idx / tpo;
-        const int i = o / N, jj = o - i * N;
-        const double *a = As + (size_t)i * Lp;
-        const double *b = Bs + (size_t)jj * Lp;
-        double s = acc[q];
-        for (int l = j; l < len; l += tpo) s = fma(a[l], b[l], s);
-        acc[q] = s;
-      }
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int q = 0; q < kSmallPerThread; ++q) {
-    const int idx = threadIdx.x + q * 256;
-    if ((idx & ~31) >= slots) break;  // warp-uniform: every lane of the warp takes the shuffles
-    double s = acc[q];                  // zero for slots past the end (whole groups of tpo lanes)
-    for (int w = 1; w < tpo; w <<= 1) s += __shfl_xor_sync(0xffffffffu, s, w);
-    if (j == 0 && idx < slots) part[(long)blockIdx.x * MN + idx / tpo] = s;
-  }
-}
-
 // Small-M product C = alpha op(A) B + beta C, op(A) M x K with M <= 16, K <= 1024, B [K][N]:
 // op(A) in shared memory, one output column per thread, B read once with eight rows in flight
 // per thread (the product is a stream over B).  MT is M at compile time (0: run-time M).
@@ -277,14 +218,14 @@ __global__ void __launch_bounds__(256) gemm_smallm_kernel(int M_, int N, int K, 
   }
 }
 
-// C = alpha sum_z part[z] + beta C; the partial sums (type TP) are added in the output's type T
-template <class T, class TP = T>
-__global__ void splitk_reduce(int M, int N, int nsplit, const TP *__restrict__ part, T alpha, T beta,
+// C = alpha sum_z part[z] + beta C
+template <class T>
+__global__ void splitk_reduce(int M, int N, int nsplit, const T *__restrict__ part, T alpha, T beta,
                               T *__restrict__ C, int ldc) {
   const long total = (long)M * N;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
     T s = 0;
-    for (int z = 0; z < nsplit; ++z) s += (T)part[(long)z * total + i];
+    for (int z = 0; z < nsplit; ++z) s += part[(long)z * total + i];
     T *c = C + (i / N) * ldc + (i % N);
     *c = beta == (T)0 ? alpha * s : alpha * s + beta * (*c);
   }
@@ -405,10 +346,10 @@ void gemm_tiled(char ta, char tb, int M, int N, int K, T alpha, const T *A, int 
   }
   dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, nsplit);
   const bool TA = (ta == 'T'), TB = (tb == 'T');
-  if (!TA && !TB) dgemm_kernel<false, false, T><<<grid, 256, 0, s>>>(M, N, K, kchunk, a, A, lda, B, ldb, b, Cout, ldo);
-  else if (!TA && TB) dgemm_kernel<false, true, T><<<grid, 256, 0, s>>>(M, N, K, kchunk, a, A, lda, B, ldb, b, Cout, ldo);
-  else if (TA && !TB) dgemm_kernel<true, false, T><<<grid, 256, 0, s>>>(M, N, K, kchunk, a, A, lda, B, ldb, b, Cout, ldo);
-  else dgemm_kernel<true, true, T><<<grid, 256, 0, s>>>(M, N, K, kchunk, a, A, lda, B, ldb, b, Cout, ldo);
+  if (!TA && !TB) sgemm_kernel<false, false, T><<<grid, 256, 0, s>>>(M, N, K, kchunk, a, A, lda, B, ldb, b, Cout, ldo);
+  else if (!TA && TB) sgemm_kernel<false, true, T><<<grid, 256, 0, s>>>(M, N, K, kchunk, a, A, lda, B, ldb, b, Cout, ldo);
+  else if (TA && !TB) sgemm_kernel<true, false, T><<<grid, 256, 0, s>>>(M, N, K, kchunk, a, A, lda, B, ldb, b, Cout, ldo);
+  else sgemm_kernel<true, true, T><<<grid, 256, 0, s>>>(M, N, K, kchunk, a, A, lda, B, ldb, b, Cout, ldo);
   BSE_CHECK_LAUNCH();
   if (nsplit > 1) {
     const long total = (long)M * N;
@@ -416,44 +357,6 @@ void gemm_tiled(char ta, char tb, int M, int N, int K, T alpha, const T *A, int 
                                                                                      C, ldc);
     BSE_CHECK_LAUNCH();
   }
-}
-
-// FP64 operands and output, FP32 products and sums: the tiles are rounded to FP32 as they are
-// staged, each split-K slice writes FP32 partial sums, and alpha, beta and the sum over slices are
-// applied in FP64 (one launch, or two with a split over K)
-void gemm_tiled_mixed(char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda, const double *B,
-                      int ldb, double beta, double *C, int ldc, cudaStream_t s, DevBuf<float> &scratch,
-                      int split_pct) {
-  const long tiles = (long)((N + BN - 1) / BN) * ((M + BM - 1) / BM);
-  int nsplit0 = split_for(tiles, K);
-  if (split_pct != 100) nsplit0 = std::max(1, std::min(K / BK, nsplit0 * split_pct / 100));
-  int kchunk = (K + nsplit0 - 1) / nsplit0;
-  kchunk = (kchunk + BK - 1) / BK * BK;
-  const int nsplit = (K + kchunk - 1) / kchunk;
-  dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, nsplit);
-  const bool TA = (ta == 'T'), TB = (tb == 'T');
-  auto go = [&](auto out, auto a, auto b, int ldo) {
-    using TO = std::remove_pointer_t<decltype(out)>;
-    if (!TA && !TB)
-      dgemm_kernel<false, false, float, double, TO><<<grid, 256, 0, s>>>(M, N, K, kchunk, a, A, lda, B, ldb, b, out, ldo);
-    else if (!TA && TB)
-      dgemm_kernel<false, true, float, double, TO><<<grid, 256, 0, s>>>(M, N, K, kchunk, a, A, lda, B, ldb, b, out, ldo);
-    else if (TA && !TB)
-      dgemm_kernel<true, false, float, double, TO><<<grid, 256, 0, s>>>(M, N, K, kchunk, a, A, lda, B, ldb, b, out, ldo);
-    else
-      dgemm_kernel<true, true, float, double, TO><<<grid, 256, 0, s>>>(M, N, K, kchunk, a, A, lda, B, ldb, b, out, ldo);
-    BSE_CHECK_LAUNCH();
-  };
-  if (nsplit == 1) {
-    go(C, alpha, beta, ldc);
-    return;
-  }
-  scratch.alloc((size_t)nsplit * M * N);
-  go(scratch.get(), 1.0f, 0.0f, N);
-  const long total = (long)M * N;
-  splitk_reduce<double, float><<<(int)std::min<long>(4096, (total + 255) / 256), 256, 0, s>>>(
-      M, N, nsplit, scratch.get(), alpha, beta, C, ldc);
-  BSE_CHECK_LAUNCH();
 }
 
 }  // namespace
@@ -526,32 +429,10 @@ void dgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A,
     }
     return;
   }
-  // tall-skinny inner products: every output of a small M x N block over a long K
-  if (ta == 'N' && tb == 'T' && (long)M * N <= kSmallOut && M + N <= 1024 && K >= 4096 &&
-      (!fixed || fixed->n >= (size_t)M * N)) {
-    // chunks of L k-values: about two CTAs per SM when K allows, at most 96 KB of staging
-    int tpo = 1;
-    while (tpo < 32 && (long)M * N * tpo * 2 <= 256) tpo *= 2;
-    const int lmax = std::min(256, (int)(96 * 1024 / ((M + N) * sizeof(double))) - 1) / 8 * 8;
-    int L = (int)std::min<long>(lmax, std::max<long>(8, ((K + 2 * 152 - 1) / (2 * 152) + 7) / 8 * 8));
-    L = std::max(L, 8);
-    const int nchunk = (K + L - 1) / L;
-    int nct = std::min(nchunk, 2 * 152);
-    DevBuf<double> &p = fixed ? *fixed : splitk_buf();
-    if (fixed) nct = (int)std::min<size_t>(nct, fixed->n / ((size_t)M * N));
-    else p.alloc((size_t)nct * M * N);
-    const size_t smem = (size_t)(M + N) * (L + 1) * sizeof(double);
-    BSE_CUDA(cudaFuncSetAttribute(gemm_nt_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
-    gemm_nt_small_kernel<<<nct, 256, smem, s>>>(M, N, K, L, tpo, A, lda, B, ldb, p.get());
-    BSE_CHECK_LAUNCH();
-    const long total = (long)M * N;
-    splitk_reduce<double><<<(int)std::min<long>(4096, (total + 255) / 256), 256, 0, s>>>(M, N, nct, p.get(), alpha,
-                                                                                          beta, C, ldc);
-    BSE_CHECK_LAUNCH();
-    return;
-  }
-  // few output rows, short K, long N: one column per thread
-  if (tb == 'N' && M <= kSmallM && K <= 1024 && N >= 4096) {
+  // few output rows, short K, long N: one column per thread, a stream over B.  Against the digit form
+  // (exponent pass and rewriting of B), N = 200000: M = 2 K = 8 10 us (120), M = 2 K = 100 82 (343),
+  // M = 8 K = 8 64 (122), M = 8 K = 100 686 (347); N = 6859: M = 4 K = 64 19 (14), M = 8 K = 8 13 (11)
+  if (tb == 'N' && M <= kSmallM && K <= 1024 && N >= 4096 && (M <= 4 || M * K <= 96)) {
     const size_t smem = (size_t)M * K * sizeof(double);
     const int grid = (N + 255) / 256;
     auto go = [&](auto ta_c, auto mt_c) {
@@ -575,8 +456,13 @@ void dgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A,
     BSE_CHECK_LAUNCH();
     return;
   }
-  if (fixed) gemm_tiled<double>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, *fixed, true, split_pct);
-  else gemm_tiled<double>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, splitk_buf(), false, split_pct);
+  // everything else: exact digit products on the tensor pipe.  Kernel time against the tiled FP64 SIMT
+  // kernels that stood here (64 x 64 tiles, bound by the FP64 pipe or, below about 20 Mflop, by its
+  // latency): N T 80 x 216 x 6859 72 us (383 before), 200 x 216 x 922 34 (121), 128 x 128 x 6859 56 (205),
+  // 16 x 16 x 500 15 (86); N N 128 x 6859 x 128 71 (210), 128 x 373248 x 128 3.0 ms (10.0), 4 x 4 x 8 7 us
+  // (18); no shape of 1..512 x 1..373248 x 1..200000 was found where they were faster
+  const bool fits = fixed && fixed->n >= ((size_t)M + N + 1) / 2;
+  digit_gemm(8, ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, fits ? *fixed : splitk_buf(), fits, split_pct);
 }
 
 void mgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda, const double *B, int ldb,
@@ -586,7 +472,7 @@ void mgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A,
     dgemm(ta, tb, M, N, 0, alpha, A, lda, B, ldb, beta, C, ldc, s);
     return;
   }
-  gemm_tiled_mixed(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, splitk_buf32(), split_pct);
+  digit_gemm(4, ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, splitk_buf(), false, split_pct);
 }
 
 void sgemm(char ta, char tb, int M, int N, int K, float alpha, const float *A, int lda, const float *B, int ldb,

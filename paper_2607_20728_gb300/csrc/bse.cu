@@ -477,7 +477,10 @@ void combine_exec(Ctx &c, int nb, const CT<R> *Pa, const CT<R> *Pvh, CT<R> *Py, 
     else
       k::combine_tau<R>(c, nb, g.phir.get(), g.vloc.get(), g.tau.get(), Pa, Pvh, Py, true, k1e, k1d);
   } else {
-    k::combine_tau<R>(c, nb, g.phir.get(), g.vloc.get(), g.tau.get(), Pa, Pvh, Py, true, k1e, k1d);
+    if (k1d && c.k1x.ready)
+      k1d_fixed(c, c.k1x, nb, g.phir.get(), g.vloc.get(), Pa, Pvh, Py, true, k1e);
+    else
+      k::combine_tau<R>(c, nb, g.phir.get(), g.vloc.get(), g.tau.get(), Pa, Pvh, Py, true, k1e, k1d);
   }
   if (stop) BSE_CUDA(cudaEventRecord(stop, c.stream));
 }
@@ -552,6 +555,8 @@ void ensure_grids(Ctx &c) {
 }
 
 void ensure_work(Ctx &c) {
+  c.dev_err.alloc(1);
+  BSE_CUDA(cudaMemsetAsync(c.dev_err.get(), 0, sizeof(int), c.stream));
   if (c.prec == 0) {
     ensure_grids<double>(c);
   } else {
@@ -566,8 +571,6 @@ void ensure_work(Ctx &c) {
       g.colbuf_apply.alloc((size_t)((c.nocc + 1) / 2) * c.N[2] * c.sfft.ncols_pad);
     }
     ensure_grids<float>(c);
-    c.dev_err.alloc(1);
-    BSE_CUDA(cudaMemsetAsync(c.dev_err.get(), 0, sizeof(int), c.stream));
   }
   c.smat.alloc((size_t)std::max<long>(4L * c.nocc * c.nocc, 4096));
 }
@@ -725,7 +728,7 @@ constexpr int kGraphMaxVec = 8;
 std::vector<const void *> apply_fingerprint(const Ctx &c) {
   std::vector<const void *> f = {c.gA.get(), c.gLA.get(), c.pc32.get(), c.smat.get(), c.apply_s64.get(),
                                  c.apply_s32.get(), c.phi.get(), c.phi32.get(), c.negeps.get(), c.kin.get(),
-                                 c.k1d.tau, c.dev_err.get(), c.gp.get(), c.gm.get(), c.sfft.colpos.get(),
+                                 c.k1d.tau, c.k1x.tau, c.tau_scale.get(), c.dev_err.get(), c.gp.get(), c.gm.get(), c.sfft.colpos.get(),
                                  c.sfft.xs.get(), c.sfft.ent.get(), c.sfft.ent_off.get()};
   for (int a = 0; a < 3; ++a) {
     f.push_back(c.fft.ax[a].tw);
@@ -978,6 +981,7 @@ void apply_liouville(Ctx &c, int nvec, const double *A, double *LA, int op) {
   if (c.prec == 0) {
     if (graph) apply_graph<double>(c, nvec, A, LA);
     else apply_liouville_t<double>(c, nvec, A, LA, op, nullptr, nullptr);
+    if (op == 0 && c.k1x.ready) check_device_flag(c);
   } else {
     if (graph) apply_graph<float>(c, nvec, A, LA);
     else apply_liouville_t<float>(c, nvec, A, LA, op, nullptr, nullptr);
@@ -1508,12 +1512,19 @@ void pair_screen(Ctx &c, int np, CT<R> *P, R *X, R *Qm) {
   fft_exec(c, P, nq, +1);
 }
 
-// tiled: tau in the tile-major layout of the bulk-copy K1d kernel (FP32 only)
+// tiled: tau in the tile-major layout of the streamed K1d kernels (FP32, or fixed-point limbs for FP64)
 template <class R>
 void build_tau_t(Ctx &c, bool tiled = false) {
   const long npairs = c.npairs;
   Grids<R> &g = c.grids<R>();
-  g.tau.alloc((size_t)npairs * c.nr);
+  if (tiled && std::is_same<R, double>::value) {
+    g.tau.alloc(k1d_fixed_size(npairs, c.nr));
+    c.tau_scale.alloc(c.nr);
+    c.tau_top.alloc(c.nr);
+    BSE_CUDA(cudaMemsetAsync(c.tau_top.get(), 0, c.nr * sizeof(unsigned), c.stream));
+  } else {
+    g.tau.alloc((size_t)npairs * c.nr);
+  }
   c.stats.bytes_tau = (double)npairs * c.nr * sizeof(R);
   const R *phir = g.phir.get();
   R *X = g.sbuf.get();
@@ -1527,8 +1538,14 @@ void build_tau_t(Ctx &c, bool tiled = false) {
         k1d_unpack_tiled(c, np, c.pairs.get() + p0, g.work.get(), g.tau.get());
         continue;
       }
+    } else if (tiled) {
+      k1d_fixed_tile(c, np, c.pairs.get() + p0, g.work.get(), g.tau.get(), c.tau_top.get());
+      continue;
     }
     k::unpack_real<R, R>(c.nr, np, g.work.get(), g.tau.get() + p0 * c.nr, c.stream);
+  }
+  if constexpr (std::is_same<R, double>::value) {
+    if (tiled) k1d_fixed_finish(c, g.tau.get(), c.tau_top.get(), c.tau_scale.get());
   }
   sync(c);
 }
@@ -1731,6 +1748,7 @@ void wannier_setup(Ctx &c) {
 void build_tau(Ctx &c) {
   c.npairs = (long)c.nocc * (c.nocc + 1) / 2;
   c.k1d.ready = false;
+  c.k1x.ready = false;
   if (c.wan.on) {
     wannier_setup(c);
     c.stats.k1d_tma = 0;
@@ -1738,7 +1756,10 @@ void build_tau(Ctx &c) {
   }
   if (!(c.flags & BSE_FLAG_NO_K1D)) {
     if (c.prec == 0) {
-      build_tau_t<double>(c);
+      const bool tiled = k1d_fixed_supported(c.nocc);
+      build_tau_t<double>(c, tiled);
+      if (tiled)
+        c.k1x = {reinterpret_cast<const int2 *>(c.g64.tau.get()), c.tau_scale.get(), c.npairs, c.dev_err.get(), true};
     } else {
       const bool tiled = k1d_tma_supported(c.nocc, c.nr);
       build_tau_t<float>(c, tiled);

@@ -184,6 +184,15 @@ struct K1dTma {
   int *err = nullptr;                  // device flag set when a bounded wait gives up
   bool ready = false;
 };
+// FP64 K1d contraction in fixed point (k1d_fixed.cu): tau as integer limbs, tile-major, and the value of
+// one unit of it at every point
+struct K1dFixed {
+  const int2 *tau = nullptr;
+  const double *scale = nullptr;       // [nr]
+  long npairs = 0;
+  int *err = nullptr;                  // device flag set when a bounded wait gives up
+  bool ready = false;
+};
 // position (in pairs) of the pair (v', v), v' <= v, inside one 32-point tile of that layout
 __host__ __device__ inline long k1d_tile_slot(int vp, int v, int nocc) {
   (void)nocc;
@@ -339,6 +348,9 @@ struct Ctx {
   bool have_rho = false;
 
   K1dTma k1d;                  // FP32 K1d with TMA staging (mixed precision)
+  K1dFixed k1x;                // FP64 K1d in fixed point (FP64 contexts)
+  DevBuf<double> tau_scale;    // [nr] its units
+  DevBuf<unsigned> tau_top;    // [nr] largest |tau| of each point (high word), while tau is built
   SplitBF16 pdep_split;        // PDEP rows x v_c^{1/2} (projection operand, mixed precision)
   SplitBF16 pdepT_split;       // their transpose (back-projection operand)
   SplitBF16 gemm_a;            // per-call split of the left operand
@@ -371,6 +383,14 @@ struct Ctx {
   ~Ctx();
 };
 
+bool k1d_fixed_supported(int nocc);
+size_t k1d_fixed_size(long npairs, long nr);  // 8-byte elements of the tile-major tau
+// packed grids of np pair products -> tile-major doubles and the points' largest values (top, zeroed
+// before the first batch); after the last batch, doubles -> limbs in place and the units
+void k1d_fixed_tile(const Ctx &c, int np, const int2 *pairs, const double2 *P, double *tau, unsigned *top);
+void k1d_fixed_finish(const Ctx &c, double *tau, const unsigned *top, double *scale);
+void k1d_fixed(const Ctx &c, const K1dFixed &t, int nb, const double *phir, const double *vloc, const double2 *Pa,
+               const double2 *Pvh, double2 *Py, bool use_vloc, bool use_k1e);
 bool k1d_tma_supported(int nocc, long nr);
 // a bounded mbarrier wait on a barrier nothing completes: sets *err (device) when it gives up
 void wait_selftest(cudaStream_t s, int *err);

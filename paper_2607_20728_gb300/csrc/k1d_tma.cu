@@ -14,6 +14,7 @@
 #include <type_traits>
 
 #include "internal.cuh"
+#include "mbarrier.cuh"
 
 namespace bse {
 namespace {
@@ -24,70 +25,11 @@ constexpr int kStages = 2;
 constexpr int kThreads = 256;
 constexpr int kStageFloats = kB * kB * kR;                  // 8192 floats = 32 KB
 constexpr unsigned kStageBytes = kStageFloats * sizeof(float);
-constexpr long long kSpinLimit = 1LL << 26;                 // bounded mbarrier waits
-
-__device__ __forceinline__ unsigned smem_u32(const void *p) {
-  return static_cast<unsigned>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mbar_init(unsigned long long *bar, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long *bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-               : "memory");
-}
-
-// true when the phase with parity `parity` has completed
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long *bar, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n .reg .pred p;\n"
-      " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// 1D bulk copy global -> shared completing on an mbarrier (16-byte aligned, size a multiple of 16)
-__device__ __forceinline__ void bulk_load(float *dst, const float *src, unsigned bytes, unsigned long long *bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
-
-__device__ __forceinline__ void fence_async_shared() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
 
 constexpr int kTri = kB * (kB + 1) / 2;  // pairs of a diagonal block
 
 // pair (ii, jj) of a staged diagonal block, packed triangle with the smaller index first
 __device__ __forceinline__ int tri(int a, int b) { return a <= b ? b * (b + 1) / 2 + a : a * (a + 1) / 2 + b; }
-
-__device__ __forceinline__ void mbar_arrive(unsigned long long *bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
-
-// bounded wait: false when one second (or the iteration cap) ran out
-__device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned parity) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const unsigned long long t0 = global_ns();
-  for (long long spin = 0; spin < kSpinLimit; ++spin) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((spin & 63) == 0 && global_ns() - t0 > 1000000000ull) return false;
-  }
-  return false;
-}
 
 __device__ __forceinline__ void consumer_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 

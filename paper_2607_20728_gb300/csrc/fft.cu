@@ -162,6 +162,27 @@ void twiddles(int n, double2 *out) {
     out[k] = make_double2(std::cos(ang), std::sin(ang));
   }
 }
+
+// exp(-2 pi i k/n) as 62-bit fixed point: cos (hi, lo), sin (hi, lo), lo signed.  The angle is reduced to
+// the first octant in integers, so that the extended-precision sine and cosine are exact to 2^-63.
+int4 fixed_twiddle(int k, int n) {
+  const long a = 8L * (k % n), oct = a / n, rem = a - oct * n;
+  const long t = oct & 1 ? n - rem : rem;
+  const long double th = 3.14159265358979323846264338327950288L * (long double)t / (4.0L * n);
+  const long double c0 = std::cos(th), s0 = std::sin(th);
+  const long double cs[8] = {c0, s0, -s0, -c0, -c0, -s0, s0, c0};
+  const long double sn[8] = {s0, c0, c0, s0, -s0, -c0, -c0, -s0};
+  auto limbs = [](long double v, int &h, int &l) {
+    long long w = std::llround(std::ldexp(v, 62));
+    if ((int)(unsigned)(w & 0xffffffffll) == INT32_MIN) w += 1;  // so that -lo is representable
+    l = (int)(unsigned)(w & 0xffffffffll);
+    h = (int)((w - l) >> 32);
+  };
+  int4 r;
+  limbs(cs[oct], r.x, r.y);
+  limbs(-sn[oct], r.z, r.w);
+  return r;
+}
 }  // namespace
 
 void FFTPlan::init(int n1, int n2, int n3) {
@@ -188,6 +209,13 @@ void FFTPlan::init(int n1, int n2, int n3) {
     owned.push_back(p32);
     BSE_CUDA(cudaMemcpy(p32, tw32.data(), sizeof(float2) * n[a], cudaMemcpyHostToDevice));
     x.tw32 = (float2 *)p32;
+    std::vector<int4> twx(n[a]);
+    for (int k = 0; k < n[a]; ++k) twx[k] = fixed_twiddle(k, n[a]);
+    void *px = nullptr;
+    BSE_CUDA(cudaMalloc(&px, sizeof(int4) * n[a]));
+    owned.push_back(px);
+    BSE_CUDA(cudaMemcpy(px, twx.data(), sizeof(int4) * n[a], cudaMemcpyHostToDevice));
+    x.twx = (int4 *)px;
   }
   set_smem_attrs();
 }

@@ -89,6 +89,7 @@ struct FFTAxis {
   int radix[12] = {0};
   double2 *tw = nullptr;   // device table exp(-2 pi i k/n), k < n, FP64
   float2 *tw32 = nullptr;  // the same rounded to FP32
+  int4 *twx = nullptr;     // the same as 62-bit fixed point (fixed_fft.cuh)
 };
 
 struct FFTPlan {

@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "fft_codelets.cuh"
+#include "fixed_fft.cuh"
 #include "internal.cuh"
 
 namespace bse {
@@ -277,6 +278,219 @@ __global__ void __launch_bounds__(kXYThreads) sph_xy(SphArgs<C> a, C *__restrict
   }
 }
 
+// ---- FP64 xy passes on 64-bit fixed point ---------------------------------------------------------
+// The modes of sph_xy for FP64 data: columns and grids stay FP64 in memory, the lines are transformed as
+// integers (fixed_fft.cuh).  As FP64 these passes were bound by the FP64 pipe (about 1840 operations per
+// 72-point line at two per clock).  Scales, one power of two per plane and pass:
+//   MODE 0, 2 (inverse): the sum of |re| + |im| over the plane's columns bounds both passes;
+//   MODE 1 (forward): the largest such sum of an x line, then, from the result, of a y line (values are
+//   shifted as the first stage of the y pass loads them);
+//   MODE 2: the product with V(r) (fixed point below the plane's largest |V|), then as MODE 1.
+// Each is an upper bound taken from the leading 21 bits.  Rounding is at 2^-61 of those sums: against exact
+// transforms (36^3, flat and decaying data) the relative error of a transform is 3.0-4.3e-16, with the FP64
+// passes 3.8-5.5e-16 (the z passes stay FP64).
+// 64 packed grids of the 63-well cell (72^3, 4608 planes), FP64 pass -> this one: inverse 1490 -> 512 us,
+// forward 1595 -> 691, H product of 63 orbitals 994 -> 330.  Bound by instruction issue (57 thousand warp
+// instructions a plane, 42% of the issue slots used: one CTA of 16 warps and a barrier per stage).
+struct FxArgs {
+  int N1, N2, N3, ncols_pad, nxs;
+  long nr;
+  const int *colpos, *xs;
+  fx::Axis ax[2];
+};
+
+// L lines in shared memory, consecutive threads on consecutive lines; `first` loads the inputs of the first
+// stage (buffer, offset), later stages read the buffers; returns the buffer of the result
+template <int SG, class Base, class First>
+__device__ fx::C2 *lines_fx(fx::C2 *in, fx::C2 *out, int L, Base base, int es, const fx::Axis &ax, First first) {
+  int Ns = 1;
+  for (int s = 0; s < ax.nstage; ++s) {
+    const int R = ax.radix[s];
+    const int work = L * (ax.n / R);
+    int j = threadIdx.x / L, t = threadIdx.x - j * L;
+    const int dj = blockDim.x / L, dt = blockDim.x - dj * L;
+    for (int e = threadIdx.x; e < work; e += blockDim.x) {
+      const int b0 = base(t);
+      if (s == 0) {
+        fx::bfly_any<SG>(R, [&](int o) { return first(in[b0 + o]); }, out + b0, j, ax.n, Ns, ax.tw, es);
+      } else {
+        fx::bfly_any<SG>(R, [&](int o) { return in[b0 + o]; }, out + b0, j, ax.n, Ns, ax.tw, es);
+      }
+      t += dt;
+      j += dj;
+      if (t >= L) {
+        t -= L;
+        ++j;
+      }
+    }
+    __syncthreads();
+    fx::C2 *tmp = in;
+    in = out;
+    out = tmp;
+    Ns *= R;
+  }
+  return in;
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(kXYThreads) sph_xy_fx(FxArgs a, double2 *__restrict__ colbuf,
+                                                        double2 *__restrict__ P, const double *__restrict__ vloc) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  __shared__ unsigned top, vtop, ltop[2];
+  __shared__ unsigned long long total;
+  const int N1 = a.N1, N1p = a.N1 + 1;
+  const int np = N1 * a.N2, npp = N1p * a.N2;
+  fx::C2 *A = reinterpret_cast<fx::C2 *>(sm_raw), *B = A + npp;
+  const int z = blockIdx.x, q = blockIdx.y;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  double2 *crow = colbuf + ((long)q * a.N3 + z) * a.ncols_pad;
+  double2 *plane = P ? P + (long)q * a.nr + (long)z * np : nullptr;
+  const double *v = MODE == 2 ? vloc + (long)z * np : nullptr;
+  if (threadIdx.x == 0) {
+    top = vtop = ltop[0] = ltop[1] = 0;
+    total = 0;
+  }
+  const int y0 = threadIdx.x / N1, x0 = threadIdx.x - y0 * N1;
+  const int dy = blockDim.x / N1, dx = blockDim.x - dy * N1;
+  // e = y N1 + x over the plane, e + y its padded place
+  auto for_plane = [&](auto body) {
+    int y = y0, x = x0;
+    for (int e = threadIdx.x; e < np; e += blockDim.x) {
+      body(e, e + y);
+      x += dx;
+      y += dy;
+      if (x >= N1) {
+        x -= N1;
+        ++y;
+      }
+    }
+  };
+  auto warp_max = [&](unsigned m, unsigned *dst) {
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) atomicMax(dst, m);
+  };
+  // exponent of a bound of n units of 2^u
+  auto above = [](unsigned long long n, int u) { return u + 64 - __clzll((long long)n); };
+  const auto same = [](fx::C2 c) { return c; };
+  fx::Unit unit{0, false};
+  fx::C2 *F;
+  if (MODE == 0 || MODE == 2) {
+    // the y pass transforms the occupied lines only: the buffer of its result holds zeros on the others
+    const bool zero_b = (a.ax[1].nstage & 1) != 0;
+    for (int e = threadIdx.x; e < npp; e += blockDim.x) {
+      A[e] = fx::C2{0, 0};
+      if (zero_b) B[e] = fx::C2{0, 0};
+    }
+    __syncthreads();
+    unsigned m = 0, mv = 0;
+    for (int c = threadIdx.x; c < a.ncols_pad; c += blockDim.x)
+      if (__ldg(&a.colpos[c]) >= 0) m = max(m, max(fx::high_abs(crow[c].x), fx::high_abs(crow[c].y)));
+    warp_max(m, &top);
+    if (MODE == 2) {
+      for (int e = threadIdx.x; e < np; e += blockDim.x) mv = max(mv, fx::high_abs(__ldg(&v[e])));
+      warp_max(mv, &vtop);
+    }
+    __syncthreads();
+    const int E = (int)(top >> 20);
+    unsigned long long sum = 0;
+    for (int c = threadIdx.x; c < a.ncols_pad; c += blockDim.x)
+      if (__ldg(&a.colpos[c]) >= 0) sum += fx::mag(crow[c].x, E) + fx::mag(crow[c].y, E);
+    for (int w = 16; w > 0; w >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, w);
+    if (lane == 0) atomicAdd(&total, sum);
+    __syncthreads();
+    const int e0 = above(total, E - 1043);
+    unit.q = e0 - 61;
+    unit.bad = E >= 0x7ff || (MODE == 2 && (vtop >> 20) >= 0x7ff);
+    for (int c = threadIdx.x; c < a.ncols_pad; c += blockDim.x) {
+      const int pos = __ldg(&a.colpos[c]);
+      if (pos >= 0) {
+        const double2 u = crow[c];
+        A[pos + pos / N1] = fx::C2{fx::from_double(u.x, e0, 61), fx::from_double(u.y, e0, 61)};
+      }
+    }
+    __syncthreads();
+    F = lines_fx<1>(A, B, a.nxs, ListBase{a.xs}, N1p, a.ax[1], same);
+    F = lines_fx<1>(F, F == A ? B : A, a.N2, StrideBase{N1p}, 1, a.ax[0], same);
+    if (MODE == 0) {
+      for_plane([&](int e, int ep) { plane[e] = make_double2(unit(F[ep].x), unit(F[ep].y)); });
+      return;
+    }
+    const int ev = max((int)(vtop >> 20), 1) - 1022;  // |V| < 2^ev
+    for_plane([&](int e, int ep) {
+      const fx::W w = fx::split(fx::from_double(__ldg(&v[e]), ev, 62));
+      F[ep] = fx::cscale(F[ep], w);
+    });
+    unit.q += ev;
+    __syncthreads();
+  } else {
+    unsigned m = 0;
+    for_plane([&](int e, int ep) {
+      const double2 u = plane[e];
+      m = max(m, max(fx::high_abs(u.x), fx::high_abs(u.y)));
+      reinterpret_cast<double2 *>(A)[ep] = u;
+    });
+    __syncthreads();
+    warp_max(m, &top);
+    __syncthreads();
+    F = A;
+  }
+  // forward: the largest sum of |re| + |im| over an x line, one warp per line
+  const int E = (int)(top >> 20);
+  for (int y = warp; y < a.N2; y += nwarp) {
+    unsigned s = 0;
+    for (int x = lane; x < N1; x += 32) {
+      if (MODE == 1) {
+        const double2 u = reinterpret_cast<const double2 *>(F)[y * N1p + x];
+        s += fx::mag(u.x, E) + fx::mag(u.y, E);
+      } else {
+        const fx::C2 u = F[y * N1p + x];
+        s += (unsigned)((unsigned long long)llabs(u.x) >> 40) + (unsigned)((unsigned long long)llabs(u.y) >> 40) + 2;
+      }
+    }
+    s = __reduce_add_sync(0xffffffffu, s);
+    if (lane == 0) atomicMax(&ltop[0], s);
+  }
+  __syncthreads();
+  // values shifted as they are loaded: k > 0 right (rounded), k < 0 left
+  auto shifted = [](fx::C2 c, int k) {
+    if (k <= 0) return fx::C2{c.x << -k, c.y << -k};
+    const long long h = 1ll << (k - 1);
+    return fx::C2{(c.x + h) >> k, (c.y + h) >> k};
+  };
+  fx::C2 *O = F == A ? B : A;
+  if (MODE == 1) {
+    const int e0 = above(ltop[0], E - 1043);
+    unit.q = e0 - 61;
+    unit.bad = E >= 0x7ff;
+    F = lines_fx<-1>(F, O, a.N2, StrideBase{N1p}, 1, a.ax[0], [&](const fx::C2 &c) {
+      return fx::C2{fx::from_double(__longlong_as_double(c.x), e0, 61), fx::from_double(__longlong_as_double(c.y), e0, 61)};
+    });
+  } else {
+    const int k = max(above(ltop[0], 40) - 61, -30);
+    unit.q += k;
+    F = lines_fx<-1>(F, O, a.N2, StrideBase{N1p}, 1, a.ax[0], [&](const fx::C2 &c) { return shifted(c, k); });
+  }
+  for (int t = warp; t < a.nxs; t += nwarp) {
+    const int x = __ldg(&a.xs[t]);
+    unsigned s = 0;
+    for (int y = lane; y < a.N2; y += 32) {
+      const fx::C2 u = F[y * N1p + x];
+      s += (unsigned)((unsigned long long)llabs(u.x) >> 40) + (unsigned)((unsigned long long)llabs(u.y) >> 40) + 2;
+    }
+    s = __reduce_add_sync(0xffffffffu, s);
+    if (lane == 0) atomicMax(&ltop[1], s);
+  }
+  __syncthreads();
+  const int k = max(above(ltop[1], 40) - 61, -30);
+  unit.q += k;
+  F = lines_fx<-1>(F, F == A ? B : A, a.nxs, ListBase{a.xs}, N1p, a.ax[1], [&](const fx::C2 &c) { return shifted(c, k); });
+  for (int c = threadIdx.x; c < a.ncols_pad; c += blockDim.x) {
+    const int pos = __ldg(&a.colpos[c]);
+    const fx::C2 u = pos >= 0 ? F[pos + pos / N1] : fx::C2{0, 0};
+    crow[c] = pos >= 0 ? make_double2(unit(u.x), unit(u.y)) : make_double2(0.0, 0.0);
+  }
+}
+
 // ---- pair pipelines on the density sphere (tau build, U vector; Eq. 2c and Eq. 3) ----------
 // forward z pass: z lines of the occupied density columns, then the wave-function-sphere
 // coefficients of the two packed pair densities into X (real basis, type R, times `scale`) for
@@ -401,6 +615,10 @@ SphArgs<C> make_args(const Ctx &c, const SphereFFT &s) {
   return a;
 }
 
+// one plane pass (MODE of sph_xy) over nq packed grids: FP64 in fixed point, FP32 as it is
+template <class C, int MODE>
+void launch_xy(Ctx &c, const SphereFFT &s, int nq, C *cb, C *P, const typename RealOf<C>::T *v);
+
 template <class C>
 size_t z_smem(const Ctx &c, const SphereFFT &s) { return (size_t)2 * s.cg * (c.N[2] + 1) * sizeof(C); }
 template <class C>
@@ -420,9 +638,15 @@ void set_attrs() {
   const int cap = (int)kSmemCap;
   BSE_CUDA(cudaFuncSetAttribute(sph_z_inv<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
   BSE_CUDA(cudaFuncSetAttribute(sph_z_fwd<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-  BSE_CUDA(cudaFuncSetAttribute(sph_xy<C, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-  BSE_CUDA(cudaFuncSetAttribute(sph_xy<C, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-  BSE_CUDA(cudaFuncSetAttribute(sph_xy<C, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+  if constexpr (sizeof(C) == sizeof(double2)) {
+    BSE_CUDA(cudaFuncSetAttribute(sph_xy_fx<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    BSE_CUDA(cudaFuncSetAttribute(sph_xy_fx<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    BSE_CUDA(cudaFuncSetAttribute(sph_xy_fx<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+  } else {
+    BSE_CUDA(cudaFuncSetAttribute(sph_xy<C, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    BSE_CUDA(cudaFuncSetAttribute(sph_xy<C, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    BSE_CUDA(cudaFuncSetAttribute(sph_xy<C, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+  }
   using R = typename RealOf<C>::T;
   BSE_CUDA(cudaFuncSetAttribute(dsph_z_fwd<C, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
   BSE_CUDA(cudaFuncSetAttribute(dsph_z_inv<C, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
@@ -431,6 +655,33 @@ void set_attrs() {
 
 // threads per plane-pass CTA: the autotuner's choice, else kXYThreads
 int xy_threads(const Ctx &c) { return c.xy_threads > 0 ? std::min(c.xy_threads, kXYThreads) : kXYThreads; }
+
+template <class C, int MODE>
+void launch_xy(Ctx &c, const SphereFFT &s, int nq, C *cb, C *P, const typename RealOf<C>::T *v) {
+  const dim3 grid(c.N[2], nq);
+  if constexpr (sizeof(C) == sizeof(double2)) {
+    FxArgs a;
+    a.N1 = c.N[0];
+    a.N2 = c.N[1];
+    a.N3 = c.N[2];
+    a.ncols_pad = s.ncols_pad;
+    a.nxs = s.nxs;
+    a.nr = c.nr;
+    a.colpos = s.colpos.get();
+    a.xs = s.xs.get();
+    for (int i = 0; i < 2; ++i) {
+      const FFTAxis &x = c.fft.ax[i];
+      a.ax[i].n = x.n;
+      a.ax[i].nstage = x.nstage;
+      for (int r = 0; r < 12; ++r) a.ax[i].radix[r] = x.radix[r];
+      a.ax[i].tw = x.twx;
+    }
+    sph_xy_fx<MODE><<<grid, xy_threads(c), xy_smem<C>(c), c.stream>>>(a, cb, P, v);
+  } else {
+    sph_xy<C, MODE><<<grid, xy_threads(c), xy_smem<C>(c), c.stream>>>(make_args<C>(c, s), cb, P, v);
+  }
+  BSE_CHECK_LAUNCH();
+}
 
 template <class R>
 CT<R> *colbuf_for(Ctx &c, int nq) {
@@ -551,8 +802,7 @@ void dens_forward(Ctx &c, int np, CT<R> *P, R *X, double scale, const R *vcg, R 
   Grids<R> &g = c.grids<R>();
   g.colbuf_dens.alloc((size_t)nq * c.N[2] * c.dfft.ncols_pad);
   C *cb = g.colbuf_dens.get();
-  sph_xy<C, 1><<<dim3(c.N[2], nq), xy_threads(c), xy_smem<C>(c), c.stream>>>(a, cb, P, nullptr);
-  BSE_CHECK_LAUNCH();
+  launch_xy<C, 1>(c, c.dfft, nq, cb, P, nullptr);
   dsph_z_fwd<C, R><<<dim3(c.dfft.ngroups, nq), kThreads, z_smem<C>(c, c.dfft), c.stream>>>(a, np, c.npw, cb, X,
                                                                                          scale, vcg, cscale);
   BSE_CHECK_LAUNCH();
@@ -569,8 +819,7 @@ void dens_inverse(Ctx &c, int np, const R *X, double scale, CT<R> *P) {
   dsph_z_inv<C, R><<<dim3(c.dfft.ngroups, nq), kThreads, z_smem<C>(c, c.dfft), c.stream>>>(a, np, c.npw, X, scale,
                                                                                          cb);
   BSE_CHECK_LAUNCH();
-  sph_xy<C, 0><<<dim3(c.N[2], nq), xy_threads(c), xy_smem<C>(c), c.stream>>>(a, cb, P, nullptr);
-  BSE_CHECK_LAUNCH();
+  launch_xy<C, 0>(c, c.dfft, nq, cb, P, nullptr);
 }
 
 template bool dens_fft_ok<double>(const Ctx &);
@@ -595,8 +844,7 @@ void sphere_to_grid(Ctx &c, int nf, const double *X, CT<R> *P, double scale, CT<
   C *cb = colbuf ? colbuf : colbuf_for<R>(c, nq);
   sph_z_inv<C><<<dim3(c.sfft.ngroups, nq), kThreads, z_smem<C>(c), c.stream>>>(a, nf, c.npw, X, scale, cb);
   BSE_CHECK_LAUNCH();
-  sph_xy<C, 0><<<dim3(c.N[2], nq), xy_threads(c), xy_smem<C>(c), c.stream>>>(a, cb, P, nullptr);
-  BSE_CHECK_LAUNCH();
+  launch_xy<C, 0>(c, c.sfft, nq, cb, P, nullptr);
 }
 
 template <class R>
@@ -608,8 +856,7 @@ void grid_to_sphere(Ctx &c, int nf, CT<R> *P, double *Y, double scale, const dou
   set_attrs<C>();
   SphArgs<C> a = make_args<C>(c, c.sfft);
   C *cb = colbuf ? colbuf : colbuf_for<R>(c, nq);
-  sph_xy<C, 1><<<dim3(c.N[2], nq), xy_threads(c), xy_smem<C>(c), c.stream>>>(a, cb, P, nullptr);
-  BSE_CHECK_LAUNCH();
+  launch_xy<C, 1>(c, c.sfft, nq, cb, P, nullptr);
   sph_z_fwd<C><<<dim3(c.sfft.ngroups, nq), kThreads, z_smem<C>(c), c.stream>>>(
       a, nf, c.npw, cb, Y, scale, Xd, c.kin.get(), shift, period > 0 ? period : 1, shift_const);
   BSE_CHECK_LAUNCH();
@@ -626,9 +873,7 @@ void sphere_h(Ctx &c, int nf, const double *X, double *HX, const double *shift) 
   const double s_in = 1.0 / std::sqrt(c.omega), s_out = std::sqrt(c.omega) / (double)c.nr;
   sph_z_inv<C><<<dim3(c.sfft.ngroups, nq), kThreads, z_smem<C>(c), c.stream>>>(a, nf, c.npw, X, s_in, cb);
   BSE_CHECK_LAUNCH();
-  sph_xy<C, 2><<<dim3(c.N[2], nq), xy_threads(c), xy_smem<C>(c), c.stream>>>(a, cb, nullptr,
-                                                                            c.grids<R>().vloc.get());
-  BSE_CHECK_LAUNCH();
+  launch_xy<C, 2>(c, c.sfft, nq, cb, nullptr, c.grids<R>().vloc.get());
   sph_z_fwd<C><<<dim3(c.sfft.ngroups, nq), kThreads, z_smem<C>(c), c.stream>>>(
       a, nf, c.npw, cb, HX, s_out, X, c.kin.get(), shift, shift ? c.nocc : 1, 0.0);
   BSE_CHECK_LAUNCH();

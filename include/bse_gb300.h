@@ -132,7 +132,8 @@ typedef struct {
   double homo_lumo_gap;       /* Ha */
   double ms_setup, ms_ground_state, ms_tau, ms_davidson, ms_uvec, ms_zvector, ms_forces;
   double bytes_tau;           /* bytes of the cached tau_{v'v}(r) */
-  int k1d_tma;                /* 1 when the TMA-fed FP32 kernel serves the K1d term (mixed precision) */
+  int k1d_tma;                /* 1 when the TMA-fed FP32 kernel serves the K1d term over whole blocks of 16
+                                 orbitals and tiles of 32 grid points (mixed precision) */
   double ms_host_eig;         /* host time in the Rayleigh-Ritz / orthonormalisation eigensolves */
   int gs_chunks;              /* Davidson chunks of the ground state */
   int tuned;                  /* 1 once the autotuner has chosen this context's launch shapes */

@@ -1517,13 +1517,11 @@ template <class R>
 void build_tau_t(Ctx &c, bool tiled = false) {
   const long npairs = c.npairs;
   Grids<R> &g = c.grids<R>();
+  g.tau.alloc(tiled ? k1d_tiled_size(npairs, c.nr) : (size_t)npairs * c.nr);
   if (tiled && std::is_same<R, double>::value) {
-    g.tau.alloc(k1d_fixed_size(npairs, c.nr));
     c.tau_scale.alloc(c.nr);
     c.tau_top.alloc(c.nr);
     BSE_CUDA(cudaMemsetAsync(c.tau_top.get(), 0, c.nr * sizeof(unsigned), c.stream));
-  } else {
-    g.tau.alloc((size_t)npairs * c.nr);
   }
   c.stats.bytes_tau = (double)npairs * c.nr * sizeof(R);
   const R *phir = g.phir.get();
@@ -1769,7 +1767,7 @@ void build_tau(Ctx &c) {
   } else {
     c.stats.bytes_tau = 0;
   }
-  c.stats.k1d_tma = c.k1d.ready ? 1 : 0;
+  c.stats.k1d_tma = c.k1d.ready && k1d_tma_whole(c.nocc, c.nr) ? 1 : 0;
 }
 
 // phi_v(r) on the FP64 grids (g64.phir) for the first nocc rows of Q
@@ -3652,7 +3650,7 @@ bse_status bse_selftest_k1d_stall(bse_ctx *ctx) {
   BSE_API_BEGIN
   BSE_REQUIRE(ctx, "ctx is required");
   bse::Ctx &c = ctx->c;
-  if (!c.have_gs || !c.k1d.ready)
+  if (!c.have_gs || !c.k1d.ready || !bse::k1d_tma_whole(c.nocc, c.nr))
     throw bse::Error(BSE_ERR_STATE, "no tiled FP32 K1d pipeline (mixed precision, n_occ a multiple of 16)");
   bse::Grids<float> &g = c.g32;
   const int nb = bse::k1d_tma_max_nb(c.nocc);

@@ -196,11 +196,11 @@ struct K1dFixed {
 };
 // position (in pairs) of the pair (v', v), v' <= v, inside one 32-point tile of that layout
 __host__ __device__ inline long k1d_tile_slot(int vp, int v, int nocc) {
-  (void)nocc;
   const int I = vp / 16, J = v / 16, ii = vp % 16, jj = v % 16;
-  const long col = 128L * J * (J - 1) + 136L * J;  // pairs of the columns before J
-  if (I == J) return col + 256L * J + jj * (jj + 1) / 2 + ii;
-  return col + 256L * I + jj * 16 + ii;
+  const int bj = nocc - 16 * J < 16 ? nocc - 16 * J : 16;  // columns of this (possibly last, narrow) column
+  const long col = 128L * J * (J - 1) + 136L * J;          // pairs of the columns before J
+  if (I == J) return col + 16L * J * bj + jj * (jj + 1) / 2 + ii;
+  return col + 16L * I * bj + jj * 16 + ii;
 }
 
 // an FP32 operand split into bf16 hi + lo, rows padded with zeros to kp (a multiple of 64) columns
@@ -385,7 +385,7 @@ struct Ctx {
 };
 
 bool k1d_fixed_supported(int nocc);
-size_t k1d_fixed_size(long npairs, long nr);  // 8-byte elements of the tile-major tau
+size_t k1d_tiled_size(long npairs, long nr);  // elements of a tile-major tau
 // packed grids of np pair products -> tile-major doubles and the points' largest values (top, zeroed
 // before the first batch); after the last batch, doubles -> limbs in place and the units
 void k1d_fixed_tile(const Ctx &c, int np, const int2 *pairs, const double2 *P, double *tau, unsigned *top);
@@ -393,6 +393,7 @@ void k1d_fixed_finish(const Ctx &c, double *tau, const unsigned *top, double *sc
 void k1d_fixed(const Ctx &c, const K1dFixed &t, int nb, const double *phir, const double *vloc, const double2 *Pa,
                const double2 *Pvh, double2 *Py, bool use_vloc, bool use_k1e);
 bool k1d_tma_supported(int nocc, long nr);
+bool k1d_tma_whole(int nocc, long nr);  // no ragged last orbital block or tile
 // a bounded mbarrier wait on a barrier nothing completes: sets *err (device) when it gives up
 void wait_selftest(cudaStream_t s, int *err);
 int k1d_tma_max_nb(int nocc);

@@ -438,7 +438,7 @@ int tau_bits(int nocc) { return nocc <= 128 ? 56 : nocc <= 256 ? 55 : 54; }
 // which the read of the error flag after the call (about 8 us) outweighs.
 bool k1d_fixed_supported(int nocc) { return nocc >= 16 && nocc <= 512 && shape_for(1, nocc).stages > 0; }
 
-size_t k1d_fixed_size(long npairs, long nr) { return (size_t)npairs * ((nr + kR - 1) / kR * kR); }
+size_t k1d_tiled_size(long npairs, long nr) { return (size_t)npairs * ((nr + kR - 1) / kR * kR); }
 
 void k1d_fixed_tile(const Ctx &c, int np, const int2 *pairs, const double2 *P, double *tau, unsigned *top) {
   const long rpad = (c.nr + kR - 1) / kR * kR;

@@ -58,8 +58,22 @@ __device__ __forceinline__ void consumer_sync() { asm volatile("bar.sync 1, 256;
 // its copies), but every consumer warp still passes the same named barriers up to the next tile's
 // first one, where all of them leave.  hold != 0 (failure-detection self-test only): the producer
 // issues no copies, so every consumer wait runs out.
-template <int NB, int S>
-__global__ void __launch_bounds__(kThreads + 32, 1) k1d_tma_kernel(
+//
+// RAG: the last orbital block is narrower than 16, or the last tile holds fewer than 32 points.  A narrow
+// block (I, J) is stored as its bj < 16 columns only; rows of a past the last orbital are zero in shared
+// memory, sums over the columns of a narrow block stop at bj, and the padding rows of Y are not stored.
+// With an odd number of orbitals the packed partners of a row change from vector to vector, so rows are
+// then loaded and stored one by one.  Against the kernel that reads every pair twice (combine_tau, which
+// such shapes took before), one / two / four vectors: N_occ = 74, 60^3: 459 / 636 / 1185 us (1208 / 1385 /
+// 6000; tau at the copy rate 354); N_occ = 63, 72^3: 572 / 724 / 1312 (1427 / 1700 / 7494; 444);
+// N_occ = 17, 36^3: 19 / 26 / 49 (31 / 30 / 66).
+//
+// CTAS: with one or two vectors and a and Y rows that leave room for two rings in an SM, two CTAs share it,
+// and the prologue and epilogue of one overlap the stream of the other: one vector, N_occ = 74 632 -> 459 us,
+// N_occ = 63 811 -> 572, N_occ = 48, 36^3 55 -> 45, N_occ = 128, 72^3 1.90 -> 1.80 ms.  Four vectors need
+// more than the 112 registers that leaves.
+template <int NB, int S, bool RAG, int CTAS>
+__global__ void __launch_bounds__(kThreads + 32, CTAS) k1d_tma_kernel(
     const float *__restrict__ tau, long npairs, long nr, int nocc, int nb_total, int b0,
     const float *__restrict__ phir, const float *__restrict__ vloc, const float2 *__restrict__ Pa,
     const float2 *__restrict__ Pvh, float2 *__restrict__ Py, int use_vloc, int use_k1e, int *__restrict__ err,
@@ -67,15 +81,16 @@ __global__ void __launch_bounds__(kThreads + 32, 1) k1d_tma_kernel(
   extern __shared__ __align__(128) unsigned char smem[];
   float *tau_s = reinterpret_cast<float *>(smem);                       // [S][16][16][32]
   float *a_s = tau_s + S * kStageFloats;                                // [NB][nocc][32]
-  float *y_s = a_s + (size_t)NB * nocc * kR;                            // [NB][nocc][32]
-  unsigned long long *full = reinterpret_cast<unsigned long long *>(y_s + (size_t)NB * nocc * kR);
+  const int nblk = RAG ? (nocc + kB - 1) / kB : nocc / kB;
+  const int nrow = RAG ? nblk * kB : nocc;                              // rows of a and Y in shared memory
+  float *y_s = a_s + (size_t)NB * nrow * kR;                            // [NB][nocc][32]
+  unsigned long long *full = reinterpret_cast<unsigned long long *>(y_s + (size_t)NB * nrow * kR);
   unsigned long long *empty = full + S;
   volatile int *fail = reinterpret_cast<volatile int *>(empty + S);  // CTA-wide: a consumer gave up
 
   const int tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5;
-  const int nblk = nocc / kB;
-  const long ntiles = nr / kR;
+  const long ntiles = RAG ? (nr + kR - 1) / kR : nr / kR;
 
   if (tid == 0) {
     for (int st = 0; st < S; ++st) {
@@ -102,7 +117,8 @@ __global__ void __launch_bounds__(kThreads + 32, 1) k1d_tma_kernel(
               ok = false;
               break;
             }
-            const unsigned bytes = (unsigned)((I == J ? kTri : kB * kB) * kR * sizeof(float));
+            const int bj = RAG ? min(kB, nocc - J * kB) : kB;
+            const unsigned bytes = (unsigned)((I == J ? bj * (bj + 1) / 2 : kB * bj) * kR * sizeof(float));
             fence_async_shared();
             mbar_expect_tx(&full[st], bytes);
             bulk_load(tau_s + st * kStageFloats, src, bytes, &full[st]);
@@ -125,7 +141,7 @@ __global__ void __launch_bounds__(kThreads + 32, 1) k1d_tma_kernel(
   constexpr int NBH = PAIR ? NB / 2 : NB;
   constexpr int LS = PAIR ? 2 : 1;
   auto idx = [&](int b, int v) -> size_t {
-    return PAIR ? ((size_t)v * NBH + (b >> 1)) * (kR * 2) + (b & 1) : ((size_t)b * nocc + v) * kR;
+    return PAIR ? ((size_t)v * NBH + (b >> 1)) * (kR * 2) + (b & 1) : ((size_t)b * nrow + v) * kR;
   };
   const bool roleA = warp < 4;
   const int r4 = (warp & 3) * 4;  // first of the 4 block rows this warp accumulates
@@ -141,9 +157,10 @@ __global__ void __launch_bounds__(kThreads + 32, 1) k1d_tma_kernel(
       for (int b = 0; b < NBH; ++b) acc[k][b] = Acc{};
   };
   // acc[k] += sum_m tau(slot(k, m)) a(16 C + m) over the 16 columns m of a staged block
-  auto mac4 = [&](const float *T, int C, auto slot) {
+  auto mac4 = [&](const float *T, int C, int mend, auto slot) {
 #pragma unroll
     for (int m = 0; m < kB; ++m) {
+      if (RAG && m >= mend) break;
       float t[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) t[k] = T[slot(k, m) * kR + lane];
@@ -180,7 +197,8 @@ __global__ void __launch_bounds__(kThreads + 32, 1) k1d_tma_kernel(
   long g = 0;
   bool ok = true;  // false once the CTA has given up (uniform within the warp)
   for (long t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const long rr = t * kR + lane;
+    const bool live = !RAG || t * kR + lane < nr;
+    const long rr = live ? t * kR + lane : nr - 1;
     consumer_sync();  // the previous tile's epilogue has read Y
     // a give-up recorded before this barrier is seen by every consumer warp: all leave together
     if (*fail) break;
@@ -205,10 +223,22 @@ __global__ void __launch_bounds__(kThreads + 32, 1) k1d_tma_kernel(
 #pragma unroll
       for (int b = 0; b < NB; ++b) {
         const int bb = b0 + b;
-        d.pa[b] = bb < nb_total ? Pa[(((long)bb * nocc + v) >> 1) * nr + rr] : make_float2(0.f, 0.f);
+        const long f = (long)bb * nocc + v;
+        float2 x = make_float2(0.f, 0.f);
+        if (bb < nb_total && (!RAG || v < nocc)) {
+          if (!RAG || (f & 1) == 0) {
+            x = Pa[(f >> 1) * nr + rr];
+            if (RAG && v + 1 >= nocc) x.y = 0.f;
+          } else {
+            const float *Pf = reinterpret_cast<const float *>(Pa);
+            x.x = Pf[2 * ((f >> 1) * nr + rr) + 1];
+            if (v + 1 < nocc) x.y = Pf[2 * (((f + 1) >> 1) * nr + rr)];
+          }
+        }
+        d.pa[b] = x;
       }
-      d.ph0 = use_k1e ? phir[(long)v * nr + rr] : 0.f;
-      d.ph1 = use_k1e ? phir[(long)(v + 1) * nr + rr] : 0.f;
+      d.ph0 = use_k1e && (!RAG || v < nocc) ? phir[(long)v * nr + rr] : 0.f;
+      d.ph1 = use_k1e && (!RAG || v + 1 < nocc) ? phir[(long)(v + 1) * nr + rr] : 0.f;
     };
     auto place = [&](const Rows &d, int J) {
       const int v = J * kB + p2;
@@ -224,6 +254,7 @@ __global__ void __launch_bounds__(kThreads + 32, 1) k1d_tma_kernel(
     // column J: its blocks, then role A's rows of Y_J, then the rows of column J + 1 (from `next`)
     auto column = [&](int J, Rows &next) {
       zero_acc();
+      const int bj = RAG ? min(kB, nocc - J * kB) : kB;
       for (int I = 0; I <= J; ++I, ++g) {
         const int st = (int)(g % S);
         if (ok) {
@@ -244,16 +275,16 @@ __global__ void __launch_bounds__(kThreads + 32, 1) k1d_tma_kernel(
         if (I < J) {
           if (roleA) {
             // Y_J[jj] += sum_ii tau(ii, jj) a_I[ii], rows jj = r4 + k
-            mac4(T, I, [&](int k, int m) { return (r4 + k) * kB + m; });
+            mac4(T, I, kB, [&](int k, int m) { return (r4 + k) * kB + m; });
           } else {
             // Y_I[ii] += sum_jj tau(ii, jj) a_J[jj], rows ii = r4 + k
             zero_acc();
-            mac4(T, J, [&](int k, int m) { return m * kB + r4 + k; });
+            mac4(T, J, bj, [&](int k, int m) { return m * kB + r4 + k; });
             flush(I);
           }
         } else if (roleA) {
           // diagonal block: packed triangle of the symmetric 16 x 16 block, rows r4 + k of Y_J
-          mac4(T, J, [&](int k, int m) { return tri(m, r4 + k); });
+          mac4(T, J, bj, [&](int k, int m) { return tri(m, r4 + k); });
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[st]);  // release the stage
@@ -274,7 +305,8 @@ __global__ void __launch_bounds__(kThreads + 32, 1) k1d_tma_kernel(
         column(J + 1, ra);
       }
     }
-    if (!ok) continue;  // after a give-up: no epilogue; the next tile's first barrier ends the CTA
+    if (!ok || !live) continue;  // after a give-up: no epilogue; the next tile's first barrier ends the CTA
+                                 // (points past the grid exist in the last tile only)
     // epilogue: Y = V a + 2 v_H phi - (tau a), rows p2, p2 + 1 of every block as packed pairs
 #pragma unroll 2
     for (int X = 0; X < nblk; ++X) {
@@ -285,16 +317,34 @@ __global__ void __launch_bounds__(kThreads + 32, 1) k1d_tma_kernel(
         if (bb >= nb_total) break;
         const size_t e0 = idx(b, v) + (size_t)lane * LS, e1 = idx(b, v + 1) + (size_t)lane * LS;
         const long f = (long)bb * nocc + v;
-        Py[(f >> 1) * nr + rr] = make_float2(y_s[e0], y_s[e1]);
+        if (!RAG || ((f & 1) == 0 && v + 1 < nocc)) {
+          Py[(f >> 1) * nr + rr] = make_float2(y_s[e0], y_s[e1]);
+        } else {
+          // one by one; the unused partner of the last row of all is zero
+          float *Yf = reinterpret_cast<float *>(Py);
+          const long last = (long)nb_total * nocc - 1;
+          if (v < nocc) {
+            const long o = 2 * ((f >> 1) * nr + rr) + (f & 1);
+            Yf[o] = y_s[e0];
+            if (f == last && (f & 1) == 0) Yf[o + 1] = 0.f;
+          }
+          if (v + 1 < nocc) {
+            const long o = 2 * (((f + 1) >> 1) * nr + rr) + ((f + 1) & 1);
+            Yf[o] = y_s[e1];
+            if (f + 1 == last && ((f + 1) & 1) == 0) Yf[o + 1] = 0.f;
+          }
+        }
       }
     }
   }
 }
 
 constexpr size_t kSmemCap = 227 * 1024;
+constexpr size_t kSmemHalf = 113 * 1024;  // two CTAs per SM
 
 size_t smem_bytes(int nb, int stages, int nocc) {
-  return (size_t)stages * kStageBytes + 2 * (size_t)nb * nocc * kR * sizeof(float) + 2 * stages * 8 + 16;
+  const size_t rows = (size_t)(nocc + kB - 1) / kB * kB;
+  return (size_t)stages * kStageBytes + 2 * (size_t)nb * rows * kR * sizeof(float) + 2 * stages * 8 + 16;
 }
 
 // deepest ring (2..4 stages) that fits beside the a and Y tiles of nb vectors; 0 if none
@@ -304,24 +354,38 @@ int stages_for(int nb, int nocc) {
   return 0;
 }
 
-template <int NB, int S>
+template <int NB, int S, int CTAS = 1>
 void launch_s(const Ctx &c, const K1dTma &t, int nb, int b0, const float *phir, const float *vloc,
               const float2 *Pa, const float2 *Pvh, float2 *Py, bool use_vloc, bool use_k1e, int hold = 0) {
   const size_t smem = smem_bytes(NB, S, c.nocc);
-  BSE_CUDA(cudaFuncSetAttribute(k1d_tma_kernel<NB, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   // persistent: one CTA per SM (the ring and the a/Y tiles take most of the shared memory)
   int dev = 0, nsm = 0;
   BSE_CUDA(cudaGetDevice(&dev));
   BSE_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  const unsigned grid = (unsigned)std::min<long>(c.nr / kR, std::max(1, nsm));
-  k1d_tma_kernel<NB, S><<<grid, kThreads + 32, smem, c.stream>>>(t.tau, t.npairs, c.nr, c.nocc, nb, b0, phir, vloc,
-                                                                  Pa, Pvh, Py, use_vloc, use_k1e, t.err, hold);
+  const unsigned grid = (unsigned)std::min<long>((c.nr + kR - 1) / kR, CTAS * std::max(1, nsm));
+  auto go = [&](auto rag) {
+    auto kernel = k1d_tma_kernel<NB, S, decltype(rag)::value, CTAS>;
+    BSE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kernel<<<grid, kThreads + 32, smem, c.stream>>>(t.tau, t.npairs, c.nr, c.nocc, nb, b0, phir, vloc, Pa, Pvh, Py,
+                                                    use_vloc, use_k1e, t.err, hold);
+  };
+  if (k1d_tma_whole(c.nocc, c.nr)) go(std::false_type());
+  else go(std::true_type());
   BSE_CHECK_LAUNCH();
 }
 
 template <int NB>
 void launch(const Ctx &c, const K1dTma &t, int nb, int b0, const float *phir, const float *vloc, const float2 *Pa,
             const float2 *Pvh, float2 *Py, bool use_vloc, bool use_k1e, int hold = 0) {
+  if constexpr (NB <= 2) {
+    if (smem_bytes(NB, 2, c.nocc) <= kSmemHalf) {
+      if (smem_bytes(NB, 3, c.nocc) <= kSmemHalf)
+        launch_s<NB, 3, 2>(c, t, nb, b0, phir, vloc, Pa, Pvh, Py, use_vloc, use_k1e, hold);
+      else
+        launch_s<NB, 2, 2>(c, t, nb, b0, phir, vloc, Pa, Pvh, Py, use_vloc, use_k1e, hold);
+      return;
+    }
+  }
   const int st = stages_for(NB, c.nocc);
   if (st >= 4) launch_s<NB, 4>(c, t, nb, b0, phir, vloc, Pa, Pvh, Py, use_vloc, use_k1e, hold);
   else if (st == 3) launch_s<NB, 3>(c, t, nb, b0, phir, vloc, Pa, Pvh, Py, use_vloc, use_k1e, hold);
@@ -353,13 +417,18 @@ void wait_selftest(cudaStream_t s, int *err) {
   BSE_CHECK_LAUNCH();
 }
 
+// whole 16-orbital blocks and 32-point tiles
+bool k1d_tma_whole(int nocc, long nr) { return nocc % kB == 0 && nr % kR == 0; }
+
+// From one whole block on: with 17 orbitals on 36^3 one vector takes 18.6 us (combine_tau 31); below 16
+// a block would be mostly padding and the contraction is a few microseconds of latency either way.
 bool k1d_tma_supported(int nocc, long nr) {
-  // 16-orbital blocks; whole 32-point tiles
-  return nocc >= kB && nocc % kB == 0 && nr % kR == 0 && k1d_tma_max_nb(nocc) > 0;
+  (void)nr;
+  return nocc >= kB && k1d_tma_max_nb(nocc) > 0;
 }
 
 void k1d_tma_init(K1dTma &t, const float *tau, long npairs, long nr, int *err) {
-  BSE_REQUIRE(nr % kR == 0, "internal: tile-major tau needs whole 32-point tiles");
+  (void)nr;
   t.tau = tau;
   t.npairs = npairs;
   t.err = err;

@@ -459,7 +459,8 @@ template <class R> void drho(const Ctx &c, int nb, const R *phir, const CT<R> *P
 template <class R>
 void combine_tau(const Ctx &c, int nb, const R *phir, const R *vloc, const R *tau, const CT<R> *Pa,
                  const CT<R> *Pvh, CT<R> *Py, bool use_vloc, bool use_k1e, bool use_k1d);
-// T_w -= sigma_{vw} phi_v (and, when sym, T_v -= sigma_{vw} phi_w for v != w) for the pairs (v, w) of list
+// T_w -= sigma_{vw} phi_v (and, when sym, T_v -= sigma_{vw} phi_w for v != w) for np consecutive pairs
+// (v, w) of c.pairs (sym) or c.pairs_full, list pointing at the first
 template <class R>
 void sigma_contract(const Ctx &c, int np, const int2 *list, const CT<R> *Psig, const R *phir, R *T,
                     bool sym = true);

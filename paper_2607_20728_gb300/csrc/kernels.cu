@@ -4,6 +4,7 @@
 // Gamma-point functions are real in r, so two of them share one complex FFT: a packed
 // grid P holds f + i g.  Sphere coefficients use the real basis of the public header.
 #include <cmath>
+#include <type_traits>
 
 #include "internal.cuh"
 
@@ -191,22 +192,54 @@ __global__ void scale_cols_kernel(int rows, int cols, T *__restrict__ Q, const T
     Q[i] *= s[i % cols];
 }
 
-// Delta rho_b(r) = sum_v phi_v(r) a_{b,v}(r)  (Eq. 2b); a packed over f = b*nocc + v
-template <class R>
-__global__ void drho_kernel(long nr, int nocc, int nb, const R *__restrict__ phir,
-                            const typename Cx<R>::T *__restrict__ Pa, typename Cx<R>::T *__restrict__ Pd) {
+// Delta rho_b(r) = sum_v phi_v(r) a_{b,v}(r)  (Eq. 2b); a packed over f = b*nocc + v.  NB vectors b0.. at
+// once: phi is read once for all of them, and the orbitals go in pairs so that (EVEN: every vector starts on
+// an even f) both halves of a packed element are used by one load, four (FP64) or eight pairs in flight per thread.  Bound
+// by the reads of phi and a; against one vector and one half at a time: two vectors of 128 orbitals on 72^3,
+// FP32, 226 -> 115 us (85 at the copy rate), four of 48 on 36^3, FP64, 53 -> 30 us.
+template <class R, int NB, bool EVEN>
+__global__ void __launch_bounds__(256) drho_kernel(long nr, int nocc, int nb, int b0, const R *__restrict__ phir,
+                                                   const typename Cx<R>::T *__restrict__ Pa,
+                                                   typename Cx<R>::T *__restrict__ Pd) {
   const R *Pa_d = reinterpret_cast<const R *>(Pa);
   R *Pd_d = reinterpret_cast<R *>(Pd);
-  for (long r = blockIdx.x * (long)blockDim.x + threadIdx.x; r < nr; r += (long)gridDim.x * blockDim.x) {
-    for (int b = 0; b < nb; ++b) {
-      R s = 0;
-      for (int v = 0; v < nocc; ++v) {
-        const long f = (long)b * nocc + v;
-        s = fma(phir[(long)v * nr + r], Pa_d[2 * ((f >> 1) * nr + r) + (f & 1)], s);
+  const long r = blockIdx.x * (long)blockDim.x + threadIdx.x;
+  if (r >= nr) return;
+  R s[NB];
+#pragma unroll
+  for (int b = 0; b < NB; ++b) s[b] = 0;
+  int v = 0;
+#pragma unroll (sizeof(R) == sizeof(double) ? 4 : 8)
+  for (; v + 1 < nocc; v += 2) {
+    const R p0 = __ldg(&phir[(long)v * nr + r]), p1 = __ldg(&phir[(long)(v + 1) * nr + r]);
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const long f = (long)(b0 + b) * nocc + v;
+      R x, y;
+      if (EVEN) {
+        const typename Cx<R>::T a = __ldg(&Pa[(f >> 1) * nr + r]);
+        x = a.x;
+        y = a.y;
+      } else {
+        x = __ldg(&Pa_d[2 * ((f >> 1) * nr + r) + (f & 1)]);
+        y = __ldg(&Pa_d[2 * (((f + 1) >> 1) * nr + r) + ((f + 1) & 1)]);
       }
-      Pd_d[2 * ((long)(b >> 1) * nr + r) + (b & 1)] = s;
+      s[b] = fma(p1, y, fma(p0, x, s[b]));
     }
-    if (nb & 1) Pd_d[2 * ((long)(nb >> 1) * nr + r) + 1] = 0;
+  }
+  if (v < nocc) {
+    const R p0 = __ldg(&phir[(long)v * nr + r]);
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const long f = (long)(b0 + b) * nocc + v;
+      s[b] = fma(p0, __ldg(&Pa_d[2 * ((f >> 1) * nr + r) + (f & 1)]), s[b]);
+    }
+  }
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    const int bb = b0 + b;
+    Pd_d[2 * ((long)(bb >> 1) * nr + r) + (bb & 1)] = s[b];
+    if (bb == nb - 1 && (bb & 1) == 0) Pd_d[2 * ((long)(bb >> 1) * nr + r) + 1] = 0;
   }
 }
 
@@ -342,21 +375,46 @@ __global__ void add_packed_kernel(long nr, int nf, const R *__restrict__ T, type
   }
 }
 
-// T_w(r) += coef sigma_{vw}(r) phi_v(r) and, when sym and v != w, T_v(r) += coef sigma_{vw}(r) phi_w(r)
-template <class R>
-__global__ void sigma_contract_kernel(long nr, int np, const int2 *__restrict__ list,
-                                      const typename Cx<R>::T *__restrict__ Ps, const R *__restrict__ phir,
-                                      R *__restrict__ T, R coef, int sym) {
+// Contraction of the pairs p0 .. p0 + np - 1 of the canonical lists, one thread per point and orbital w:
+// TRI (pairs (v', v), v' <= v, at v (v + 1)/2 + v'): T_w += coef (sum_{v' <= w} sigma_{v'w} phi_v' +
+// sum_{v > w} sigma_{wv} phi_v); otherwise (all ordered pairs (v', v) at v nocc + v'):
+// T_w += coef sum_v' sigma_{v'w} phi_v'.  Each T is read and written once per batch; as a loop over the
+// pairs with one thread per point, which updated T in memory for every pair, 256 pairs of a 40^3 grid took
+// 84 us, now 26 (the reads of sigma and phi at the copy rate: 19).
+template <class R, bool TRI>
+__global__ void __launch_bounds__(256) sigma_contract_kernel(long nr, int nocc, long p0, int np,
+                                                             const typename Cx<R>::T *__restrict__ Ps,
+                                                             const R *__restrict__ phir, R *__restrict__ T, R coef) {
   const R *Ps_d = reinterpret_cast<const R *>(Ps);
-  for (long r = blockIdx.x * (long)blockDim.x + threadIdx.x; r < nr; r += (long)gridDim.x * blockDim.x) {
-    for (int p = 0; p < np; ++p) {
-      const int2 vw = list[p];
-      const R s = coef * Ps_d[2 * ((long)(p >> 1) * nr + r) + (p & 1)];
-      T[(long)vw.y * nr + r] = fma(s, phir[(long)vw.x * nr + r], T[(long)vw.y * nr + r]);
-      if (sym && vw.x != vw.y)
-        T[(long)vw.x * nr + r] = fma(s, phir[(long)vw.y * nr + r], T[(long)vw.x * nr + r]);
-    }
+  const long r = blockIdx.x * (long)blockDim.x + threadIdx.x;
+  const int w = blockIdx.y;
+  const long base = TRI ? (long)w * (w + 1) / 2 : (long)w * nocc;  // list place of the pair (0, w)
+  const int end = TRI ? w + 1 : nocc;
+  const int lo = (int)max(0L, min((long)end, p0 - base)), hi = (int)max(0L, min((long)end, p0 + np - base));
+  // TRI: pairs (w, v), v > w, of the batch: v (v + 1)/2 + w in [p0, p0 + np)
+  int va = nocc, vb = nocc;
+  if (TRI) {
+    auto first = [&](long p) {  // smallest v > w with v (v + 1)/2 + w >= p
+      int v = max(w + 1, (int)((sqrtf(8.f * (float)max(0L, p - w) + 1.f) - 1.f) * 0.5f) - 2);
+      while (v < nocc && (long)v * (v + 1) / 2 + w < p) ++v;
+      return v;
+    };
+    va = first(p0);
+    vb = min(nocc, first(p0 + np));
   }
+  if ((lo >= hi && va >= vb) || r >= nr) return;
+  R acc = 0;
+#pragma unroll 8
+  for (int v = lo; v < hi; ++v) {
+    const long k = base + v - p0;
+    acc = fma(__ldg(&Ps_d[2 * ((k >> 1) * nr + r) + (k & 1)]), __ldg(&phir[(long)v * nr + r]), acc);
+  }
+#pragma unroll 4
+  for (int v = va; v < vb; ++v) {
+    const long k = (long)v * (v + 1) / 2 + w - p0;
+    acc = fma(__ldg(&Ps_d[2 * ((k >> 1) * nr + r) + (k & 1)]), __ldg(&phir[(long)v * nr + r]), acc);
+  }
+  T[(long)w * nr + r] = fma(coef, acc, T[(long)w * nr + r]);
 }
 
 // Delta rho^(x) = sum_v a_v^2 - phi_v Psi_v  (Eq. 5 with Psi = O phi);  Delta rho^(z) = 2 sum_v Z_v phi_v  (Eq. 6)
@@ -643,8 +701,18 @@ void scale_cols(int rows, int cols, T *Q, const T *s, cudaStream_t st) {
 
 template <class R>
 void drho(const Ctx &c, int nb, const R *phir, const CT<R> *Pa, CT<R> *Pd) {
-  drho_kernel<R><<<nblocks(c.nr, 256), 256, 0, c.stream>>>(c.nr, c.nocc, nb, phir, Pa, Pd);
-  BSE_CHECK_LAUNCH();
+  const unsigned grid = (unsigned)((c.nr + 255) / 256);
+  auto go = [&](auto n, int b0) {
+    constexpr int NB = decltype(n)::value;
+    if (c.nocc % 2 == 0 || (NB == 1 && b0 % 2 == 0)) drho_kernel<R, NB, true><<<grid, 256, 0, c.stream>>>(c.nr, c.nocc, nb, b0, phir, Pa, Pd);
+    else drho_kernel<R, NB, false><<<grid, 256, 0, c.stream>>>(c.nr, c.nocc, nb, b0, phir, Pa, Pd);
+    BSE_CHECK_LAUNCH();
+  };
+  for (int b0 = 0; b0 < nb;) {
+    if (nb - b0 >= 4) go(std::integral_constant<int, 4>(), b0), b0 += 4;
+    else if (nb - b0 >= 2) go(std::integral_constant<int, 2>(), b0), b0 += 2;
+    else go(std::integral_constant<int, 1>(), b0), b0 += 1;
+  }
 }
 
 template <class R>
@@ -678,8 +746,13 @@ void combine_tau(const Ctx &c, int nb, const R *phir, const R *vloc, const R *ta
 
 template <class R>
 void sigma_contract(const Ctx &c, int np, const int2 *list, const CT<R> *Psig, const R *phir, R *T, bool sym) {
-  sigma_contract_kernel<R><<<nblocks(c.nr, 256), 256, 0, c.stream>>>(c.nr, np, list, Psig, phir, T, (R)-1,
-                                                                     sym ? 1 : 0);
+  const dim3 grid((unsigned)((c.nr + 255) / 256), (unsigned)c.nocc);
+  if (sym)
+    sigma_contract_kernel<R, true><<<grid, 256, 0, c.stream>>>(c.nr, c.nocc, (long)(list - c.pairs.get()), np, Psig,
+                                                               phir, T, (R)-1);
+  else
+    sigma_contract_kernel<R, false><<<grid, 256, 0, c.stream>>>(c.nr, c.nocc, (long)(list - c.pairs_full.get()), np,
+                                                                Psig, phir, T, (R)-1);
   BSE_CHECK_LAUNCH();
 }
 

@@ -605,6 +605,23 @@ void apply_h(Ctx &c, int kf, const double *X, double *HX, const double *shift) {
   }
 }
 
+// n real densities packed in P -> scale v_c * them (Eq. 2b), in place.  v_c is zero outside the density
+// sphere, so the density-sphere-pruned transforms do it where they fit, with the kernel fused: one density
+// on 72^3 takes 74 us in FP64 and 31 in FP32, the full-grid transforms and the product 167 and 49
+template <class R>
+void coulomb_packed(Ctx &c, int n, CT<R> *P, double scale) {
+  Grids<R> &g = c.grids<R>();
+  if (dens_fft_ok<R>(c)) {
+    dens_forward<R>(c, n, P, nullptr, 0.0, g.vcg.get(), (R)(scale / c.nr));
+    dens_inverse<R>(c, n, nullptr, 0.0, P);
+    return;
+  }
+  const int nq = (n + 1) / 2;
+  fft_exec(c, P, nq, -1);
+  k::mul_grid<R>(c.nr, nq, P, g.vcg.get(), (R)(scale / c.nr), c.stream);
+  fft_exec(c, P, nq, +1);
+}
+
 // P_c X for rows of `nf` functions with the occupied orbitals (nf = nvec * nocc); keeps S if asked
 // (fixed: split-K scratch of fixed size, for the apply path whose launches may be captured)
 void project_pc(Ctx &c, int nf, double *X, double *S_keep, DevBuf<double> *fixed = nullptr) {
@@ -699,11 +716,8 @@ void apply_liouville_t(Ctx &c, int nvec, const double *A, double *LA, int op, do
     }
     if (k1e) {
       // v_H = v_c * Delta rho (Eq. 2b)
-      const int nqb = (nb + 1) / 2;
       k::drho<R>(c, nb, g.phir.get(), g.work.get(), vh.get());
-      fft_exec(c, vh.get(), nqb, -1);
-      k::mul_grid<R>(c.nr, nqb, vh.get(), g.vcg.get(), (R)(vh_scale / c.nr), c.stream);
-      fft_exec(c, vh.get(), nqb, +1);
+      coulomb_packed<R>(c, nb, vh.get(), vh_scale);
       if (vh_keep) k::unpack_real<R, R>(c.nr, 1, vh.get(), vh_keep, c.stream);
     }
     combine_exec<R>(c, nb, g.work.get(), vh.get(), g.work2.get(), k1e, k1d);
@@ -737,7 +751,7 @@ std::vector<const void *> apply_fingerprint(const Ctx &c) {
   auto grids = [&f](const auto &g) {
     for (const void *p : {(const void *)g.work.get(), (const void *)g.work2.get(), (const void *)g.vh.get(),
                           (const void *)g.colbuf_apply.get(), (const void *)g.tau.get(), (const void *)g.phir.get(),
-                          (const void *)g.vloc.get(), (const void *)g.vcg.get()})
+                          (const void *)g.vloc.get(), (const void *)g.vcg.get(), (const void *)g.colbuf_dens.get()})
       f.push_back(p);
   };
   grids(c.g64);
@@ -925,11 +939,8 @@ void apply_wannier_t(Ctx &c, int nvec, const double *A, double *LA) {
       fft_exec(c, g.work.get(), nq, +1);
     }
     if (k1e) {
-      const int nqb = (nb + 1) / 2;
       k::drho<R>(c, nb, g.wphir.get(), g.work.get(), g.vh.get());
-      fft_exec(c, g.vh.get(), nqb, -1);
-      k::mul_grid<R>(c.nr, nqb, g.vh.get(), g.vcg.get(), (R)(1.0 / c.nr), c.stream);
-      fft_exec(c, g.vh.get(), nqb, +1);
+      coulomb_packed<R>(c, nb, g.vh.get(), 1.0);
     }
     {
       cudaEvent_t stop;
@@ -1795,9 +1806,7 @@ template <class R>
 void coulomb_grid(Ctx &c, R *rho) {
   Grids<R> &g = c.grids<R>();
   k::pack_real<R>(c.nr, 1, rho, g.work.get(), c.stream);
-  fft_exec(c, g.work.get(), 1, -1);
-  k::mul_grid<R>(c.nr, 1, g.work.get(), g.vcg.get(), (R)(1.0 / c.nr), c.stream);
-  fft_exec(c, g.work.get(), 1, +1);
+  coulomb_packed<R>(c, 1, g.work.get(), 1.0);
   k::unpack_real<R, R>(c.nr, 1, g.work.get(), rho, c.stream);
 }
 
@@ -2181,10 +2190,7 @@ void apply_b_t(Ctx &c, int nvec, const double *A, double *BA) {
     double *out = BA + (long)b * vlen;
     for (int f0 = 0; f0 < no; f0 += (int)capf) {
       const int nf = (int)std::min<long>(capf, no - f0);
-      const int nq = (nf + 1) / 2;
-      BSE_CUDA(cudaMemsetAsync(g.work.get(), 0, (size_t)nq * c.nr * sizeof(CT<R>), c.stream));
-      k::scatter_pairs<R, double>(c, nf, a + (long)f0 * c.npw, g.work.get(), 1.0 / std::sqrt(c.omega));
-      fft_exec(c, g.work.get(), nq, +1);
+      sphere_to_grid_util<R>(c, nf, a + (long)f0 * c.npw, g.work.get());
       k::unpack_real<R, R>(c.nr, nf, g.work.get(), g.bar.get() + (long)f0 * c.nr, c.stream);
     }
     BSE_CUDA(cudaMemsetAsync(g.bt.get(), 0, (size_t)no * c.nr * sizeof(R), c.stream));
@@ -2206,10 +2212,8 @@ void apply_b_t(Ctx &c, int nvec, const double *A, double *BA) {
     }
     for (int f0 = 0; f0 < no; f0 += (int)capf) {
       const int nf = (int)std::min<long>(capf, no - f0);
-      const int nq = (nf + 1) / 2;
       k::pack_real<R>(c.nr, nf, g.bt.get() + (long)f0 * c.nr, g.work.get(), c.stream);
-      fft_exec(c, g.work.get(), nq, -1);
-      k::gather_pairs<R, double>(c, nf, g.work.get(), out + (long)f0 * c.npw, std::sqrt(c.omega) / c.nr);
+      grid_to_sphere_util<R>(c, nf, g.work.get(), out + (long)f0 * c.npw);
     }
     project_pc(c, no, out, nullptr);
   }
@@ -2538,10 +2542,7 @@ void uvector_t(Ctx &c, int root, double *U) {
   const long capf = (long)(g.work.n / c.nr) * 2;
   for (int f0 = 0; f0 < c.nocc; f0 += (int)capf) {
     const int nf = (int)std::min<long>(capf, c.nocc - f0);
-    const int nq = (nf + 1) / 2;
-    BSE_CUDA(cudaMemsetAsync(g.work.get(), 0, (size_t)nq * c.nr * sizeof(CT<R>), c.stream));
-    k::scatter_pairs<R, double>(c, nf, A + (long)f0 * c.npw, g.work.get(), 1.0 / std::sqrt(c.omega));
-    fft_exec(c, g.work.get(), nq, +1);
+    sphere_to_grid_util<R>(c, nf, A + (long)f0 * c.npw, g.work.get());
     k::unpack_real<R, R>(c.nr, nf, g.work.get(), ar.get() + (long)f0 * c.nr, c.stream);
   }
   if (c.wan.on && k1d) {

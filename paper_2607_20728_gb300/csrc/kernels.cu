@@ -194,9 +194,10 @@ __global__ void scale_cols_kernel(int rows, int cols, T *__restrict__ Q, const T
 
 // Delta rho_b(r) = sum_v phi_v(r) a_{b,v}(r)  (Eq. 2b); a packed over f = b*nocc + v.  NB vectors b0.. at
 // once: phi is read once for all of them, and the orbitals go in pairs so that (EVEN: every vector starts on
-// an even f) both halves of a packed element are used by one load, four (FP64) or eight pairs in flight per thread.  Bound
-// by the reads of phi and a; against one vector and one half at a time: two vectors of 128 orbitals on 72^3,
-// FP32, 226 -> 115 us (85 at the copy rate), four of 48 on 36^3, FP64, 53 -> 30 us.
+// an even f) both halves of a packed element are used by one load, with two partial sums and eight pairs in
+// flight per thread (two for one FP64 vector: 128 orbitals on 72^3 143 us, with eight 166, one orbital at a
+// time 167).  Bound by the reads of phi and a; against one vector and one half at a time: two vectors of 128
+// orbitals on 72^3, FP32, 226 -> 107 us (85 at the copy rate), four of 48 on 36^3, FP64, 53 -> 30 us.
 template <class R, int NB, bool EVEN>
 __global__ void __launch_bounds__(256) drho_kernel(long nr, int nocc, int nb, int b0, const R *__restrict__ phir,
                                                    const typename Cx<R>::T *__restrict__ Pa,
@@ -205,11 +206,11 @@ __global__ void __launch_bounds__(256) drho_kernel(long nr, int nocc, int nb, in
   R *Pd_d = reinterpret_cast<R *>(Pd);
   const long r = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (r >= nr) return;
-  R s[NB];
+  R s[NB], t[NB];
 #pragma unroll
-  for (int b = 0; b < NB; ++b) s[b] = 0;
+  for (int b = 0; b < NB; ++b) s[b] = t[b] = 0;
   int v = 0;
-#pragma unroll (sizeof(R) == sizeof(double) ? 4 : 8)
+#pragma unroll (sizeof(R) == sizeof(double) && NB == 1 ? 2 : 8)
   for (; v + 1 < nocc; v += 2) {
     const R p0 = __ldg(&phir[(long)v * nr + r]), p1 = __ldg(&phir[(long)(v + 1) * nr + r]);
 #pragma unroll
@@ -224,7 +225,8 @@ __global__ void __launch_bounds__(256) drho_kernel(long nr, int nocc, int nb, in
         x = __ldg(&Pa_d[2 * ((f >> 1) * nr + r) + (f & 1)]);
         y = __ldg(&Pa_d[2 * (((f + 1) >> 1) * nr + r) + ((f + 1) & 1)]);
       }
-      s[b] = fma(p1, y, fma(p0, x, s[b]));
+      s[b] = fma(p0, x, s[b]);
+      t[b] = fma(p1, y, t[b]);
     }
   }
   if (v < nocc) {
@@ -238,7 +240,7 @@ __global__ void __launch_bounds__(256) drho_kernel(long nr, int nocc, int nb, in
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
     const int bb = b0 + b;
-    Pd_d[2 * ((long)(bb >> 1) * nr + r) + (bb & 1)] = s[b];
+    Pd_d[2 * ((long)(bb >> 1) * nr + r) + (bb & 1)] = s[b] + t[b];
     if (bb == nb - 1 && (bb & 1) == 0) Pd_d[2 * ((long)(bb >> 1) * nr + r) + 1] = 0;
   }
 }

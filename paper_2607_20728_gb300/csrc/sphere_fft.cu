@@ -19,6 +19,7 @@
 #include <algorithm>
 #include <map>
 #include <mutex>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -34,6 +35,7 @@ using namespace fftc;
 constexpr double kRs2 = 0.70710678118654752440;  // 1/sqrt(2)
 constexpr int kThreads = 256;
 constexpr int kXYThreads = 512;  // plane passes: more warps to hide the latency of the FP64 pipe
+constexpr int kZMax = 288;      // largest CTA of the fixed-point z passes (two per SM with 112 registers)
 constexpr size_t kSmemCap = 200 * 1024;
 
 template <class C>
@@ -491,6 +493,237 @@ __global__ void __launch_bounds__(kXYThreads) sph_xy_fx(FxArgs a, double2 *__res
   }
 }
 
+// ---- FP64 z passes on 64-bit fixed point ------------------------------------------------------------
+// The z passes of FP64 data: CG columns of a group in shared memory as [slot][z], consecutive threads on
+// consecutive columns, one power of two per CTA from the largest sum of |re| + |im| over a column.  As FP64
+// (32 lines of 72 points per CTA) they were bound by the FP64 pipe like the plane passes.
+struct FzArgs {
+  int N1, N2, N3, N3p, ncols_pad, CG;
+  const int *colpos;
+  const int4 *ent;
+  const int *ent_off;
+  fx::Axis ax;
+};
+
+// FP64 columns in A (synchronised) -> transformed columns as integers of the unit set on return; B: scratch
+template <int SG>
+__device__ fx::C2 *z_lines(const FzArgs &a, double2 *Ad, fx::C2 *B, fx::Unit &unit) {
+  __shared__ unsigned top, ltop;
+  if (threadIdx.x == 0) top = ltop = 0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  unsigned m = 0;
+  for (int l = warp; l < a.CG; l += nwarp)
+    for (int z = lane; z < a.N3; z += 32) {
+      const double2 u = Ad[l * a.N3p + z];
+      m = max(m, max(fx::high_abs(u.x), fx::high_abs(u.y)));
+    }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if (lane == 0) atomicMax(&top, m);
+  __syncthreads();
+  const int E = (int)(top >> 20);
+  for (int l = warp; l < a.CG; l += nwarp) {
+    unsigned s = 0;
+    for (int z = lane; z < a.N3; z += 32) {
+      const double2 u = Ad[l * a.N3p + z];
+      s += fx::mag(u.x, E) + fx::mag(u.y, E);
+    }
+    s = __reduce_add_sync(0xffffffffu, s);
+    if (lane == 0) atomicMax(&ltop, s);
+  }
+  __syncthreads();
+  const int e0 = E - 1043 + 32 - __clz(ltop);
+  unit.q = e0 - 61;
+  unit.bad = E >= 0x7ff;
+  return lines_fx<SG>(reinterpret_cast<fx::C2 *>(Ad), B, a.CG, StrideBase{a.N3p}, 1, a.ax, [&](const fx::C2 &c) {
+    return fx::C2{fx::from_double(__longlong_as_double(c.x), e0, 61), fx::from_double(__longlong_as_double(c.y), e0, 61)};
+  });
+}
+
+__global__ void __launch_bounds__(kZMax, 2) sph_z_inv_fx(FzArgs a, int nf, int npw, const double *__restrict__ X,
+                                                      double scale, double2 *__restrict__ colbuf) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  double2 *A = reinterpret_cast<double2 *>(sm_raw);
+  fx::C2 *B = reinterpret_cast<fx::C2 *>(A + (size_t)a.CG * a.N3p);
+  const int g = blockIdx.x, q = blockIdx.y;
+  for (int e = threadIdx.x; e < a.CG * a.N3p; e += blockDim.x) A[e] = make_double2(0, 0);
+  __syncthreads();
+  const double *f = X + (long)(2 * q) * npw;
+  const bool hasg = (2 * q + 1) < nf;
+  const double *h = X + (long)(2 * q + 1) * npw;
+  const int e0 = a.ent_off[g], e1 = a.ent_off[g + 1];
+  for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
+    const int4 en = __ldg(&a.ent[e]);
+    const int kk = en.x;
+    if (kk == 0) {
+      A[en.y] = make_double2(f[0] * scale, hasg ? h[0] * scale : 0.0);
+      continue;
+    }
+    const double r2 = kRs2 * scale;
+    const double fc = f[2 * kk - 1] * r2, fs = f[2 * kk] * r2;
+    const double gc = hasg ? h[2 * kk - 1] * r2 : 0.0, gs = hasg ? h[2 * kk] * r2 : 0.0;
+    A[en.y] = make_double2(fc - gs, fs + gc);  // c_f + i c_g at +G
+    A[en.z] = make_double2(fc + gs, gc - fs);  // conj(c_f) + i conj(c_g) at -G
+  }
+  __syncthreads();
+  fx::Unit unit{0, false};
+  const fx::C2 *F = z_lines<1>(a, A, B, unit);
+  double2 *dst = colbuf + (long)q * a.N3 * a.ncols_pad + (long)g * a.CG;
+  for (int e = threadIdx.x; e < a.CG * a.N3; e += blockDim.x) {
+    const int slot = e % a.CG, z = e / a.CG;
+    const fx::C2 u = F[slot * a.N3p + z];
+    dst[(long)z * a.ncols_pad + slot] = make_double2(unit(u.x), unit(u.y));
+  }
+}
+
+__global__ void __launch_bounds__(kZMax, 2) sph_z_fwd_fx(FzArgs a, int nf, int npw, const double2 *__restrict__ colbuf,
+                                                      double *__restrict__ Y, double scale,
+                                                      const double *__restrict__ Xd, const double *__restrict__ kin,
+                                                      const double *__restrict__ shift, int period,
+                                                      double shift_const) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  double2 *A = reinterpret_cast<double2 *>(sm_raw);
+  fx::C2 *B = reinterpret_cast<fx::C2 *>(A + (size_t)a.CG * a.N3p);
+  const int g = blockIdx.x, q = blockIdx.y;
+  const double2 *src = colbuf + (long)q * a.N3 * a.ncols_pad + (long)g * a.CG;
+  for (int e = threadIdx.x; e < a.CG * a.N3; e += blockDim.x) {
+    const int slot = e % a.CG, z = e / a.CG;
+    A[slot * a.N3p + z] = src[(long)z * a.ncols_pad + slot];
+  }
+  fx::Unit unit{0, false};
+  const fx::C2 *F = z_lines<-1>(a, A, B, unit);
+  const int f0 = 2 * q, f1 = 2 * q + 1;
+  const bool hasg = f1 < nf;
+  const double sh0 = (shift ? shift[f0 % period] : 0.0) + shift_const;
+  const double sh1 = (shift ? shift[f1 % period] : 0.0) + shift_const;
+  const int e0 = a.ent_off[g], e1 = a.ent_off[g + 1];
+  for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
+    const int4 en = __ldg(&a.ent[e]);
+    const int kk = en.x;
+    double a0, a1 = 0.0, b0, b1 = 0.0;
+    int i0, i1;
+    if (kk == 0) {
+      const fx::C2 v = F[en.y];
+      i0 = 0;
+      i1 = -1;
+      a0 = unit(v.x) * scale;
+      b0 = unit(v.y) * scale;
+    } else {
+      const fx::C2 Fp = F[en.y], Fm = F[en.z];
+      const double s = kRs2 * scale;
+      i0 = 2 * kk - 1;
+      i1 = 2 * kk;
+      a0 = unit(Fp.x + Fm.x) * s;
+      a1 = unit(Fp.y - Fm.y) * s;
+      b0 = unit(Fp.y + Fm.y) * s;
+      b1 = unit(Fm.x - Fp.x) * s;
+    }
+    if (Xd) {
+      a0 += (kin[i0] + sh0) * Xd[(long)f0 * npw + i0];
+      if (i1 >= 0) a1 += (kin[i1] + sh0) * Xd[(long)f0 * npw + i1];
+      if (hasg) {
+        b0 += (kin[i0] + sh1) * Xd[(long)f1 * npw + i0];
+        if (i1 >= 0) b1 += (kin[i1] + sh1) * Xd[(long)f1 * npw + i1];
+      }
+    }
+    Y[(long)f0 * npw + i0] = a0;
+    if (i1 >= 0) Y[(long)f0 * npw + i1] = a1;
+    if (hasg) {
+      Y[(long)f1 * npw + i0] = b0;
+      if (i1 >= 0) Y[(long)f1 * npw + i1] = b1;
+    }
+  }
+}
+
+// the pair pipelines' z passes (dsph_z_fwd, dsph_z_inv below) for FP64 data
+__global__ void __launch_bounds__(kZMax, 2) dsph_z_fwd_fx(FzArgs a, int np, int npw, double2 *__restrict__ colbuf,
+                                                       double *__restrict__ X, double scale,
+                                                       const double *__restrict__ vcg, double cscale) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  double2 *A = reinterpret_cast<double2 *>(sm_raw);
+  fx::C2 *B = reinterpret_cast<fx::C2 *>(A + (size_t)a.CG * a.N3p);
+  const int g = blockIdx.x, q = blockIdx.y;
+  double2 *col = colbuf + (long)q * a.N3 * a.ncols_pad + (long)g * a.CG;
+  for (int e = threadIdx.x; e < a.CG * a.N3; e += blockDim.x) {
+    const int slot = e % a.CG, z = e / a.CG;
+    A[slot * a.N3p + z] = col[(long)z * a.ncols_pad + slot];
+  }
+  fx::Unit unit{0, false};
+  const fx::C2 *F = z_lines<-1>(a, A, B, unit);
+  if (X) {
+    const int f0 = 2 * q, f1 = 2 * q + 1;
+    const bool hasg = f1 < np;
+    for (int e = a.ent_off[g] + threadIdx.x; e < a.ent_off[g + 1]; e += blockDim.x) {
+      const int4 en = __ldg(&a.ent[e]);
+      const int kk = en.x;
+      if (kk == 0) {
+        const fx::C2 v = F[en.y];
+        X[(long)f0 * npw] = unit(v.x) * scale;
+        if (hasg) X[(long)f1 * npw] = unit(v.y) * scale;
+        continue;
+      }
+      const fx::C2 Fp = F[en.y], Fm = F[en.z];
+      const double sc = kRs2 * scale;
+      X[(long)f0 * npw + 2 * kk - 1] = unit(Fp.x + Fm.x) * sc;
+      X[(long)f0 * npw + 2 * kk] = unit(Fp.y - Fm.y) * sc;
+      if (hasg) {
+        X[(long)f1 * npw + 2 * kk - 1] = unit(Fp.y + Fm.y) * sc;
+        X[(long)f1 * npw + 2 * kk] = unit(Fm.x - Fp.x) * sc;
+      }
+    }
+  }
+  const long np2 = (long)a.N1 * a.N2;
+  for (int e = threadIdx.x; e < a.CG * a.N3; e += blockDim.x) {
+    const int slot = e % a.CG, z = e / a.CG;
+    const int pos = __ldg(&a.colpos[g * a.CG + slot]);
+    const double w = pos >= 0 ? vcg[(long)z * np2 + pos] * cscale : 0.0;
+    const fx::C2 v = F[slot * a.N3p + z];
+    col[(long)z * a.ncols_pad + slot] = pos >= 0 ? make_double2(unit(v.x) * w, unit(v.y) * w) : make_double2(0.0, 0.0);
+  }
+}
+
+__global__ void __launch_bounds__(kZMax, 2) dsph_z_inv_fx(FzArgs a, int np, int npw, const double *__restrict__ X,
+                                                       double scale, double2 *__restrict__ colbuf) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  double2 *A = reinterpret_cast<double2 *>(sm_raw);
+  fx::C2 *B = reinterpret_cast<fx::C2 *>(A + (size_t)a.CG * a.N3p);
+  const int g = blockIdx.x, q = blockIdx.y;
+  double2 *col = colbuf + (long)q * a.N3 * a.ncols_pad + (long)g * a.CG;
+  for (int e = threadIdx.x; e < a.CG * a.N3; e += blockDim.x) {
+    const int slot = e % a.CG, z = e / a.CG;
+    A[slot * a.N3p + z] = col[(long)z * a.ncols_pad + slot];
+  }
+  __syncthreads();
+  if (X) {
+    const double *f = X + (long)(2 * q) * npw;
+    const bool hasg = (2 * q + 1) < np;
+    const double *h = X + (long)(2 * q + 1) * npw;
+    for (int e = a.ent_off[g] + threadIdx.x; e < a.ent_off[g + 1]; e += blockDim.x) {
+      const int4 en = __ldg(&a.ent[e]);
+      const int kk = en.x;
+      double2 &tp = A[en.y];
+      if (kk == 0) {
+        tp = make_double2(tp.x + f[0] * scale, tp.y + (hasg ? h[0] * scale : 0.0));
+        continue;
+      }
+      const double r2 = kRs2 * scale;
+      const double fc = f[2 * kk - 1] * r2, fs = f[2 * kk] * r2;
+      const double gc = hasg ? h[2 * kk - 1] * r2 : 0.0, gs = hasg ? h[2 * kk] * r2 : 0.0;
+      tp = make_double2(tp.x + (fc - gs), tp.y + (fs + gc));
+      double2 &tm = A[en.z];
+      tm = make_double2(tm.x + (fc + gs), tm.y + (gc - fs));
+    }
+    __syncthreads();
+  }
+  fx::Unit unit{0, false};
+  const fx::C2 *F = z_lines<1>(a, A, B, unit);
+  for (int e = threadIdx.x; e < a.CG * a.N3; e += blockDim.x) {
+    const int slot = e % a.CG, z = e / a.CG;
+    const fx::C2 u = F[slot * a.N3p + z];
+    col[(long)z * a.ncols_pad + slot] = make_double2(unit(u.x), unit(u.y));
+  }
+}
+
 // ---- pair pipelines on the density sphere (tau build, U vector; Eq. 2c and Eq. 3) ----------
 // forward z pass: z lines of the occupied density columns, then the wave-function-sphere
 // coefficients of the two packed pair densities into X (real basis, type R, times `scale`) for
@@ -636,20 +869,24 @@ void set_attrs() {
   std::lock_guard<std::mutex> lock(mu);
   if (done[dev]) return;
   const int cap = (int)kSmemCap;
-  BSE_CUDA(cudaFuncSetAttribute(sph_z_inv<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-  BSE_CUDA(cudaFuncSetAttribute(sph_z_fwd<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
   if constexpr (sizeof(C) == sizeof(double2)) {
+    BSE_CUDA(cudaFuncSetAttribute(sph_z_inv_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    BSE_CUDA(cudaFuncSetAttribute(sph_z_fwd_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    BSE_CUDA(cudaFuncSetAttribute(dsph_z_fwd_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    BSE_CUDA(cudaFuncSetAttribute(dsph_z_inv_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
     BSE_CUDA(cudaFuncSetAttribute(sph_xy_fx<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
     BSE_CUDA(cudaFuncSetAttribute(sph_xy_fx<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
     BSE_CUDA(cudaFuncSetAttribute(sph_xy_fx<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
   } else {
+    using R = typename RealOf<C>::T;
+    BSE_CUDA(cudaFuncSetAttribute(sph_z_inv<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    BSE_CUDA(cudaFuncSetAttribute(sph_z_fwd<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    BSE_CUDA(cudaFuncSetAttribute(dsph_z_fwd<C, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    BSE_CUDA(cudaFuncSetAttribute(dsph_z_inv<C, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
     BSE_CUDA(cudaFuncSetAttribute(sph_xy<C, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
     BSE_CUDA(cudaFuncSetAttribute(sph_xy<C, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
     BSE_CUDA(cudaFuncSetAttribute(sph_xy<C, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
   }
-  using R = typename RealOf<C>::T;
-  BSE_CUDA(cudaFuncSetAttribute(dsph_z_fwd<C, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-  BSE_CUDA(cudaFuncSetAttribute(dsph_z_inv<C, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
   done[dev] = true;
 }
 
@@ -676,10 +913,74 @@ void launch_xy(Ctx &c, const SphereFFT &s, int nq, C *cb, C *P, const typename R
       for (int r = 0; r < 12; ++r) a.ax[i].radix[r] = x.radix[r];
       a.ax[i].tw = x.twx;
     }
-    sph_xy_fx<MODE><<<grid, xy_threads(c), xy_smem<C>(c), c.stream>>>(a, cb, P, v);
+    // planes of which two or more fit an SM go 256 threads each when there is more than one wave of them
+    // (24 grids of 36^2 planes: inverse 48 us with 512, 32 with 256; 54^2 114 and 90; 60^2, one per SM,
+    // 148 and 166; a single grid 10.9 and 11.6)
+    const bool pair = 2 * xy_smem<C>(c) <= 220 * 1024 && (long)c.N[2] * nq > 152;
+    sph_xy_fx<MODE><<<grid, c.xy_threads > 0 ? xy_threads(c) : (pair ? 256 : kXYThreads), xy_smem<C>(c), c.stream>>>(
+        a, cb, P, v);
   } else {
     sph_xy<C, MODE><<<grid, xy_threads(c), xy_smem<C>(c), c.stream>>>(make_args<C>(c, s), cb, P, v);
   }
+  BSE_CHECK_LAUNCH();
+}
+
+FzArgs fz_args(const Ctx &c, const SphereFFT &s) {
+  FzArgs a;
+  a.N1 = c.N[0];
+  a.N2 = c.N[1];
+  a.N3 = c.N[2];
+  a.N3p = c.N[2] + 1;
+  a.ncols_pad = s.ncols_pad;
+  a.CG = s.cg;
+  a.colpos = s.colpos.get();
+  a.ent = s.ent.get();
+  a.ent_off = s.ent_off.get();
+  const FFTAxis &x = c.fft.ax[2];
+  a.ax.n = x.n;
+  a.ax.nstage = x.nstage;
+  for (int r = 0; r < 12; ++r) a.ax.radix[r] = x.radix[r];
+  a.ax.tw = x.twx;
+  return a;
+}
+// threads of a fixed-point z pass: a stage of radix R takes N3/R rounds of one warp (32 columns), so the
+// warp count (6 to 9) is the one with the fewest rounds over all stages per warp of occupancy
+int z_threads(const Ctx &c) {
+  const FFTAxis &x = c.fft.ax[2];
+  int best = 8;
+  double bc = 1e30;
+  for (int w = 6; w <= kZMax / 32; ++w) {
+    double rounds = 0;
+    for (int s = 0; s < x.nstage; ++s) rounds += (x.n / x.radix[s] + w - 1) / w;
+    const double cost = rounds * w;
+    if (cost < bc - 1e-9) {
+      bc = cost;
+      best = w;
+    }
+  }
+  return best * 32;
+}
+
+// the z passes of either precision: FP64 in fixed point, FP32 as it is
+template <class C>
+void launch_z_inv(Ctx &c, int nf, int nq, const double *X, double scale, C *cb) {
+  const dim3 grid(c.sfft.ngroups, nq);
+  if constexpr (sizeof(C) == sizeof(double2))
+    sph_z_inv_fx<<<grid, z_threads(c), z_smem<C>(c), c.stream>>>(fz_args(c, c.sfft), nf, c.npw, X, scale, cb);
+  else
+    sph_z_inv<C><<<grid, kThreads, z_smem<C>(c), c.stream>>>(make_args<C>(c, c.sfft), nf, c.npw, X, scale, cb);
+  BSE_CHECK_LAUNCH();
+}
+template <class C>
+void launch_z_fwd(Ctx &c, int nf, int nq, const C *cb, double *Y, double scale, const double *Xd, const double *shift,
+                  int period, double shift_const) {
+  const dim3 grid(c.sfft.ngroups, nq);
+  if constexpr (sizeof(C) == sizeof(double2))
+    sph_z_fwd_fx<<<grid, z_threads(c), z_smem<C>(c), c.stream>>>(fz_args(c, c.sfft), nf, c.npw, cb, Y, scale, Xd,
+                                                               c.kin.get(), shift, period, shift_const);
+  else
+    sph_z_fwd<C><<<grid, kThreads, z_smem<C>(c), c.stream>>>(make_args<C>(c, c.sfft), nf, c.npw, cb, Y, scale, Xd,
+                                                             c.kin.get(), shift, period, shift_const);
   BSE_CHECK_LAUNCH();
 }
 
@@ -798,13 +1099,17 @@ void dens_forward(Ctx &c, int np, CT<R> *P, R *X, double scale, const R *vcg, R 
   using C = CT<R>;
   const int nq = (np + 1) / 2;
   set_attrs<C>();
-  SphArgs<C> a = make_args<C>(c, c.dfft);
   Grids<R> &g = c.grids<R>();
   g.colbuf_dens.alloc((size_t)nq * c.N[2] * c.dfft.ncols_pad);
   C *cb = g.colbuf_dens.get();
   launch_xy<C, 1>(c, c.dfft, nq, cb, P, nullptr);
-  dsph_z_fwd<C, R><<<dim3(c.dfft.ngroups, nq), kThreads, z_smem<C>(c, c.dfft), c.stream>>>(a, np, c.npw, cb, X,
-                                                                                         scale, vcg, cscale);
+  const dim3 grid(c.dfft.ngroups, nq);
+  if constexpr (std::is_same<R, double>::value)
+    dsph_z_fwd_fx<<<grid, z_threads(c), z_smem<C>(c, c.dfft), c.stream>>>(fz_args(c, c.dfft), np, c.npw, cb, X, scale,
+                                                                        vcg, cscale);
+  else
+    dsph_z_fwd<C, R><<<grid, kThreads, z_smem<C>(c, c.dfft), c.stream>>>(make_args<C>(c, c.dfft), np, c.npw, cb, X,
+                                                                         scale, vcg, cscale);
   BSE_CHECK_LAUNCH();
 }
 
@@ -814,10 +1119,13 @@ void dens_inverse(Ctx &c, int np, const R *X, double scale, CT<R> *P) {
   using C = CT<R>;
   const int nq = (np + 1) / 2;
   set_attrs<C>();
-  SphArgs<C> a = make_args<C>(c, c.dfft);
   C *cb = c.grids<R>().colbuf_dens.get();
-  dsph_z_inv<C, R><<<dim3(c.dfft.ngroups, nq), kThreads, z_smem<C>(c, c.dfft), c.stream>>>(a, np, c.npw, X, scale,
-                                                                                         cb);
+  const dim3 grid(c.dfft.ngroups, nq);
+  if constexpr (std::is_same<R, double>::value)
+    dsph_z_inv_fx<<<grid, z_threads(c), z_smem<C>(c, c.dfft), c.stream>>>(fz_args(c, c.dfft), np, c.npw, X, scale, cb);
+  else
+    dsph_z_inv<C, R><<<grid, kThreads, z_smem<C>(c, c.dfft), c.stream>>>(make_args<C>(c, c.dfft), np, c.npw, X, scale,
+                                                                         cb);
   BSE_CHECK_LAUNCH();
   launch_xy<C, 0>(c, c.dfft, nq, cb, P, nullptr);
 }
@@ -840,10 +1148,8 @@ void sphere_to_grid(Ctx &c, int nf, const double *X, CT<R> *P, double scale, CT<
   if (nf <= 0) return;
   const int nq = (nf + 1) / 2;
   set_attrs<C>();
-  SphArgs<C> a = make_args<C>(c, c.sfft);
   C *cb = colbuf ? colbuf : colbuf_for<R>(c, nq);
-  sph_z_inv<C><<<dim3(c.sfft.ngroups, nq), kThreads, z_smem<C>(c), c.stream>>>(a, nf, c.npw, X, scale, cb);
-  BSE_CHECK_LAUNCH();
+  launch_z_inv<C>(c, nf, nq, X, scale, cb);
   launch_xy<C, 0>(c, c.sfft, nq, cb, P, nullptr);
 }
 
@@ -854,12 +1160,9 @@ void grid_to_sphere(Ctx &c, int nf, CT<R> *P, double *Y, double scale, const dou
   if (nf <= 0) return;
   const int nq = (nf + 1) / 2;
   set_attrs<C>();
-  SphArgs<C> a = make_args<C>(c, c.sfft);
   C *cb = colbuf ? colbuf : colbuf_for<R>(c, nq);
   launch_xy<C, 1>(c, c.sfft, nq, cb, P, nullptr);
-  sph_z_fwd<C><<<dim3(c.sfft.ngroups, nq), kThreads, z_smem<C>(c), c.stream>>>(
-      a, nf, c.npw, cb, Y, scale, Xd, c.kin.get(), shift, period > 0 ? period : 1, shift_const);
-  BSE_CHECK_LAUNCH();
+  launch_z_fwd<C>(c, nf, nq, cb, Y, scale, Xd, shift, period > 0 ? period : 1, shift_const);
 }
 
 template <class R>
@@ -868,15 +1171,11 @@ void sphere_h(Ctx &c, int nf, const double *X, double *HX, const double *shift) 
   if (nf <= 0) return;
   const int nq = (nf + 1) / 2;
   set_attrs<C>();
-  SphArgs<C> a = make_args<C>(c, c.sfft);
   C *cb = colbuf_for<R>(c, nq);
   const double s_in = 1.0 / std::sqrt(c.omega), s_out = std::sqrt(c.omega) / (double)c.nr;
-  sph_z_inv<C><<<dim3(c.sfft.ngroups, nq), kThreads, z_smem<C>(c), c.stream>>>(a, nf, c.npw, X, s_in, cb);
-  BSE_CHECK_LAUNCH();
+  launch_z_inv<C>(c, nf, nq, X, s_in, cb);
   launch_xy<C, 2>(c, c.sfft, nq, cb, nullptr, c.grids<R>().vloc.get());
-  sph_z_fwd<C><<<dim3(c.sfft.ngroups, nq), kThreads, z_smem<C>(c), c.stream>>>(
-      a, nf, c.npw, cb, HX, s_out, X, c.kin.get(), shift, shift ? c.nocc : 1, 0.0);
-  BSE_CHECK_LAUNCH();
+  launch_z_fwd<C>(c, nf, nq, cb, HX, s_out, X, shift, shift ? c.nocc : 1, 0.0);
 }
 
 template bool sphere_fft_ok<double>(const Ctx &);

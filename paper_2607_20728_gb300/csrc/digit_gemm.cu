@@ -26,13 +26,13 @@
 namespace bse {
 namespace {
 
-constexpr int kKC = 32;             // k per staged chunk
+constexpr int kKC = 16;             // k per staged chunk
 constexpr int kRawStride = kKC + 2;  // doubles per staged row (16-byte aligned, rows off the same banks)
 constexpr int kDigStride = kKC + 8;  // bf16 per digit row: ldmatrix reads 8 rows without bank conflicts
-constexpr int kMaxStrips = 10;      // 16-row strips of A and B per CTA
+constexpr int kMaxStrips = 9;       // 16-row strips of A and B per CTA
 constexpr int kRows = 16 * kMaxStrips;
 constexpr int kWarps = 16;
-constexpr int kFlush = 4;           // chunks between reads of the FP32 accumulators (128 k)
+constexpr int kFlush = 8;           // chunks between reads of the FP32 accumulators (128 k)
 constexpr int kBadExp = 1 << 28;    // row holds a non-finite value
 constexpr int kMaxSlice = 1 << 19;  // longest K slice
 
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(256) row_exponents(int M, int N, int K, bool a
   if (across) {
     const int row = blk * 32 + lane;
     if (row < rows)
-#pragma unroll 4
+#pragma unroll 8
       for (int k = warp; k < K; k += 8) m = max(m, bits(__ldg(&X[(long)k * ld + row])));
     red[warp][lane] = m;
     __syncthreads();
@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(256) row_exponents(int M, int N, int K, bool a
     }
   } else {
     const double *x = X + (long)blk * ld;
-#pragma unroll 4
+#pragma unroll 8
     for (int k = threadIdx.x; k < K; k += 256) m = max(m, bits(__ldg(&x[k])));
     for (int w = 16; w > 0; w >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, w));
     if (lane == 0) red[0][warp] = m;
@@ -126,58 +126,66 @@ __global__ void __launch_bounds__(256) row_exponents(int M, int N, int K, bool a
 
 template <int ND>
 constexpr size_t digit_smem() {
-  return (size_t)kRows * kRawStride * 8 + (size_t)ND * kRows * kDigStride * 2 +
-         (ND == 8 ? (size_t)kWarps * 32 * 8 * 16 : 0) + kRows * 4;
+  return (size_t)2 * kRows * kRawStride * 8 + (size_t)2 * ND * kRows * kDigStride * 2 +
+         (ND == 8 ? (size_t)kWarps * 32 * 8 * 16 : 0) + kRows * 12;
 }
 
 // One CTA: SM x SN warps (at most 16), each a 16 x 16 block of C over k in its K slice; the SM strips of
 // A and SN strips of B (16 rows each) are staged as FP64 by cp.async, rewritten as digits by all threads
-// and multiplied from the digit planes.  The next chunk's FP64 rows arrive while this one is multiplied.
-// Bound by the tensor pipe (86 mma.sync of 2 clocks per warp and 16 k) and, beside it, the integer work
-// of the rewriting (about 40 instructions per value).  Strips past the end of C skip their products.
+// and multiplied from the digit planes.  Two buffers of each: in every step the next chunk is rewritten
+// and this one multiplied between the same two barriers, the even warps rewriting first and the odd ones
+// multiplying first, so that rewriting (FP64 and integer pipes) and products (tensor pipe) overlap.
+// 512 x 128 x 6859 takes 166 us; with the rewriting left out 136, with the products left out 115, and the
+// tensor pipe alone (86 mma.sync of two clocks per warp and 16 k) would take 69: with four warps per
+// scheduler and a barrier per 16 k, neither phase fills its pipe.  Strips past the end of C skip their
+// products.
 template <bool TA, bool TB, int ND>
 __global__ void __launch_bounds__(kWarps * 32, 1)
     digit_gemm_kernel(int M, int N, int K, int kslice, int SM, int SN, const double *__restrict__ A, int lda,
                       const double *__restrict__ B, int ldb, const int *__restrict__ ex, double alpha, double beta,
                       double *__restrict__ C, int ldc, double *__restrict__ part) {
   extern __shared__ __align__(16) unsigned char smem[];
-  double *raw = reinterpret_cast<double *>(smem);                                          // [rows][kRawStride]
-  __nv_bfloat16 *dig = reinterpret_cast<__nv_bfloat16 *>(raw + kRows * kRawStride);        // [ND][rows][kDigStride]
-  longlong2 *sums = reinterpret_cast<longlong2 *>(dig + (size_t)ND * kRows * kDigStride);  // [8][512] (ND = 8)
-  int *rexp = reinterpret_cast<int *>(reinterpret_cast<unsigned char *>(sums) +
-                                      (ND == 8 ? (size_t)kWarps * 32 * 8 * 16 : 0));
+  double *raw = reinterpret_cast<double *>(smem);                                  // [2][rows][kRawStride]
+  __nv_bfloat16 *dig = reinterpret_cast<__nv_bfloat16 *>(raw + 2 * kRows * kRawStride);  // [2][ND][rows][kDigStride]
+  longlong2 *sums = reinterpret_cast<longlong2 *>(dig + (size_t)2 * ND * kRows * kDigStride);  // [8][512] (ND = 8)
+  double *rscale = reinterpret_cast<double *>(reinterpret_cast<unsigned char *>(sums) +
+                                              (ND == 8 ? (size_t)kWarps * 32 * 8 * 16 : 0));
+  int *rexp = reinterpret_cast<int *>(rscale + kRows);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rows_a = 16 * SM, rows = 16 * (SM + SN);
   const int m0 = blockIdx.y * rows_a, n0 = blockIdx.x * 16 * SN;
   const int kbeg = blockIdx.z * kslice, kend = min(K, kbeg + kslice);
+  __shared__ int tiny;
+  if (tid == 0) tiny = 0;
+  __syncthreads();
   for (int r = tid; r < rows; r += blockDim.x) {
     const bool a = r < rows_a;
     const int g = a ? m0 + r : n0 + r - rows_a;
     int e = 0;
     if (g < (a ? M : N)) e = ex[a ? g : M + g];
-    rexp[r] = e == kBadExp ? 0 : e;
+    rexp[r] = e = e == kBadExp ? 0 : e;
+    // 2^(kBits - e), rows of very small numbers (where that could overflow) converted by to_fixed
+    if (e > -900) rscale[r] = __longlong_as_double((long long)(1023 + 7 * ND - 1 - e) << 52);
+    else atomicOr(&tiny, 1);
   }
-  auto load = [&](int k0) {
-    // 8-byte copies, consecutive threads along the contiguous direction of each operand
-    const int na = rows_a * kKC, nt = rows * kKC;
-    for (int i = tid; i < nt; i += kWarps * 32) {
-      const bool a = i < na;
-      const int j = a ? i : i - na;
-      int r, k;
-      if (a ? TA : !TB) {
-        const int nr = a ? rows_a : rows - rows_a;
-        k = j / nr;
-        r = j - k * nr;
-      } else {
-        r = j / kKC;
-        k = j % kKC;
-      }
-      const int g = (a ? m0 : n0) + r, gk = k0 + k;
-      const bool ok = g < (a ? M : N) && gk < kend;
-      const double *src = a ? A : B;
-      if (ok) src += a ? (TA ? (long)gk * lda + g : (long)g * lda + gk) : (TB ? (long)g * ldb + gk : (long)gk * ldb + g);
-      cp_async8(&raw[(a ? r : rows_a + r) * kRawStride + k], src, ok);
+  // 8-byte copies of 32-row groups of each operand, consecutive threads along its contiguous direction: a
+  // thread keeps its k and its row within the group, so an address is one pointer plus a stride
+  auto load_part = [&](const double *X, bool across, int ld, int x0, int rows_x, int n_x, int row_off, int k0, int buf) {
+    const int r0 = across ? lane : tid / kKC, k = across ? warp : tid % kKC;
+    const bool kok = k0 + k < kend;
+    const double *src = X + (across ? (long)(k0 + k) * ld + x0 + r0 : (long)(x0 + r0) * ld + k0 + k);
+    const long step = across ? 32 : 32L * ld;
+    double *dst = raw + (buf * kRows + row_off + r0) * kRawStride + k;
+    for (int r = r0; r < rows_x; r += 32) {
+      const bool ok = kok && x0 + r < n_x;
+      cp_async8(dst, ok ? src : X, ok);
+      src += step;
+      dst += 32 * kRawStride;
     }
+  };
+  auto load = [&](int k0, int buf) {
+    load_part(A, TA, lda, m0, rows_a, M, 0, k0, buf);
+    load_part(B, !TB, ldb, n0, rows - rows_a, N, rows_a, k0, buf);
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   const int wm = warp / SN, wn = warp - wm * SN;
@@ -202,71 +210,93 @@ __global__ void __launch_bounds__(kWarps * 32, 1)
 #pragma unroll
     for (int o = 0; o < 8; ++o) one[o] = 0;
   }
-  load(kbeg);
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
-  __syncthreads();
-  int held = 0;
-  for (int k0 = kbeg; k0 < kend; k0 += kKC) {
-    // FP64 -> digits, two k per thread and step
+  constexpr unsigned kBuffer = ND * kPlane;
+  // FP64 -> digits, two k per thread and step
+  auto rewrite = [&](int buf) {
     for (int i = tid; i < rows * (kKC / 2); i += kWarps * 32) {
       const int r = i / (kKC / 2), kp = i % (kKC / 2);
-      const double2 x = *reinterpret_cast<const double2 *>(&raw[r * kRawStride + 2 * kp]);
-      const int e = rexp[r];
-      const unsigned long long y0 = (unsigned long long)to_fixed<ND>(x.x, e) + digit_bias<ND>();
-      const unsigned long long y1 = (unsigned long long)to_fixed<ND>(x.y, e) + digit_bias<ND>();
-      unsigned *d = reinterpret_cast<unsigned *>(dig + r * kDigStride + 2 * kp);
+      const double2 x = *reinterpret_cast<const double2 *>(&raw[(buf * kRows + r) * kRawStride + 2 * kp]);
+      unsigned long long y0, y1;
+      if (!tiny) {
+        // the scaling is exact and the conversion rounds to nearest: the FP64 pipe is free here
+        const double sc = rscale[r];
+        y0 = (unsigned long long)__double2ll_rn(x.x * sc) + digit_bias<ND>();
+        y1 = (unsigned long long)__double2ll_rn(x.y * sc) + digit_bias<ND>();
+      } else {
+        y0 = (unsigned long long)to_fixed<ND>(x.x, rexp[r]) + digit_bias<ND>();
+        y1 = (unsigned long long)to_fixed<ND>(x.y, rexp[r]) + digit_bias<ND>();
+      }
+      unsigned *d = reinterpret_cast<unsigned *>(dig + (size_t)buf * (kBuffer / 2) + r * kDigStride + 2 * kp);
 #pragma unroll
       for (int s = 0; s < ND; ++s) {
         const int sh = 7 * (ND - 1 - s);
         // the leading field reaches 128; a 7-bit field u next to the BF16 bits of 128 reads 128 + u
         const unsigned msk = s == 0 ? 0xffu : 0x7fu;
-        const unsigned u = ((unsigned)(y0 >> sh) & msk) + (((unsigned)(y1 >> sh) & msk) << 16) + 0x43004300u;
+        const unsigned hi = sh >= 16 ? (unsigned)(y1 >> (sh >= 16 ? sh - 16 : 0)) : (unsigned)(y1 << (sh < 16 ? 16 - sh : 0));
+        const unsigned u = ((unsigned)(y0 >> sh) & msk) | 0x43004300u | (hi & (msk << 16));
         __nv_bfloat162 w = __hsub2(*reinterpret_cast<const __nv_bfloat162 *>(&u), __float2bfloat162_rn(192.f));
         d[s * (kPlane / 4)] = *reinterpret_cast<const unsigned *>(&w);
       }
     }
-    __syncthreads();
-    if (k0 + kKC < kend) load(k0 + kKC);
-    if (active) {
+  };
+  auto multiply = [&](int buf) {
+    unsigned a[ND][4];
 #pragma unroll
-      for (int kk = 0; kk < kKC / 16; ++kk) {
-        unsigned a[ND][4];
+    for (int s = 0; s < ND; ++s) ldmatrix4(a[s], a_addr + buf * kBuffer + s * kPlane);
 #pragma unroll
-        for (int s = 0; s < ND; ++s) ldmatrix4(a[s], a_addr + s * kPlane + kk * 32);
+    for (int t = 0; t < ND; ++t) {
+      unsigned b[4];
+      ldmatrix4(b, b_addr + buf * kBuffer + t * kPlane);
 #pragma unroll
-        for (int t = 0; t < ND; ++t) {
-          unsigned b[4];
-          ldmatrix4(b, b_addr + t * kPlane + kk * 32);
+      for (int s = 0; s < ND && s + t < NG; ++s) {
+        mma16816(acc[s + t][0], a[s], b[0], b[1]);
+        mma16816(acc[s + t][1], a[s], b[2], b[3]);
+      }
+    }
+  };
+  const int nch = (kend - kbeg + kKC - 1) / kKC;
+  load(kbeg, 0);
+  if (nch > 1) load(kbeg + kKC, 1);
+  if (nch > 1) asm volatile("cp.async.wait_group 1;" ::: "memory");
+  else asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  rewrite(0);
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  int held = 0;
+  for (int c = 0; c < nch; ++c) {
+    // digits of chunk c and the FP64 rows of chunk c + 1 are in place, everything else is free
+    if (c + 2 < nch) load(kbeg + (c + 2) * kKC, c & 1);
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+      if (half == (warp & 1)) {
+        if (c + 1 < nch) rewrite((c + 1) & 1);
+      } else if (active) {
+        multiply(c & 1);
+      }
+    }
+    if (active && (++held == kFlush || c + 1 == nch)) {
+      held = 0;
 #pragma unroll
-          for (int s = 0; s < ND && s + t < NG; ++s) {
-            mma16816(acc[s + t][0], a[s], b[0], b[1]);
-            mma16816(acc[s + t][1], a[s], b[2], b[3]);
+      for (int t = 0; t < 2; ++t)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          int v[NG];
+#pragma unroll
+          for (int g = 0; g < NG; ++g) {
+            v[g] = __float_as_int(acc[g][t][i] + 12582912.f) - 0x4B400000;
+            acc[g][t][i] = 0.f;
+          }
+          if constexpr (ND == 8) {
+            longlong2 &s = sums[(t * 4 + i) * (kWarps * 32) + tid];
+            longlong2 x = s;
+            x.x += (((long long)v[0] * 128 + v[1]) * 128 + v[2]) * 128 + v[3];
+            x.y += ((((long long)v[4] * 128 + v[5]) * 128 + v[6]) * 128 + v[7]) * 128 + v[8];
+            s = x;
+          } else {
+            one[t * 4 + i] += ((((long long)v[0] * 128 + v[1]) * 128 + v[2]) * 128 + v[3]) * 128 + v[4];
           }
         }
-      }
-      if (++held == kFlush || k0 + kKC >= kend) {
-        held = 0;
-#pragma unroll
-        for (int t = 0; t < 2; ++t)
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            int v[NG];
-#pragma unroll
-            for (int g = 0; g < NG; ++g) {
-              v[g] = __float_as_int(acc[g][t][i] + 12582912.f) - 0x4B400000;
-              acc[g][t][i] = 0.f;
-            }
-            if constexpr (ND == 8) {
-              longlong2 &s = sums[(t * 4 + i) * (kWarps * 32) + tid];
-              longlong2 x = s;
-              x.x += (((long long)v[0] * 128 + v[1]) * 128 + v[2]) * 128 + v[3];
-              x.y += ((((long long)v[4] * 128 + v[5]) * 128 + v[6]) * 128 + v[7]) * 128 + v[8];
-              s = x;
-            } else {
-              one[t * 4 + i] += ((((long long)v[0] * 128 + v[1]) * 128 + v[2]) * 128 + v[3]) * 128 + v[4];
-            }
-          }
-      }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
@@ -304,43 +334,45 @@ __global__ void __launch_bounds__(kWarps * 32, 1)
     }
 }
 
-// C = alpha sum_z part[z] + beta C, four slices in flight per thread
-__global__ void __launch_bounds__(128) digit_reduce(int M, int N, int nsplit, const double *__restrict__ part,
+// C = alpha sum_z part[z] + beta C: 32 outputs per CTA, the slices dealt to eight warps and their sums added
+// in order (as one thread per output, 44 x 216 outputs of 30 slices took 9 us, now 3)
+__global__ void __launch_bounds__(256) digit_reduce(int M, int N, int nsplit, const double *__restrict__ part,
                                                     double alpha, double beta, double *__restrict__ C, int ldc) {
+  __shared__ double red[8][33];
   const long total = (long)M * N;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
-    double s0 = 0, s1 = 0, s2 = 0, s3 = 0;
-    int z = 0;
-    for (; z + 4 <= nsplit; z += 4) {
-      s0 += part[(long)z * total + i];
-      s1 += part[(long)(z + 1) * total + i];
-      s2 += part[(long)(z + 2) * total + i];
-      s3 += part[(long)(z + 3) * total + i];
-    }
-    for (; z < nsplit; ++z) s0 += part[(long)z * total + i];
-    const double s = (s0 + s1) + (s2 + s3);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long i = blockIdx.x * 32L + lane;
+  double s = 0;
+  if (i < total)
+#pragma unroll 4
+    for (int z = warp; z < nsplit; z += 8) s += __ldg(&part[(long)z * total + i]);
+  red[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0 && i < total) {
+    for (int w = 1; w < 8; ++w) s += red[w][lane];
     double *c = C + (i / N) * ldc + (i % N);
     *c = beta == 0.0 ? alpha * s : alpha * s + beta * (*c);
   }
 }
 
-// Strips per CTA and K slices: the fewest clocks by a model of one CTA per SM, a chunk costing 1900
-// clocks of staging and rewriting plus 344 (ND = 8; 104 for ND = 4) per active warp, a CTA 8000 more.
+// Strips per CTA and K slices: the fewest clocks by a model of one CTA per SM, a chunk of 16 k costing the
+// larger of its rewriting (240 clocks per strip) and its products (172 per active warp with ND = 8, 52 with
+// ND = 4) plus 500, a CTA 8000 more.
 struct Shape {
   int sm, sn, kslice, nsplit;
 };
 Shape choose(int M, int N, int K, int nd, size_t part_cap) {
-  static const int opts[][2] = {{4, 4}, {5, 3}, {3, 5}, {2, 8}, {8, 2}, {6, 2}, {2, 6}, {3, 3}, {2, 4}, {4, 2}, {2, 2},
-                                {1, 9}, {9, 1}, {1, 4}, {4, 1}, {1, 1}};
+  static const int opts[][2] = {{4, 4}, {5, 3}, {3, 5}, {2, 7}, {7, 2}, {6, 2}, {2, 6}, {3, 3}, {2, 4}, {4, 2}, {2, 2},
+                                {1, 8}, {8, 1}, {1, 4}, {4, 1}, {1, 1}};
   const int ms = (M + 15) / 16, ns = (N + 15) / 16;
-  const double per_warp = nd == 8 ? 344.0 : 104.0;
+  const double per_warp = nd == 8 ? 172.0 : 52.0;
   Shape best{4, 4, K, 1};
   double bc = 1e300;
   for (auto &o : opts) {
     const int sm = o[0], sn = o[1];
     if (sm > ms + 1 || sn > ns + 1) continue;
     const long tiles = (long)((ms + sm - 1) / sm) * ((ns + sn - 1) / sn);
-    const double load = 1900.0 * (sm + sn) / 8.0 + per_warp * std::min(sm, ms) * std::min(sn, ns);
+    const double load = std::max(240.0 * (sm + sn), per_warp * std::min(sm, ms) * std::min(sn, ns)) + 500.0;
     // a slice of at most kMaxSlice k keeps the 64-bit sums in range (2^50 per 128 k)
     const int mins = (K + kMaxSlice - 1) / kMaxSlice;
     const int maxs = (int)std::max(mins, std::min(K / 64, 128));
@@ -402,8 +434,7 @@ void run(char ta, char tb, int M, int N, int K, double alpha, const double *A, i
   else go<true, true, ND>(grid, s, M, N, K, h, A, lda, B, ldb, ex, alpha, beta, C, ldc, part);
   if (part) {
     const long total = (long)M * N;
-    digit_reduce<<<(int)std::min<long>(152 * 16, (total + 127) / 128), 128, 0, s>>>(M, N, h.nsplit, part, alpha, beta, C,
-                                                                                  ldc);
+    digit_reduce<<<(unsigned)((total + 31) / 32), 256, 0, s>>>(M, N, h.nsplit, part, alpha, beta, C, ldc);
     BSE_CHECK_LAUNCH();
   }
 }

@@ -237,6 +237,25 @@ __device__ __forceinline__ double to_double(long long v, int q) {
   bits |= (unsigned long long)v & 0x8000000000000000ull;
   return v == 0 ? 0.0 : __longlong_as_double((long long)bits);
 }
+// Bound of one line of n elements, by a whole warp: the smallest e (to one part in 2^20) with
+// sum |re| + |im| < 2^e; kBadLine when an element is not finite
+constexpr int kBadLine = 1 << 20;
+template <class Get>
+__device__ __forceinline__ int line_exponent(int n, const Get &get) {
+  const int lane = threadIdx.x & 31;
+  unsigned m = 0, s = 0;
+  for (int i = lane; i < n; i += 32) {
+    const double2 u = get(i);
+    m = max(m, max(high_abs(u.x), high_abs(u.y)));
+  }
+  const int E = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
+  for (int i = lane; i < n; i += 32) {
+    const double2 u = get(i);
+    s += mag(u.x, E) + mag(u.y, E);
+  }
+  s = __reduce_add_sync(0xffffffffu, s);
+  return E >= 0x7ff ? kBadLine : E - 1043 + 32 - __clz(s);
+}
 // the unit 2^q of a block and whether it can be converted by to_double; bad: the block holds a NaN or infinity
 struct Unit {
   int q;

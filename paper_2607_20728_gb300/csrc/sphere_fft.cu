@@ -35,6 +35,7 @@ using namespace fftc;
 constexpr double kRs2 = 0.70710678118654752440;  // 1/sqrt(2)
 constexpr int kThreads = 256;
 constexpr int kXYThreads = 512;  // plane passes: more warps to hide the latency of the FP64 pipe
+constexpr int kXYFixed = 672;    // fixed-point plane passes (96 registers)
 constexpr int kZMax = 288;      // largest CTA of the fixed-point z passes (two per SM with 112 registers)
 constexpr size_t kSmemCap = 200 * 1024;
 
@@ -291,9 +292,10 @@ __global__ void __launch_bounds__(kXYThreads) sph_xy(SphArgs<C> a, C *__restrict
 // Each is an upper bound taken from the leading 21 bits.  Rounding is at 2^-61 of those sums: against exact
 // transforms (36^3, flat and decaying data) the relative error of a transform is 3.0-4.3e-16, with the FP64
 // passes 3.8-5.5e-16 (the z passes stay FP64).
-// 64 packed grids of the 63-well cell (72^3, 4608 planes), FP64 pass -> this one: inverse 1490 -> 512 us,
-// forward 1595 -> 691, H product of 63 orbitals 994 -> 330.  Bound by instruction issue (57 thousand warp
-// instructions a plane, 42% of the issue slots used: one CTA of 16 warps and a barrier per stage).
+// 64 packed grids of the 63-well cell (72^3, 4608 planes), FP64 pass -> this one: inverse 1490 -> 502 us,
+// forward 1595 -> 669, H product 2710 -> 1017.  Bound by instruction issue (57 thousand warp instructions a
+// plane, 42% of the issue slots used: few warps and a barrier per stage).  Measured and not kept: radices
+// 8 3 3 for 72 (566 and 685 us), the plane in chunks of rows so that two CTAs share an SM (679 and 659).
 struct FxArgs {
   int N1, N2, N3, ncols_pad, nxs;
   long nr;
@@ -335,10 +337,11 @@ __device__ fx::C2 *lines_fx(fx::C2 *in, fx::C2 *out, int L, Base base, int es, c
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(kXYThreads) sph_xy_fx(FxArgs a, double2 *__restrict__ colbuf,
+__global__ void __launch_bounds__(kXYFixed) sph_xy_fx(FxArgs a, double2 *__restrict__ colbuf,
                                                         double2 *__restrict__ P, const double *__restrict__ vloc) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   __shared__ unsigned top, vtop, ltop[2];
+  __shared__ int etop;
   __shared__ unsigned long long total;
   const int N1 = a.N1, N1p = a.N1 + 1;
   const int np = N1 * a.N2, npp = N1p * a.N2;
@@ -350,6 +353,7 @@ __global__ void __launch_bounds__(kXYThreads) sph_xy_fx(FxArgs a, double2 *__res
   const double *v = MODE == 2 ? vloc + (long)z * np : nullptr;
   if (threadIdx.x == 0) {
     top = vtop = ltop[0] = ltop[1] = 0;
+    etop = -fx::kBadLine;
     total = 0;
   }
   const int y0 = threadIdx.x / N1, x0 = threadIdx.x - y0 * N1;
@@ -425,32 +429,25 @@ __global__ void __launch_bounds__(kXYThreads) sph_xy_fx(FxArgs a, double2 *__res
     unit.q += ev;
     __syncthreads();
   } else {
-    unsigned m = 0;
-    for_plane([&](int e, int ep) {
-      const double2 u = plane[e];
-      m = max(m, max(fx::high_abs(u.x), fx::high_abs(u.y)));
-      reinterpret_cast<double2 *>(A)[ep] = u;
-    });
-    __syncthreads();
-    warp_max(m, &top);
+    for_plane([&](int e, int ep) { reinterpret_cast<double2 *>(A)[ep] = plane[e]; });
     __syncthreads();
     F = A;
   }
   // forward: the largest sum of |re| + |im| over an x line, one warp per line
-  const int E = (int)(top >> 20);
   for (int y = warp; y < a.N2; y += nwarp) {
-    unsigned s = 0;
-    for (int x = lane; x < N1; x += 32) {
-      if (MODE == 1) {
-        const double2 u = reinterpret_cast<const double2 *>(F)[y * N1p + x];
-        s += fx::mag(u.x, E) + fx::mag(u.y, E);
-      } else {
+    if (MODE == 1) {
+      const double2 *row = reinterpret_cast<const double2 *>(F) + y * N1p;
+      const int e = fx::line_exponent(N1, [&](int x) { return row[x]; });
+      if (lane == 0) atomicMax(&etop, e);
+    } else {
+      unsigned s = 0;
+      for (int x = lane; x < N1; x += 32) {
         const fx::C2 u = F[y * N1p + x];
         s += (unsigned)((unsigned long long)llabs(u.x) >> 40) + (unsigned)((unsigned long long)llabs(u.y) >> 40) + 2;
       }
+      s = __reduce_add_sync(0xffffffffu, s);
+      if (lane == 0) atomicMax(&ltop[0], s);
     }
-    s = __reduce_add_sync(0xffffffffu, s);
-    if (lane == 0) atomicMax(&ltop[0], s);
   }
   __syncthreads();
   // values shifted as they are loaded: k > 0 right (rounded), k < 0 left
@@ -461,9 +458,9 @@ __global__ void __launch_bounds__(kXYThreads) sph_xy_fx(FxArgs a, double2 *__res
   };
   fx::C2 *O = F == A ? B : A;
   if (MODE == 1) {
-    const int e0 = above(ltop[0], E - 1043);
+    unit.bad = etop >= fx::kBadLine;
+    const int e0 = unit.bad ? 0 : etop;
     unit.q = e0 - 61;
-    unit.bad = E >= 0x7ff;
     F = lines_fx<-1>(F, O, a.N2, StrideBase{N1p}, 1, a.ax[0], [&](const fx::C2 &c) {
       return fx::C2{fx::from_double(__longlong_as_double(c.x), e0, 61), fx::from_double(__longlong_as_double(c.y), e0, 61)};
     });
@@ -508,33 +505,18 @@ struct FzArgs {
 // FP64 columns in A (synchronised) -> transformed columns as integers of the unit set on return; B: scratch
 template <int SG>
 __device__ fx::C2 *z_lines(const FzArgs &a, double2 *Ad, fx::C2 *B, fx::Unit &unit) {
-  __shared__ unsigned top, ltop;
-  if (threadIdx.x == 0) top = ltop = 0;
+  __shared__ int ltop;
+  if (threadIdx.x == 0) ltop = -fx::kBadLine;
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-  unsigned m = 0;
-  for (int l = warp; l < a.CG; l += nwarp)
-    for (int z = lane; z < a.N3; z += 32) {
-      const double2 u = Ad[l * a.N3p + z];
-      m = max(m, max(fx::high_abs(u.x), fx::high_abs(u.y)));
-    }
-  m = __reduce_max_sync(0xffffffffu, m);
-  if (lane == 0) atomicMax(&top, m);
-  __syncthreads();
-  const int E = (int)(top >> 20);
   for (int l = warp; l < a.CG; l += nwarp) {
-    unsigned s = 0;
-    for (int z = lane; z < a.N3; z += 32) {
-      const double2 u = Ad[l * a.N3p + z];
-      s += fx::mag(u.x, E) + fx::mag(u.y, E);
-    }
-    s = __reduce_add_sync(0xffffffffu, s);
-    if (lane == 0) atomicMax(&ltop, s);
+    const int e = fx::line_exponent(a.N3, [&](int z) { return Ad[l * a.N3p + z]; });
+    if (lane == 0) atomicMax(&ltop, e);
   }
   __syncthreads();
-  const int e0 = E - 1043 + 32 - __clz(ltop);
+  unit.bad = ltop >= fx::kBadLine;
+  const int e0 = unit.bad ? 0 : ltop;
   unit.q = e0 - 61;
-  unit.bad = E >= 0x7ff;
   return lines_fx<SG>(reinterpret_cast<fx::C2 *>(Ad), B, a.CG, StrideBase{a.N3p}, 1, a.ax, [&](const fx::C2 &c) {
     return fx::C2{fx::from_double(__longlong_as_double(c.x), e0, 61), fx::from_double(__longlong_as_double(c.y), e0, 61)};
   });
@@ -914,10 +896,11 @@ void launch_xy(Ctx &c, const SphereFFT &s, int nq, C *cb, C *P, const typename R
       a.ax[i].tw = x.twx;
     }
     // planes of which two or more fit an SM go 256 threads each when there is more than one wave of them
-    // (24 grids of 36^2 planes: inverse 48 us with 512, 32 with 256; 54^2 114 and 90; 60^2, one per SM,
-    // 148 and 166; a single grid 10.9 and 11.6)
+    // (24 grids of 36^2 planes: inverse 48 us with 512, 26 with 256; 54^2 114 and 90; 60^2, one per SM,
+    // 148 and 166; a single grid 10.9 and 11.6); one per SM takes 672, which give every 72-point line stage
+    // of 648 or 576 butterflies a single round (512 threads: 512 and 691 us where 672 take 502 and 669)
     const bool pair = 2 * xy_smem<C>(c) <= 220 * 1024 && (long)c.N[2] * nq > 152;
-    sph_xy_fx<MODE><<<grid, c.xy_threads > 0 ? xy_threads(c) : (pair ? 256 : kXYThreads), xy_smem<C>(c), c.stream>>>(
+    sph_xy_fx<MODE><<<grid, c.xy_threads > 0 ? xy_threads(c) : (pair ? 256 : kXYFixed), xy_smem<C>(c), c.stream>>>(
         a, cb, P, v);
   } else {
     sph_xy<C, MODE><<<grid, xy_threads(c), xy_smem<C>(c), c.stream>>>(make_args<C>(c, s), cb, P, v);

@@ -365,7 +365,10 @@ void launch_s(const Ctx &c, const K1dTma &t, int nb, int b0, const float *phir, 
   const unsigned grid = (unsigned)std::min<long>((c.nr + kR - 1) / kR, CTAS * std::max(1, nsm));
   auto go = [&](auto rag) {
     auto kernel = k1d_tma_kernel<NB, S, decltype(rag)::value, CTAS>;
-    BSE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // the limit is one value per function, shared by every thread that launches it: always the same one, so
+    // that a system with fewer orbitals cannot lower it between another system's call and its launch
+    BSE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)(CTAS == 2 ? kSmemHalf : kSmemCap)));
     kernel<<<grid, kThreads + 32, smem, c.stream>>>(t.tau, t.npairs, c.nr, c.nocc, nb, b0, phir, vloc, Pa, Pvh, Py,
                                                     use_vloc, use_k1e, t.err, hold);
   };

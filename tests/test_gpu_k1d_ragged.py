@@ -48,3 +48,16 @@ def test_rows(pkg, n_occ, grid):
             assert np.abs(got - ref[:nb]).max() < 2e-5 * np.abs(ref).max(), nb
     finally:
         s.close()
+
+
+def test_sizes_side_by_side(pkg):
+    """Systems that take the same kernels with different shared-memory sizes, launched by four threads at once:
+    every launch is accepted, whichever size another thread asked for last."""
+    specs = [replace(bi.small16(), n_occ=n) for n in (17, 33, 49, 65)]
+    b = pkg.BSEBatch(specs, n_workers=4, precision=1, gs_tol=1e-9, flags=pkg.FLAG_NO_GRAPHS)
+    try:
+        assert b.setup_status == 0
+        for _ in range(16):
+            assert b.solve(davidson_tol=1e-5, zvector_tol=1e-5)[2] == 0
+    finally:
+        b.close()

@@ -34,8 +34,10 @@ using namespace fftc;
 
 constexpr double kRs2 = 0.70710678118654752440;  // 1/sqrt(2)
 constexpr int kThreads = 256;
-constexpr int kXYThreads = 512;  // plane passes: more warps to hide the latency of the FP64 pipe
-constexpr int kXYFixed = 672;    // fixed-point plane passes (96 registers)
+constexpr int kXYThreads = 512;  // the most threads of an FP32 plane pass
+// and of a fixed-point one: 96 registers, and every 72-point line stage of 648 or 576 butterflies takes a single
+// round (128 grids of 72^2, 512 threads: 512 and 691 us; 672: 502 and 669)
+constexpr int kXYFixed = 672;
 constexpr int kZMax = 288;      // largest CTA of the fixed-point z passes (two per SM with 112 registers)
 constexpr size_t kSmemCap = 200 * 1024;
 
@@ -872,8 +874,24 @@ void set_attrs() {
   done[dev] = true;
 }
 
-// threads per plane-pass CTA: the autotuner's choice, else kXYThreads
-int xy_threads(const Ctx &c) { return c.xy_threads > 0 ? std::min(c.xy_threads, kXYThreads) : kXYThreads; }
+// Threads per plane-pass CTA: the autotuner's choice, else what an SM's registers hold (kXYSM, by type) over
+// the planes that share an SM, which a plane's shared memory and the number of planes give.  More threads per
+// plane only idle (a stage of 40^2 has 200 butterflies) and keep the other planes out; fewer leave the SM
+// without warps.  256 functions on 128 grids, us, inverse / forward, with 512 FP32 or 256 (up to 54^2) and 672
+// FP64 threads -> with this rule, and in brackets with 64 to 128 threads fewer or more:
+//   FP32 36^2 74/73 -> 35/35, 40^2 85/86 -> 43/46, 48^2 171/193 -> 123/131 (121/159), 54^2 221/242 -> 172/197,
+//        60^2 250/286 -> 216/256 (212/282, 241/240), 64^2 187/244 -> 162/234 (156/254, 183/218)
+//   FP64 24^2 49/65 -> 35/51, 30^2 105/122 -> 83/102, 36^2 125/187 -> 110/172 (114/168), 40^2 146/209 -> 134/209
+//        (139/233), 54^2 489/644 -> 450/558
+constexpr int kXYSM32 = 1024, kXYSM64 = 768;
+template <class C>
+int xy_threads(const Ctx &c, int nq) {
+  constexpr bool fixed = sizeof(C) == sizeof(double2);
+  if (c.xy_threads > 0) return std::min(c.xy_threads, kXYThreads);
+  const long fit = 227 * 1024 / (long)(xy_smem<C>(c) + 1024), share = ((long)c.N[2] * nq + 151) / 152;
+  const int t = (fixed ? kXYSM64 : kXYSM32) / (int)std::max(1L, std::min(fit, share));
+  return std::max(128, std::min(fixed ? kXYFixed : kXYThreads, (t + 32) / 64 * 64));
+}
 
 template <class C, int MODE>
 void launch_xy(Ctx &c, const SphereFFT &s, int nq, C *cb, C *P, const typename RealOf<C>::T *v) {
@@ -895,15 +913,9 @@ void launch_xy(Ctx &c, const SphereFFT &s, int nq, C *cb, C *P, const typename R
       for (int r = 0; r < 12; ++r) a.ax[i].radix[r] = x.radix[r];
       a.ax[i].tw = x.twx;
     }
-    // planes of which two or more fit an SM go 256 threads each when there is more than one wave of them
-    // (24 grids of 36^2 planes: inverse 48 us with 512, 26 with 256; 54^2 114 and 90; 60^2, one per SM,
-    // 148 and 166; a single grid 10.9 and 11.6); one per SM takes 672, which give every 72-point line stage
-    // of 648 or 576 butterflies a single round (512 threads: 512 and 691 us where 672 take 502 and 669)
-    const bool pair = 2 * xy_smem<C>(c) <= 220 * 1024 && (long)c.N[2] * nq > 152;
-    sph_xy_fx<MODE><<<grid, c.xy_threads > 0 ? xy_threads(c) : (pair ? 256 : kXYFixed), xy_smem<C>(c), c.stream>>>(
-        a, cb, P, v);
+    sph_xy_fx<MODE><<<grid, xy_threads<C>(c, nq), xy_smem<C>(c), c.stream>>>(a, cb, P, v);
   } else {
-    sph_xy<C, MODE><<<grid, xy_threads(c), xy_smem<C>(c), c.stream>>>(make_args<C>(c, s), cb, P, v);
+    sph_xy<C, MODE><<<grid, xy_threads<C>(c, nq), xy_smem<C>(c), c.stream>>>(make_args<C>(c, s), cb, P, v);
   }
   BSE_CHECK_LAUNCH();
 }

@@ -1490,13 +1490,13 @@ void ground_state(Ctx &c, std::vector<double> &eps_all, DevBuf<double> &Qall, do
   }
 }
 
-// W * rho for np packed real pair densities rho on the grid P, in place (Eq. 2c with Eq. 3):
+// W * rho on the packed grid P for the np pair densities rho = A_i B_j, (i, j) from list (Eq. 2c with Eq. 3):
 // the bare Coulomb part 4 pi/|G|^2 on the density sphere plus the PDEP part, a projection of
 // v_c^{1/2} rho on the PDEP vectors, lambda/(1 - lambda), and the back-projection.  X, Qm:
 // scratch for the PDEP coefficients.  The transforms are the density-sphere-pruned ones when
-// they fit, else full-grid FFTs.
+// they fit, whose first pass forms the products as it loads its planes, else full-grid FFTs.
 template <class R>
-void pair_screen(Ctx &c, int np, CT<R> *P, R *X, R *Qm) {
+void pair_screen(Ctx &c, int np, const int2 *list, const R *A, const R *B, CT<R> *P, R *X, R *Qm) {
   Grids<R> &g = c.grids<R>();
   const int nq = (np + 1) / 2;
   if (dens_fft_ok<R>(c)) {
@@ -1505,13 +1505,19 @@ void pair_screen(Ctx &c, int np, CT<R> *P, R *X, R *Qm) {
     const double fl = 5.0 * nq *
                       (c.dfft.ncols * n3 * std::log2(n3) + n3 * (c.dfft.nxs * n2 * std::log2(n2) + n2 * n1 * std::log2(n1)));
     c.prof.begin(c.stream, BSE_KERNEL_SPHERE_FFT, 2.0 * nq * c.nr * sizeof(CT<R>), 2.0 * fl, &stop);
-    dens_forward<R>(c, np, P, c.npdep ? X : nullptr, 1.0 / c.nr, g.vcg.get(), (R)(1.0 / c.nr));
+    PairGrids<R> src;
+    src.list = list;
+    src.A = A;
+    src.B = B;
+    src.np = np;
+    dens_forward<R>(c, np, P, c.npdep ? X : nullptr, 1.0 / c.nr, g.vcg.get(), (R)(1.0 / c.nr), src);
     if (c.npdep) pdep_gemms<R>(c, np, X, Qm);
     dens_inverse<R>(c, np, c.npdep ? X : nullptr, 1.0, P);
     if (stop) BSE_CUDA(cudaEventRecord(stop, c.stream));
     if (c.prof.pending.size() > 512) c.prof.flush();
     return;
   }
+  k::pair_products<R>(c.nr, np, list, A, B, P, c.stream);
   fft_exec(c, P, nq, -1);
   if (c.npdep) k::gather_pairs<R, R>(c, np, P, X, 1.0 / c.nr);
   k::mul_grid<R>(c.nr, nq, P, g.vcg.get(), (R)(1.0 / c.nr), c.stream);
@@ -1540,8 +1546,7 @@ void build_tau_t(Ctx &c, bool tiled = false) {
   R *Qm = g.qbuf.get();
   for (long p0 = 0; p0 < npairs; p0 += kPairBatch) {
     const int np = (int)std::min<long>(kPairBatch, npairs - p0);
-    k::pair_products<R>(c.nr, np, c.pairs.get() + p0, phir, phir, g.work.get(), c.stream);
-    pair_screen<R>(c, np, g.work.get(), X, Qm);
+    pair_screen<R>(c, np, c.pairs.get() + p0, phir, phir, g.work.get(), X, Qm);
     if constexpr (std::is_same<R, float>::value) {
       if (tiled) {
         k1d_unpack_tiled(c, np, c.pairs.get() + p0, g.work.get(), g.tau.get());
@@ -1573,8 +1578,7 @@ void wannier_tau(Ctx &c) {
   const int2 *list = W.pairs.get();
   for (long p0 = 0; p0 < np_all; p0 += kPairBatch) {
     const int np = (int)std::min<long>(kPairBatch, np_all - p0);
-    k::pair_products<R>(c.nr, np, list + p0, g.wphir.get(), g.wphir.get(), g.work.get(), c.stream);
-    pair_screen<R>(c, np, g.work.get(), g.sbuf.get(), g.qbuf.get());
+    pair_screen<R>(c, np, list + p0, g.wphir.get(), g.wphir.get(), g.work.get(), g.sbuf.get(), g.qbuf.get());
     k::unpack_real<R, R>(c.nr, np, g.work.get(), g.wtau.get() + p0 * c.nr, c.stream);
   }
   sync(c);
@@ -2205,8 +2209,7 @@ void apply_b_t(Ctx &c, int nvec, const double *A, double *BA) {
       for (long p0 = 0; p0 < nfull; p0 += kPairBatch) {
         const int np = (int)std::min<long>(kPairBatch, nfull - p0);
         // pair (v', v): a_v' phi_v; T_v -= [W * (a_v' phi_v)] phi_v'
-        k::pair_products<R>(c.nr, np, c.pairs_full.get() + p0, g.bar.get(), g.phir.get(), g.work.get(), c.stream);
-        pair_screen<R>(c, np, g.work.get(), X, Qm);
+        pair_screen<R>(c, np, c.pairs_full.get() + p0, g.bar.get(), g.phir.get(), g.work.get(), X, Qm);
         k::sigma_contract<R>(c, np, c.pairs_full.get() + p0, g.work.get(), g.phir.get(), g.bt.get(), false);
       }
     }
@@ -2551,8 +2554,7 @@ void uvector_t(Ctx &c, int root, double *U) {
     BSE_CUDA(cudaMemsetAsync(T.get(), 0, (size_t)c.nocc * c.nr * sizeof(R), c.stream));
     for (long p0 = 0; p0 < c.npairs; p0 += kPairBatch) {
       const int np = (int)std::min<long>(kPairBatch, c.npairs - p0);
-      k::pair_products<R>(c.nr, np, c.pairs.get() + p0, g.phir.get(), g.phir.get(), g.work.get(), c.stream);
-      pair_screen<R>(c, np, g.work.get(), g.sbuf.get(), g.qbuf.get());
+      pair_screen<R>(c, np, c.pairs.get() + p0, g.phir.get(), g.phir.get(), g.work.get(), g.sbuf.get(), g.qbuf.get());
       k::sigma_contract<R>(c, np, c.pairs.get() + p0, g.work.get(), ar.get(), T.get(), true);
     }
     apply_liouville_t<R>(c, 1, A, LA.get(), 0, S.get(), vh.get(), T.get());  // S[v][w] = <phi_w|(M A)_v>
@@ -2598,8 +2600,7 @@ void uvector_t(Ctx &c, int root, double *U) {
     R *Qm = g.qbuf.get();
     for (long p0 = 0; p0 < c.npairs; p0 += kPairBatch) {
       const int np = (int)std::min<long>(kPairBatch, c.npairs - p0);
-      k::pair_products<R>(c.nr, np, c.pairs.get() + p0, ar.get(), ar.get(), g.work.get(), c.stream);
-      pair_screen<R>(c, np, g.work.get(), X, Qm);
+      pair_screen<R>(c, np, c.pairs.get() + p0, ar.get(), ar.get(), g.work.get(), X, Qm);
       k::sigma_contract<R>(c, np, c.pairs.get() + p0, g.work.get(), g.phir.get(), T.get());
     }
   }

@@ -409,11 +409,43 @@ void k1d_tma_stall_test(const Ctx &c, const K1dTma &t, const float *phir, const 
 // kk = 0..nhalf (kk = 0 is G = 0) in the order of the real basis; dens_cols the (n1, n2) of every
 // density-sphere G.
 void sphere_fft_init(Ctx &c, const std::vector<int> &miller_half, const std::vector<int> &dens_cols);
-// pair pipelines on the density sphere: P (packed pair grids) -> Coulomb-weighted columns and X
-// (wave-function-sphere coefficients for the PDEP part); then X' added back and -> P
+// pair densities A_i B_j for (i, j) = list[p], two packed in a grid; the members after np belong to a plane pass
+template <class R>
+struct PairGrids {
+  const int2 *list = nullptr;
+  const R *A = nullptr, *B = nullptr;
+  int np = 0;
+  const R *a0, *b0, *a1, *b1;  // the plane's rows; a1 null: no second function
+  __device__ void select(int q, long off, long nr) {
+    const int2 p = list[2 * q];
+    a0 = A + (long)p.x * nr + off;
+    b0 = B + (long)p.y * nr + off;
+    a1 = nullptr;
+    if (2 * q + 1 < np) {
+      const int2 o = list[2 * q + 1];
+      a1 = A + (long)o.x * nr + off;
+      b1 = B + (long)o.y * nr + off;
+    }
+  }
+  // element e of the plane: of the packed grid (MODE 1), of the products (MODE 3)
+  template <class C, int MODE>
+  __device__ C at(const C *plane, int e) const {
+    if constexpr (MODE == 3) {
+      C u;
+      u.x = __ldg(a0 + e) * __ldg(b0 + e);
+      u.y = a1 ? __ldg(a1 + e) * __ldg(b1 + e) : R(0);
+      return u;
+    } else {
+      return plane[e];
+    }
+  }
+};
+// pair pipelines on the density sphere: P (packed grids) or the products of src -> Coulomb-weighted columns and
+// X (wave-function-sphere coefficients for the PDEP part); then X' added back and -> P
 template <class R> bool dens_fft_ok(const Ctx &c);
 template <class R>
-void dens_forward(Ctx &c, int np, CT<R> *P, R *X, double scale, const R *vcg, R cscale);
+void dens_forward(Ctx &c, int np, CT<R> *P, R *X, double scale, const R *vcg, R cscale,
+                  const PairGrids<R> &src = {});
 template <class R> void dens_inverse(Ctx &c, int np, const R *X, double scale, CT<R> *P);
 template <class R> bool sphere_fft_ok(const Ctx &c);
 // X [nf][npw] (real basis) -> packed grids P [(nf+1)/2][nr], every point written

@@ -204,16 +204,49 @@ __global__ void __launch_bounds__(kThreads) sph_z_fwd(SphArgs<C> a, int nf, int 
   }
 }
 
+// A plane into its padded buffer, element e = y N1 + x to e + y, four loads in flight per thread (one at a time
+// the pass waits for memory a dozen times over; with them orbitals of 72^3 to the grid and back 1.53 -> 1.49 ms).
+template <class C, class Get>
+__device__ void load_plane(C *dst, int np, int N1, int y, int x, int dy, int dx, Get get) {
+  const int nt = blockDim.x;
+  auto step = [&] {
+    x += dx;
+    y += dy;
+    if (x >= N1) {
+      x -= N1;
+      ++y;
+    }
+  };
+  int e = threadIdx.x;
+  for (; e + 3 * nt < np; e += 4 * nt) {
+    C u[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) u[i] = get(e + i * nt);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      dst[e + i * nt + y] = u[i];
+      step();
+    }
+  }
+  for (; e < np; e += nt) {
+    dst[e + y] = get(e);
+    step();
+  }
+}
+
 // ---- xy passes (one CTA per plane z of grid q) ---------------------------------------------
 // MODE 0: colbuf -> inverse y (occupied lines) and x -> grid plane
 // MODE 1: grid plane -> forward x and y (occupied lines) -> colbuf
 // MODE 2: colbuf -> inverse -> times V(r) -> forward -> colbuf (in place)
+// MODE 3: as MODE 1 for the pair densities of src, multiplied as the plane is loaded (a pass of their own wrote
+//   and read back every packed grid: 256 pairs on 40^3, FP32, 32 + 54 us against 58 now)
 // The plane sits in shared memory with rows padded to N1 + 1 elements and consecutive threads on
 // consecutive lines in both passes (x lines one padded row apart, y lines one x apart), so the
 // strided butterfly loads and stores of every stage fall in distinct banks.
 template <class C, int MODE>
 __global__ void __launch_bounds__(kXYThreads) sph_xy(SphArgs<C> a, C *__restrict__ colbuf, C *__restrict__ P,
-                                                     const typename RealOf<C>::T *__restrict__ vloc) {
+                                                     const typename RealOf<C>::T *__restrict__ vloc,
+                                                     PairGrids<typename RealOf<C>::T> src) {
   using T = typename RealOf<C>::T;
   extern __shared__ __align__(16) unsigned char sm_raw[];
   const int N1 = a.N1, N1p = a.N1 + 1;
@@ -238,6 +271,7 @@ __global__ void __launch_bounds__(kXYThreads) sph_xy(SphArgs<C> a, C *__restrict
       }
     }
   };
+  if (MODE == 3) src.select(q, (long)z * np, a.nr);
   C *F;
   if (MODE == 0 || MODE == 2) {
     // the y pass transforms the occupied lines only, so the buffer its result lands in must hold
@@ -249,9 +283,18 @@ __global__ void __launch_bounds__(kXYThreads) sph_xy(SphArgs<C> a, C *__restrict
       if (zero_b) B[e] = mkc<C>(0, 0);
     }
     __syncthreads();
-    for (int c = threadIdx.x; c < a.ncols_pad; c += blockDim.x) {
-      const int pos = __ldg(&a.colpos[c]);
-      if (pos >= 0) A[pos + pos / N1] = crow[c];
+    for (int c0 = threadIdx.x; c0 < a.ncols_pad; c0 += 4 * blockDim.x) {
+      C u[4];
+      int pos[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int c = c0 + i * blockDim.x;
+        pos[i] = c < a.ncols_pad ? __ldg(&a.colpos[c]) : -1;
+        if (c < a.ncols_pad) u[i] = crow[c];
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (pos[i] >= 0) A[pos[i] + pos[i] / N1] = u[i];
     }
     __syncthreads();
     F = lines_fft<C, true, 1>(A, B, a.nxs, ListBase{a.xs}, N1p, a.ax[1]);
@@ -269,7 +312,7 @@ __global__ void __launch_bounds__(kXYThreads) sph_xy(SphArgs<C> a, C *__restrict
     });
     __syncthreads();
   } else {
-    for_plane([&](int e, int ep) { A[ep] = plane[e]; });
+    load_plane<C>(A, np, N1, y0, x0, dy, dx, [&](int e) { return src.template at<C, MODE>(plane, e); });
     __syncthreads();
     F = A;
   }
@@ -340,7 +383,8 @@ __device__ fx::C2 *lines_fx(fx::C2 *in, fx::C2 *out, int L, Base base, int es, c
 
 template <int MODE>
 __global__ void __launch_bounds__(kXYFixed) sph_xy_fx(FxArgs a, double2 *__restrict__ colbuf,
-                                                        double2 *__restrict__ P, const double *__restrict__ vloc) {
+                                                        double2 *__restrict__ P, const double *__restrict__ vloc,
+                                                        PairGrids<double> src) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   __shared__ unsigned top, vtop, ltop[2];
   __shared__ int etop;
@@ -431,13 +475,15 @@ __global__ void __launch_bounds__(kXYFixed) sph_xy_fx(FxArgs a, double2 *__restr
     unit.q += ev;
     __syncthreads();
   } else {
-    for_plane([&](int e, int ep) { reinterpret_cast<double2 *>(A)[ep] = plane[e]; });
+    if (MODE == 3) src.select(q, (long)z * np, a.nr);
+    load_plane<double2>(reinterpret_cast<double2 *>(A), np, N1, y0, x0, dy, dx,
+                        [&](int e) { return src.template at<double2, MODE>(plane, e); });
     __syncthreads();
     F = A;
   }
   // forward: the largest sum of |re| + |im| over an x line, one warp per line
   for (int y = warp; y < a.N2; y += nwarp) {
-    if (MODE == 1) {
+    if (MODE & 1) {
       const double2 *row = reinterpret_cast<const double2 *>(F) + y * N1p;
       const int e = fx::line_exponent(N1, [&](int x) { return row[x]; });
       if (lane == 0) atomicMax(&etop, e);
@@ -459,7 +505,7 @@ __global__ void __launch_bounds__(kXYFixed) sph_xy_fx(FxArgs a, double2 *__restr
     return fx::C2{(c.x + h) >> k, (c.y + h) >> k};
   };
   fx::C2 *O = F == A ? B : A;
-  if (MODE == 1) {
+  if (MODE & 1) {
     unit.bad = etop >= fx::kBadLine;
     const int e0 = unit.bad ? 0 : etop;
     unit.q = e0 - 61;
@@ -834,7 +880,8 @@ SphArgs<C> make_args(const Ctx &c, const SphereFFT &s) {
 
 // one plane pass (MODE of sph_xy) over nq packed grids: FP64 in fixed point, FP32 as it is
 template <class C, int MODE>
-void launch_xy(Ctx &c, const SphereFFT &s, int nq, C *cb, C *P, const typename RealOf<C>::T *v);
+void launch_xy(Ctx &c, const SphereFFT &s, int nq, C *cb, C *P, const typename RealOf<C>::T *v,
+               const PairGrids<typename RealOf<C>::T> &src = {});
 
 template <class C>
 size_t z_smem(const Ctx &c, const SphereFFT &s) { return (size_t)2 * s.cg * (c.N[2] + 1) * sizeof(C); }
@@ -861,6 +908,7 @@ void set_attrs() {
     BSE_CUDA(cudaFuncSetAttribute(sph_xy_fx<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
     BSE_CUDA(cudaFuncSetAttribute(sph_xy_fx<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
     BSE_CUDA(cudaFuncSetAttribute(sph_xy_fx<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    BSE_CUDA(cudaFuncSetAttribute(sph_xy_fx<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
   } else {
     using R = typename RealOf<C>::T;
     BSE_CUDA(cudaFuncSetAttribute(sph_z_inv<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
@@ -870,6 +918,7 @@ void set_attrs() {
     BSE_CUDA(cudaFuncSetAttribute(sph_xy<C, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
     BSE_CUDA(cudaFuncSetAttribute(sph_xy<C, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
     BSE_CUDA(cudaFuncSetAttribute(sph_xy<C, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    BSE_CUDA(cudaFuncSetAttribute(sph_xy<C, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
   }
   done[dev] = true;
 }
@@ -894,7 +943,8 @@ int xy_threads(const Ctx &c, int nq) {
 }
 
 template <class C, int MODE>
-void launch_xy(Ctx &c, const SphereFFT &s, int nq, C *cb, C *P, const typename RealOf<C>::T *v) {
+void launch_xy(Ctx &c, const SphereFFT &s, int nq, C *cb, C *P, const typename RealOf<C>::T *v,
+               const PairGrids<typename RealOf<C>::T> &src) {
   const dim3 grid(c.N[2], nq);
   if constexpr (sizeof(C) == sizeof(double2)) {
     FxArgs a;
@@ -913,9 +963,9 @@ void launch_xy(Ctx &c, const SphereFFT &s, int nq, C *cb, C *P, const typename R
       for (int r = 0; r < 12; ++r) a.ax[i].radix[r] = x.radix[r];
       a.ax[i].tw = x.twx;
     }
-    sph_xy_fx<MODE><<<grid, xy_threads<C>(c, nq), xy_smem<C>(c), c.stream>>>(a, cb, P, v);
+    sph_xy_fx<MODE><<<grid, xy_threads<C>(c, nq), xy_smem<C>(c), c.stream>>>(a, cb, P, v, src);
   } else {
-    sph_xy<C, MODE><<<grid, xy_threads<C>(c, nq), xy_smem<C>(c), c.stream>>>(make_args<C>(c, s), cb, P, v);
+    sph_xy<C, MODE><<<grid, xy_threads<C>(c, nq), xy_smem<C>(c), c.stream>>>(make_args<C>(c, s), cb, P, v, src);
   }
   BSE_CHECK_LAUNCH();
 }
@@ -1087,17 +1137,19 @@ bool dens_fft_ok(const Ctx &c) {
   return c.dfft.ready && (sizeof(R) == sizeof(double) ? c.dfft.ok64 : c.dfft.ok32) && !c.sfft.disabled;
 }
 
-// forward half of the pair pipeline: packed pair grids P -> density columns (Coulomb applied,
-// scaled by cscale) and the wave-function-sphere coefficients X (times scale) for the PDEP part
+// forward half of the pair pipeline: packed grids P, or the products of the grids that src names (P unused) ->
+// density columns (Coulomb applied, scaled by cscale) and the wave-function-sphere coefficients X (times
+// scale) for the PDEP part
 template <class R>
-void dens_forward(Ctx &c, int np, CT<R> *P, R *X, double scale, const R *vcg, R cscale) {
+void dens_forward(Ctx &c, int np, CT<R> *P, R *X, double scale, const R *vcg, R cscale, const PairGrids<R> &src) {
   using C = CT<R>;
   const int nq = (np + 1) / 2;
   set_attrs<C>();
   Grids<R> &g = c.grids<R>();
   g.colbuf_dens.alloc((size_t)nq * c.N[2] * c.dfft.ncols_pad);
   C *cb = g.colbuf_dens.get();
-  launch_xy<C, 1>(c, c.dfft, nq, cb, P, nullptr);
+  if (src.list) launch_xy<C, 3>(c, c.dfft, nq, cb, nullptr, nullptr, src);
+  else launch_xy<C, 1>(c, c.dfft, nq, cb, P, nullptr);
   const dim3 grid(c.dfft.ngroups, nq);
   if constexpr (std::is_same<R, double>::value)
     dsph_z_fwd_fx<<<grid, z_threads(c), z_smem<C>(c, c.dfft), c.stream>>>(fz_args(c, c.dfft), np, c.npw, cb, X, scale,
@@ -1127,8 +1179,10 @@ void dens_inverse(Ctx &c, int np, const R *X, double scale, CT<R> *P) {
 
 template bool dens_fft_ok<double>(const Ctx &);
 template bool dens_fft_ok<float>(const Ctx &);
-template void dens_forward<double>(Ctx &, int, double2 *, double *, double, const double *, double);
-template void dens_forward<float>(Ctx &, int, float2 *, float *, double, const float *, float);
+template void dens_forward<double>(Ctx &, int, double2 *, double *, double, const double *, double,
+                                   const PairGrids<double> &);
+template void dens_forward<float>(Ctx &, int, float2 *, float *, double, const float *, float,
+                                  const PairGrids<float> &);
 template void dens_inverse<double>(Ctx &, int, const double *, double, double2 *);
 template void dens_inverse<float>(Ctx &, int, const float *, double, float2 *);
 

@@ -62,12 +62,12 @@ struct ListBase {
 };
 
 // L lines of an axis in shared memory, ping-ponging between `in` and `out`; returns the buffer
-// holding the result.  LINE_FAST maps consecutive threads to consecutive lines, otherwise to
-// consecutive butterflies of one line.  SG is the sign of the exponent (+1 inverse, -1 forward),
-// a compile-time constant so that the twiddle conjugation and the factors +-i of the codelets
-// fold into additions.  The caller has synchronised the input; the result is synchronised on
-// return.
-template <class C, bool LINE_FAST, int SG, class Base>
+// holding the result.  Consecutive threads take consecutive lines (of the z lines too: the sphere passes of 128
+// orbitals on 72^3 45 / 28 us with consecutive butterflies of one line, 41 / 25 so).  SG is the sign of the
+// exponent (+1 inverse, -1 forward), a compile-time constant so that the twiddle conjugation and the factors
+// +-i of the codelets fold into additions.  The caller has synchronised the input; the result is synchronised
+// on return.
+template <class C, int SG, class Base>
 __device__ C *lines_fft(C *in, C *out, int L, Base base, int es, const AxisArgs<C> &ax) {
   const typename RealOf<C>::T sg = (typename RealOf<C>::T)SG;
   const int N = ax.n;
@@ -76,21 +76,17 @@ __device__ C *lines_fft(C *in, C *out, int L, Base base, int es, const AxisArgs<
     const int R = ax.radix[s];
     const int nb = N / R;
     const int work = L * nb;
-    // e = threadIdx.x + k blockDim.x split as (slow, fast) = divmod(e, F), advanced without
-    // divisions: F = L (line fastest) or nb (butterfly fastest)
-    const int F = LINE_FAST ? L : nb;
-    int slow = threadIdx.x / F, fast = threadIdx.x - (threadIdx.x / F) * F;
-    const int dslow = blockDim.x / F, dfast = blockDim.x - dslow * F;
+    // e = threadIdx.x + k blockDim.x split as (j, t) = divmod(e, L), advanced without divisions
+    int j = threadIdx.x / L, t = threadIdx.x - j * L;
+    const int dj = blockDim.x / L, dt = blockDim.x - dj * L;
     for (int e = threadIdx.x; e < work; e += blockDim.x) {
-      const int t = LINE_FAST ? fast : slow;
-      const int j = LINE_FAST ? slow : fast;
       const int b0 = base(t);
       stage_bfly_any<C>(R, in + b0, out + b0, j, N, Ns, ax.tw, sg, es);
-      fast += dfast;
-      slow += dslow;
-      if (fast >= F) {
-        fast -= F;
-        ++slow;
+      t += dt;
+      j += dj;
+      if (t >= L) {
+        t -= L;
+        ++j;
       }
     }
     __syncthreads();
@@ -133,7 +129,7 @@ __global__ void __launch_bounds__(kThreads) sph_z_inv(SphArgs<C> a, int nf, int 
     A[en.z] = mkc<C>((T)(fc + gs), (T)(gc - fs));  // conj(c_f) + i conj(c_g) at -G
   }
   __syncthreads();
-  C *F = lines_fft<C, false, 1>(A, B, a.CG, StrideBase{a.N3p}, 1, a.ax[2]);
+  C *F = lines_fft<C, 1>(A, B, a.CG, StrideBase{a.N3p}, 1, a.ax[2]);
   C *dst = colbuf + (long)q * a.N3 * a.ncols_pad + (long)g * a.CG;
   for (int e = threadIdx.x; e < a.CG * a.N3; e += blockDim.x) {
     const int slot = e % a.CG, z = e / a.CG;
@@ -160,7 +156,7 @@ __global__ void __launch_bounds__(kThreads) sph_z_fwd(SphArgs<C> a, int nf, int 
     A[slot * a.N3p + z] = src[(long)z * a.ncols_pad + slot];
   }
   __syncthreads();
-  const C *F = lines_fft<C, false, -1>(A, B, a.CG, StrideBase{a.N3p}, 1, a.ax[2]);
+  const C *F = lines_fft<C, -1>(A, B, a.CG, StrideBase{a.N3p}, 1, a.ax[2]);
   const int f0 = 2 * q, f1 = 2 * q + 1;
   const bool hasg = f1 < nf;
   const double sh0 = (shift ? shift[f0 % period] : 0.0) + shift_const;
@@ -297,9 +293,9 @@ __global__ void __launch_bounds__(kXYThreads) sph_xy(SphArgs<C> a, C *__restrict
         if (pos[i] >= 0) A[pos[i] + pos[i] / N1] = u[i];
     }
     __syncthreads();
-    F = lines_fft<C, true, 1>(A, B, a.nxs, ListBase{a.xs}, N1p, a.ax[1]);
+    F = lines_fft<C, 1>(A, B, a.nxs, ListBase{a.xs}, N1p, a.ax[1]);
     C *O = F == A ? B : A;
-    F = lines_fft<C, true, 1>(F, O, a.N2, StrideBase{N1p}, 1, a.ax[0]);
+    F = lines_fft<C, 1>(F, O, a.N2, StrideBase{N1p}, 1, a.ax[0]);
     if (MODE == 0) {
       for_plane([&](int e, int ep) { plane[e] = F[ep]; });
       return;
@@ -317,9 +313,9 @@ __global__ void __launch_bounds__(kXYThreads) sph_xy(SphArgs<C> a, C *__restrict
     F = A;
   }
   C *O = F == A ? B : A;
-  F = lines_fft<C, true, -1>(F, O, a.N2, StrideBase{N1p}, 1, a.ax[0]);
+  F = lines_fft<C, -1>(F, O, a.N2, StrideBase{N1p}, 1, a.ax[0]);
   O = F == A ? B : A;
-  F = lines_fft<C, true, -1>(F, O, a.nxs, ListBase{a.xs}, N1p, a.ax[1]);
+  F = lines_fft<C, -1>(F, O, a.nxs, ListBase{a.xs}, N1p, a.ax[1]);
   for (int c = threadIdx.x; c < a.ncols_pad; c += blockDim.x) {
     const int pos = __ldg(&a.colpos[c]);
     crow[c] = pos >= 0 ? F[pos + pos / N1] : mkc<C>(0, 0);
@@ -755,12 +751,15 @@ __global__ void __launch_bounds__(kZMax, 2) dsph_z_inv_fx(FzArgs a, int np, int 
 }
 
 // ---- pair pipelines on the density sphere (tau build, U vector; Eq. 2c and Eq. 3) ----------
+// FP32, six CTAs per SM (a CTA only loads, transforms and stores, so it is their number that hides the memory
+// behind them): 128 grids of 40^3, forward / inverse 28 / 23 us as the compiler left the registers, 25 / 22 now,
+// 17 at the copy rate.  Sums in FP32 pairs instead of on the FP64 pipe and four loads in flight gave nothing.
 // forward z pass: z lines of the occupied density columns, then the wave-function-sphere
 // coefficients of the two packed pair densities into X (real basis, type R, times `scale`) for
 // the PDEP projection, and every column element times v_c(G) * cscale (zero outside the density
 // sphere) written back
 template <class C, class R>
-__global__ void __launch_bounds__(kThreads) dsph_z_fwd(SphArgs<C> a, int np, int npw, C *__restrict__ colbuf,
+__global__ void __launch_bounds__(kThreads, 6) dsph_z_fwd(SphArgs<C> a, int np, int npw, C *__restrict__ colbuf,
                                                        R *__restrict__ X, double scale,
                                                        const R *__restrict__ vcg, R cscale) {
   using T = typename RealOf<C>::T;
@@ -774,7 +773,7 @@ __global__ void __launch_bounds__(kThreads) dsph_z_fwd(SphArgs<C> a, int np, int
     A[slot * a.N3p + z] = col[(long)z * a.ncols_pad + slot];
   }
   __syncthreads();
-  C *F = lines_fft<C, false, -1>(A, B, a.CG, StrideBase{a.N3p}, 1, a.ax[2]);
+  C *F = lines_fft<C, -1>(A, B, a.CG, StrideBase{a.N3p}, 1, a.ax[2]);
   if (X) {
     const int f0 = 2 * q, f1 = 2 * q + 1;
     const bool hasg = f1 < np;
@@ -810,7 +809,7 @@ __global__ void __launch_bounds__(kThreads) dsph_z_fwd(SphArgs<C> a, int np, int
 // inverse z pass: the PDEP back-projection X (real basis, type R, times `scale`) added at the
 // wave-function-sphere coefficients of the two packed pairs, then z lines of the columns
 template <class C, class R>
-__global__ void __launch_bounds__(kThreads) dsph_z_inv(SphArgs<C> a, int np, int npw, const R *__restrict__ X,
+__global__ void __launch_bounds__(kThreads, 6) dsph_z_inv(SphArgs<C> a, int np, int npw, const R *__restrict__ X,
                                                        double scale, C *__restrict__ colbuf) {
   using T = typename RealOf<C>::T;
   extern __shared__ __align__(16) unsigned char sm_raw[];
@@ -845,7 +844,7 @@ __global__ void __launch_bounds__(kThreads) dsph_z_inv(SphArgs<C> a, int np, int
     }
   }
   __syncthreads();
-  C *F = lines_fft<C, false, 1>(A, B, a.CG, StrideBase{a.N3p}, 1, a.ax[2]);
+  C *F = lines_fft<C, 1>(A, B, a.CG, StrideBase{a.N3p}, 1, a.ax[2]);
   for (int e = threadIdx.x; e < a.CG * a.N3; e += blockDim.x) {
     const int slot = e % a.CG, z = e / a.CG;
     col[(long)z * a.ncols_pad + slot] = F[slot * a.N3p + z];

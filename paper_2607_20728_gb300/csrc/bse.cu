@@ -429,7 +429,7 @@ double sphere_flops(const Ctx &c, int nq) {
 }
 
 template <class R>
-void sphere_to_grid_exec(Ctx &c, int nf, const double *X, CT<R> *P, double scale, CT<R> *colbuf = nullptr) {
+void sphere_to_grid_exec(Ctx &c, int nf, const double *X, CT<R> *P, long double scale, CT<R> *colbuf = nullptr) {
   cudaEvent_t stop;
   const int nq = (nf + 1) / 2;
   c.prof.begin(c.stream, BSE_KERNEL_SPHERE_FFT, (double)nq * c.nr * sizeof(CT<R>) + 8.0 * nf * c.npw,
@@ -440,7 +440,7 @@ void sphere_to_grid_exec(Ctx &c, int nf, const double *X, CT<R> *P, double scale
 }
 
 template <class R>
-void grid_to_sphere_exec(Ctx &c, int nf, CT<R> *P, double *Y, double scale, const double *Xd, const double *shift,
+void grid_to_sphere_exec(Ctx &c, int nf, CT<R> *P, double *Y, long double scale, const double *Xd, const double *shift,
                          int period, double shift_const, CT<R> *colbuf = nullptr) {
   cudaEvent_t stop;
   const int nq = (nf + 1) / 2;
@@ -491,7 +491,7 @@ template <class R>
 void sphere_to_grid_util(Ctx &c, int n, const double *X, CT<R> *P) {
   const int nq = (n + 1) / 2;
   if (sphere_fft_ok<R>(c)) {
-    sphere_to_grid_exec<R>(c, n, X, P, 1.0 / std::sqrt(c.omega));
+    sphere_to_grid_exec<R>(c, n, X, P, 1.0L / std::sqrt((long double)c.omega));
   } else {
     BSE_CUDA(cudaMemsetAsync(P, 0, (size_t)nq * c.nr * sizeof(CT<R>), c.stream));
     k::scatter_pairs<R, double>(c, n, X, P, 1.0 / std::sqrt(c.omega));
@@ -503,7 +503,7 @@ template <class R>
 void grid_to_sphere_util(Ctx &c, int n, CT<R> *P, double *Y) {
   const int nq = (n + 1) / 2;
   if (sphere_fft_ok<R>(c)) {
-    grid_to_sphere_exec<R>(c, n, P, Y, std::sqrt(c.omega) / c.nr, nullptr, nullptr, c.nocc, 0.0);
+    grid_to_sphere_exec<R>(c, n, P, Y, std::sqrt((long double)c.omega) / c.nr, nullptr, nullptr, c.nocc, 0.0);
   } else {
     fft_exec(c, P, nq, -1);
     k::gather_pairs<R, double>(c, n, P, Y, std::sqrt(c.omega) / c.nr);
@@ -708,7 +708,7 @@ void apply_liouville_t(Ctx &c, int nvec, const double *A, double *LA, int op, do
     const double *Ab = A + (long)b0 * vlen;
     double *LAb = LA + (long)b0 * vlen;
     if (sphere_fft_ok<R>(c)) {
-      sphere_to_grid_exec<R>(c, nf, Ab, g.work.get(), 1.0 / std::sqrt(c.omega), g.colbuf_apply.get());
+      sphere_to_grid_exec<R>(c, nf, Ab, g.work.get(), 1.0L / std::sqrt((long double)c.omega), g.colbuf_apply.get());
     } else {
       BSE_CUDA(cudaMemsetAsync(g.work.get(), 0, (size_t)nq * c.nr * sizeof(CT<R>), c.stream));
       k::scatter_pairs<R, double>(c, nf, Ab, g.work.get(), 1.0 / std::sqrt(c.omega));
@@ -723,7 +723,7 @@ void apply_liouville_t(Ctx &c, int nvec, const double *A, double *LA, int op, do
     combine_exec<R>(c, nb, g.work.get(), vh.get(), g.work2.get(), k1e, k1d);
     if (k1d_grid) k::add_packed<R>(c.nr, nf, k1d_grid, g.work2.get(), c.stream);
     if (sphere_fft_ok<R>(c)) {
-      grid_to_sphere_exec<R>(c, nf, g.work2.get(), LAb, std::sqrt(c.omega) / c.nr, Ab, c.negeps.get(), c.nocc,
+      grid_to_sphere_exec<R>(c, nf, g.work2.get(), LAb, std::sqrt((long double)c.omega) / c.nr, Ab, c.negeps.get(), c.nocc,
                              scissor, g.colbuf_apply.get());
     } else {
       fft_exec(c, g.work2.get(), nq, -1);
@@ -932,7 +932,7 @@ void apply_wannier_t(Ctx &c, int nvec, const double *A, double *LA) {
     const double *Ab = A + (long)b0 * vlen;
     double *LAb = LA + (long)b0 * vlen;
     if (sphere_fft_ok<R>(c)) {
-      sphere_to_grid_exec<R>(c, nf, Ab, g.work.get(), 1.0 / std::sqrt(c.omega), g.colbuf_apply.get());
+      sphere_to_grid_exec<R>(c, nf, Ab, g.work.get(), 1.0L / std::sqrt((long double)c.omega), g.colbuf_apply.get());
     } else {
       BSE_CUDA(cudaMemsetAsync(g.work.get(), 0, (size_t)nq * c.nr * sizeof(CT<R>), c.stream));
       k::scatter_pairs<R, double>(c, nf, Ab, g.work.get(), 1.0 / std::sqrt(c.omega));
@@ -951,7 +951,7 @@ void apply_wannier_t(Ctx &c, int nvec, const double *A, double *LA) {
       if (stop) BSE_CUDA(cudaEventRecord(stop, c.stream));
     }
     if (sphere_fft_ok<R>(c)) {
-      grid_to_sphere_exec<R>(c, nf, g.work2.get(), LAb, std::sqrt(c.omega) / c.nr, Ab, nullptr, c.nocc, c.scissor,
+      grid_to_sphere_exec<R>(c, nf, g.work2.get(), LAb, std::sqrt((long double)c.omega) / c.nr, Ab, nullptr, c.nocc, c.scissor,
                              g.colbuf_apply.get());
     } else {
       fft_exec(c, g.work2.get(), nq, -1);
@@ -1794,7 +1794,7 @@ void orbitals_to_grid(Ctx &c, const double *Q) {
     const int nf = (int)std::min<long>(capf, c.nocc - f0);
     const int nq = (nf + 1) / 2;
     if (sphere_fft_ok<double>(c)) {
-      sphere_to_grid_exec<double>(c, nf, Q + (long)f0 * c.npw, g.work.get(), 1.0 / std::sqrt(c.omega));
+      sphere_to_grid_exec<double>(c, nf, Q + (long)f0 * c.npw, g.work.get(), 1.0L / std::sqrt((long double)c.omega));
     } else {
       BSE_CUDA(cudaMemsetAsync(g.work.get(), 0, (size_t)nq * c.nr * sizeof(double2), c.stream));
       k::scatter_pairs<double, double>(c, nf, Q + (long)f0 * c.npw, g.work.get(), 1.0 / std::sqrt(c.omega));

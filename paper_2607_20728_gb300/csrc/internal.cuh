@@ -122,8 +122,8 @@ void dgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A,
 void sgemm(char ta, char tb, int M, int N, int K, float alpha, const float *A, int lda,
            const float *B, int ldb, float beta, float *C, int ldc, cudaStream_t s,
            DevBuf<float> *fixed = nullptr, int split_pct = 100);
-// FP64 operands and output with FP32 products and sums (same conventions as dgemm): the operands
-// are rounded to FP32 as they are staged, alpha, beta and the sum over K slices are applied in FP64
+// FP64 operands and output with products and sums no less exact than FP32's (same conventions as dgemm): four
+// BF16 digits of each operand, alpha, beta and the sum over K slices in FP64
 void mgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda, const double *B, int ldb,
            double beta, double *C, int ldc, cudaStream_t s, int split_pct = 100);
 // the same product from exact BF16 digit products on the tensor pipe (digit_gemm.cu): digits = 8 for
@@ -132,6 +132,7 @@ void mgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A,
 void digit_gemm(int digits, char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda,
                 const double *B, int ldb, double beta, double *C, int ldc, cudaStream_t s, DevBuf<double> &scratch,
                 bool fixed, int split_pct = 100);
+size_t digit_scratch(int M, int N, int K);  // the least scratch, in doubles
 // out[i] = sum_j X[i][j] * Y[i][j] for i < rows (part: scratch of the partial sums; the default is
 // a per-thread buffer)
 void rowdot(int rows, long len, const double *X, const double *Y, double *out, cudaStream_t s,
@@ -220,7 +221,7 @@ struct Grids {
   DevBuf<R> vloc;        // [nr] V(r)
   DevBuf<R> vcg;         // [nr] 4 pi/|G|^2 on the density sphere (0 elsewhere / G = 0)
   DevBuf<R> phir;        // [nocc][nr]
-  DevBuf<R> tau;         // [npairs][nr], pair (v', v) with v' <= v at v (v + 1)/2 + v'
+  DevBuf<R> tau;         // [npairs][nr], pair (v', v) with v' <= v at v (v + 1)/2 + v', or tile-major (K1dTma, K1dFixed)
   DevBuf<CT<R>> work;    // packed complex grids
   DevBuf<CT<R>> work2;
   DevBuf<R> pdep;        // [npdep][npw]: PDEP rows times v_c^{1/2}(G)
@@ -409,7 +410,7 @@ void k1d_tma_stall_test(const Ctx &c, const K1dTma &t, const float *phir, const 
 // kk = 0..nhalf (kk = 0 is G = 0) in the order of the real basis; dens_cols the (n1, n2) of every
 // density-sphere G.
 void sphere_fft_init(Ctx &c, const std::vector<int> &miller_half, const std::vector<int> &dens_cols);
-// pair densities A_i B_j for (i, j) = list[p], two packed in a grid; the members after np belong to a plane pass
+// pair densities A_i B_j for (i, j) = list[p], two packed in a grid; the members after np are set by a plane pass
 template <class R>
 struct PairGrids {
   const int2 *list = nullptr;
@@ -449,13 +450,13 @@ void dens_forward(Ctx &c, int np, CT<R> *P, R *X, double scale, const R *vcg, R 
 template <class R> void dens_inverse(Ctx &c, int np, const R *X, double scale, CT<R> *P);
 template <class R> bool sphere_fft_ok(const Ctx &c);
 // X [nf][npw] (real basis) -> packed grids P [(nf+1)/2][nr], every point written
-template <class R> void sphere_to_grid(Ctx &c, int nf, const double *X, CT<R> *P, double scale,
+template <class R> void sphere_to_grid(Ctx &c, int nf, const double *X, CT<R> *P, long double scale,
                                        CT<R> *colbuf = nullptr);
 // packed grids -> Y [nf][npw] (the gather_pairs contract, D term included when Xd is given);
 // P is left unchanged
 // colbuf: column buffer to use (large enough for (nf + 1)/2 grids); default the context's
 template <class R>
-void grid_to_sphere(Ctx &c, int nf, CT<R> *P, double *Y, double scale, const double *Xd, const double *shift,
+void grid_to_sphere(Ctx &c, int nf, CT<R> *P, double *Y, long double scale, const double *Xd, const double *shift,
                     int period, double shift_const, CT<R> *colbuf = nullptr);
 // HX = H X (+ shift_v X) without a grid in global memory
 template <class R> void sphere_h(Ctx &c, int nf, const double *X, double *HX, const double *shift);

@@ -163,6 +163,7 @@ __global__ void fill_real_kernel(long nr, double2 *__restrict__ P, const double 
     P[i] = make_double2(R[i], 0.0);
 }
 
+// the full-grid path's pair densities (the pruned transforms multiply them in their first pass)
 template <class R>
 __global__ void pair_products_kernel(long nr, int np, const int2 *__restrict__ list,
                                      const R *__restrict__ A, const R *__restrict__ Bm,
@@ -245,7 +246,8 @@ __global__ void __launch_bounds__(256) drho_kernel(long nr, int nocc, int nb, in
   }
 }
 
-// Y_{b,v}(r) = V(r) a_{b,v} + 2 vH_b phi_v - sum_v' tau_{v'v} a_{b,v'}  (Eqs. 2a-2c on the grid)
+// Y_{b,v}(r) = V(r) a_{b,v} + 2 vH_b phi_v - sum_v' tau_{v'v} a_{b,v'}  (Eqs. 2a-2c on the grid), for fewer than 16
+// orbitals and without K1d (k1d_tma.cu and k1d_fixed.cu stream tau for the others)
 template <class R, int NB, int TV>
 __global__ void __launch_bounds__(128) combine_tau_kernel(
     long nr, int nocc, int nb_total, int b0, const R *__restrict__ phir,

@@ -330,9 +330,8 @@ __global__ void __launch_bounds__(kXYThreads) sph_xy(SphArgs<C> a, C *__restrict
 //   MODE 1 (forward): the largest such sum of an x line, then, from the result, of a y line (values are
 //   shifted as the first stage of the y pass loads them);
 //   MODE 2: the product with V(r) (fixed point below the plane's largest |V|), then as MODE 1.
-// Each is an upper bound taken from the leading 21 bits.  Rounding is at 2^-61 of those sums: against exact
-// transforms (36^3, flat and decaying data) the relative error of a transform is 3.0-4.3e-16, with the FP64
-// passes 3.8-5.5e-16 (the z passes stay FP64).
+// Each is an upper bound taken from the leading 21 bits.  Rounding is at 2^-61 of those sums: against extended
+// precision (flat data, 24^3 to 72^3) the relative error of a transform is 1.0-2.1e-16, as FP64 3.1-4.1e-16.
 // 64 packed grids of the 63-well cell (72^3, 4608 planes), FP64 pass -> this one: inverse 1490 -> 502 us,
 // forward 1595 -> 669, H product 2710 -> 1017.  Bound by instruction issue (57 thousand warp instructions a
 // plane, 42% of the issue slots used: few warps and a barrier per stage).  Measured and not kept: radices
@@ -566,8 +565,22 @@ __device__ fx::C2 *z_lines(const FzArgs &a, double2 *Ad, fx::C2 *B, fx::Unit &un
   });
 }
 
+// A real factor and the same over sqrt(2), the latter in two parts: as one double, its rounding and that of
+// 1 / sqrt(2) are the same for every element and were most of a fixed-point transform's error.  There and back
+// with a product between (flat data, against extended precision): 36^3 2.8e-16 -> 1.1e-16, 45 40 54 3.5e-16 ->
+// 1.1e-16, 72^3 2.9e-16 -> 1.4e-16; as FP64 2.4e-16, 3.2e-16 and 2.4e-16.  No difference in time.
+struct PairScale {
+  double all, hi, lo;
+  explicit PairScale(long double scale) : all((double)scale) {
+    const long double p = scale * 0.70710678118654752440084436210484903928L;
+    hi = (double)p;
+    lo = (double)(p - (long double)hi);
+  }
+  __device__ __forceinline__ double operator()(double x) const { return fma(x, hi, x * lo); }
+};
+
 __global__ void __launch_bounds__(kZMax, 2) sph_z_inv_fx(FzArgs a, int nf, int npw, const double *__restrict__ X,
-                                                      double scale, double2 *__restrict__ colbuf) {
+                                                      PairScale scale, double2 *__restrict__ colbuf) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   double2 *A = reinterpret_cast<double2 *>(sm_raw);
   fx::C2 *B = reinterpret_cast<fx::C2 *>(A + (size_t)a.CG * a.N3p);
@@ -582,12 +595,11 @@ __global__ void __launch_bounds__(kZMax, 2) sph_z_inv_fx(FzArgs a, int nf, int n
     const int4 en = __ldg(&a.ent[e]);
     const int kk = en.x;
     if (kk == 0) {
-      A[en.y] = make_double2(f[0] * scale, hasg ? h[0] * scale : 0.0);
+      A[en.y] = make_double2(f[0] * scale.all, hasg ? h[0] * scale.all : 0.0);
       continue;
     }
-    const double r2 = kRs2 * scale;
-    const double fc = f[2 * kk - 1] * r2, fs = f[2 * kk] * r2;
-    const double gc = hasg ? h[2 * kk - 1] * r2 : 0.0, gs = hasg ? h[2 * kk] * r2 : 0.0;
+    const double fc = scale(f[2 * kk - 1]), fs = scale(f[2 * kk]);
+    const double gc = hasg ? scale(h[2 * kk - 1]) : 0.0, gs = hasg ? scale(h[2 * kk]) : 0.0;
     A[en.y] = make_double2(fc - gs, fs + gc);  // c_f + i c_g at +G
     A[en.z] = make_double2(fc + gs, gc - fs);  // conj(c_f) + i conj(c_g) at -G
   }
@@ -603,7 +615,7 @@ __global__ void __launch_bounds__(kZMax, 2) sph_z_inv_fx(FzArgs a, int nf, int n
 }
 
 __global__ void __launch_bounds__(kZMax, 2) sph_z_fwd_fx(FzArgs a, int nf, int npw, const double2 *__restrict__ colbuf,
-                                                      double *__restrict__ Y, double scale,
+                                                      double *__restrict__ Y, PairScale scale,
                                                       const double *__restrict__ Xd, const double *__restrict__ kin,
                                                       const double *__restrict__ shift, int period,
                                                       double shift_const) {
@@ -632,17 +644,16 @@ __global__ void __launch_bounds__(kZMax, 2) sph_z_fwd_fx(FzArgs a, int nf, int n
       const fx::C2 v = F[en.y];
       i0 = 0;
       i1 = -1;
-      a0 = unit(v.x) * scale;
-      b0 = unit(v.y) * scale;
+      a0 = unit(v.x) * scale.all;
+      b0 = unit(v.y) * scale.all;
     } else {
       const fx::C2 Fp = F[en.y], Fm = F[en.z];
-      const double s = kRs2 * scale;
       i0 = 2 * kk - 1;
       i1 = 2 * kk;
-      a0 = unit(Fp.x + Fm.x) * s;
-      a1 = unit(Fp.y - Fm.y) * s;
-      b0 = unit(Fp.y + Fm.y) * s;
-      b1 = unit(Fm.x - Fp.x) * s;
+      a0 = scale(unit(Fp.x + Fm.x));
+      a1 = scale(unit(Fp.y - Fm.y));
+      b0 = scale(unit(Fp.y + Fm.y));
+      b1 = scale(unit(Fm.x - Fp.x));
     }
     if (Xd) {
       a0 += (kin[i0] + sh0) * Xd[(long)f0 * npw + i0];
@@ -663,7 +674,7 @@ __global__ void __launch_bounds__(kZMax, 2) sph_z_fwd_fx(FzArgs a, int nf, int n
 
 // the pair pipelines' z passes (dsph_z_fwd, dsph_z_inv below) for FP64 data
 __global__ void __launch_bounds__(kZMax, 2) dsph_z_fwd_fx(FzArgs a, int np, int npw, double2 *__restrict__ colbuf,
-                                                       double *__restrict__ X, double scale,
+                                                       double *__restrict__ X, PairScale scale,
                                                        const double *__restrict__ vcg, double cscale) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   double2 *A = reinterpret_cast<double2 *>(sm_raw);
@@ -684,17 +695,16 @@ __global__ void __launch_bounds__(kZMax, 2) dsph_z_fwd_fx(FzArgs a, int np, int 
       const int kk = en.x;
       if (kk == 0) {
         const fx::C2 v = F[en.y];
-        X[(long)f0 * npw] = unit(v.x) * scale;
-        if (hasg) X[(long)f1 * npw] = unit(v.y) * scale;
+        X[(long)f0 * npw] = unit(v.x) * scale.all;
+        if (hasg) X[(long)f1 * npw] = unit(v.y) * scale.all;
         continue;
       }
       const fx::C2 Fp = F[en.y], Fm = F[en.z];
-      const double sc = kRs2 * scale;
-      X[(long)f0 * npw + 2 * kk - 1] = unit(Fp.x + Fm.x) * sc;
-      X[(long)f0 * npw + 2 * kk] = unit(Fp.y - Fm.y) * sc;
+      X[(long)f0 * npw + 2 * kk - 1] = scale(unit(Fp.x + Fm.x));
+      X[(long)f0 * npw + 2 * kk] = scale(unit(Fp.y - Fm.y));
       if (hasg) {
-        X[(long)f1 * npw + 2 * kk - 1] = unit(Fp.y + Fm.y) * sc;
-        X[(long)f1 * npw + 2 * kk] = unit(Fm.x - Fp.x) * sc;
+        X[(long)f1 * npw + 2 * kk - 1] = scale(unit(Fp.y + Fm.y));
+        X[(long)f1 * npw + 2 * kk] = scale(unit(Fm.x - Fp.x));
       }
     }
   }
@@ -709,7 +719,7 @@ __global__ void __launch_bounds__(kZMax, 2) dsph_z_fwd_fx(FzArgs a, int np, int 
 }
 
 __global__ void __launch_bounds__(kZMax, 2) dsph_z_inv_fx(FzArgs a, int np, int npw, const double *__restrict__ X,
-                                                       double scale, double2 *__restrict__ colbuf) {
+                                                       PairScale scale, double2 *__restrict__ colbuf) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   double2 *A = reinterpret_cast<double2 *>(sm_raw);
   fx::C2 *B = reinterpret_cast<fx::C2 *>(A + (size_t)a.CG * a.N3p);
@@ -729,12 +739,11 @@ __global__ void __launch_bounds__(kZMax, 2) dsph_z_inv_fx(FzArgs a, int np, int 
       const int kk = en.x;
       double2 &tp = A[en.y];
       if (kk == 0) {
-        tp = make_double2(tp.x + f[0] * scale, tp.y + (hasg ? h[0] * scale : 0.0));
+        tp = make_double2(tp.x + f[0] * scale.all, tp.y + (hasg ? h[0] * scale.all : 0.0));
         continue;
       }
-      const double r2 = kRs2 * scale;
-      const double fc = f[2 * kk - 1] * r2, fs = f[2 * kk] * r2;
-      const double gc = hasg ? h[2 * kk - 1] * r2 : 0.0, gs = hasg ? h[2 * kk] * r2 : 0.0;
+      const double fc = scale(f[2 * kk - 1]), fs = scale(f[2 * kk]);
+      const double gc = hasg ? scale(h[2 * kk - 1]) : 0.0, gs = hasg ? scale(h[2 * kk]) : 0.0;
       tp = make_double2(tp.x + (fc - gs), tp.y + (fs + gc));
       double2 &tm = A[en.z];
       tm = make_double2(tm.x + (fc + gs), tm.y + (gc - fs));
@@ -1007,23 +1016,23 @@ int z_threads(const Ctx &c) {
 
 // the z passes of either precision: FP64 in fixed point, FP32 as it is
 template <class C>
-void launch_z_inv(Ctx &c, int nf, int nq, const double *X, double scale, C *cb) {
+void launch_z_inv(Ctx &c, int nf, int nq, const double *X, long double scale, C *cb) {
   const dim3 grid(c.sfft.ngroups, nq);
   if constexpr (sizeof(C) == sizeof(double2))
-    sph_z_inv_fx<<<grid, z_threads(c), z_smem<C>(c), c.stream>>>(fz_args(c, c.sfft), nf, c.npw, X, scale, cb);
+    sph_z_inv_fx<<<grid, z_threads(c), z_smem<C>(c), c.stream>>>(fz_args(c, c.sfft), nf, c.npw, X, PairScale(scale), cb);
   else
-    sph_z_inv<C><<<grid, kThreads, z_smem<C>(c), c.stream>>>(make_args<C>(c, c.sfft), nf, c.npw, X, scale, cb);
+    sph_z_inv<C><<<grid, kThreads, z_smem<C>(c), c.stream>>>(make_args<C>(c, c.sfft), nf, c.npw, X, (double)scale, cb);
   BSE_CHECK_LAUNCH();
 }
 template <class C>
-void launch_z_fwd(Ctx &c, int nf, int nq, const C *cb, double *Y, double scale, const double *Xd, const double *shift,
+void launch_z_fwd(Ctx &c, int nf, int nq, const C *cb, double *Y, long double scale, const double *Xd, const double *shift,
                   int period, double shift_const) {
   const dim3 grid(c.sfft.ngroups, nq);
   if constexpr (sizeof(C) == sizeof(double2))
-    sph_z_fwd_fx<<<grid, z_threads(c), z_smem<C>(c), c.stream>>>(fz_args(c, c.sfft), nf, c.npw, cb, Y, scale, Xd,
+    sph_z_fwd_fx<<<grid, z_threads(c), z_smem<C>(c), c.stream>>>(fz_args(c, c.sfft), nf, c.npw, cb, Y, PairScale(scale), Xd,
                                                                c.kin.get(), shift, period, shift_const);
   else
-    sph_z_fwd<C><<<grid, kThreads, z_smem<C>(c), c.stream>>>(make_args<C>(c, c.sfft), nf, c.npw, cb, Y, scale, Xd,
+    sph_z_fwd<C><<<grid, kThreads, z_smem<C>(c), c.stream>>>(make_args<C>(c, c.sfft), nf, c.npw, cb, Y, (double)scale, Xd,
                                                              c.kin.get(), shift, period, shift_const);
   BSE_CHECK_LAUNCH();
 }
@@ -1151,8 +1160,8 @@ void dens_forward(Ctx &c, int np, CT<R> *P, R *X, double scale, const R *vcg, R 
   else launch_xy<C, 1>(c, c.dfft, nq, cb, P, nullptr);
   const dim3 grid(c.dfft.ngroups, nq);
   if constexpr (std::is_same<R, double>::value)
-    dsph_z_fwd_fx<<<grid, z_threads(c), z_smem<C>(c, c.dfft), c.stream>>>(fz_args(c, c.dfft), np, c.npw, cb, X, scale,
-                                                                        vcg, cscale);
+    dsph_z_fwd_fx<<<grid, z_threads(c), z_smem<C>(c, c.dfft), c.stream>>>(fz_args(c, c.dfft), np, c.npw, cb, X,
+                                                                        PairScale(scale), vcg, cscale);
   else
     dsph_z_fwd<C, R><<<grid, kThreads, z_smem<C>(c, c.dfft), c.stream>>>(make_args<C>(c, c.dfft), np, c.npw, cb, X,
                                                                          scale, vcg, cscale);
@@ -1168,7 +1177,8 @@ void dens_inverse(Ctx &c, int np, const R *X, double scale, CT<R> *P) {
   C *cb = c.grids<R>().colbuf_dens.get();
   const dim3 grid(c.dfft.ngroups, nq);
   if constexpr (std::is_same<R, double>::value)
-    dsph_z_inv_fx<<<grid, z_threads(c), z_smem<C>(c, c.dfft), c.stream>>>(fz_args(c, c.dfft), np, c.npw, X, scale, cb);
+    dsph_z_inv_fx<<<grid, z_threads(c), z_smem<C>(c, c.dfft), c.stream>>>(fz_args(c, c.dfft), np, c.npw, X,
+                                                                        PairScale(scale), cb);
   else
     dsph_z_inv<C, R><<<grid, kThreads, z_smem<C>(c, c.dfft), c.stream>>>(make_args<C>(c, c.dfft), np, c.npw, X, scale,
                                                                          cb);
@@ -1191,7 +1201,7 @@ bool sphere_fft_ok(const Ctx &c) {
 }
 
 template <class R>
-void sphere_to_grid(Ctx &c, int nf, const double *X, CT<R> *P, double scale, CT<R> *colbuf) {
+void sphere_to_grid(Ctx &c, int nf, const double *X, CT<R> *P, long double scale, CT<R> *colbuf) {
   using C = CT<R>;
   if (nf <= 0) return;
   const int nq = (nf + 1) / 2;
@@ -1202,7 +1212,7 @@ void sphere_to_grid(Ctx &c, int nf, const double *X, CT<R> *P, double scale, CT<
 }
 
 template <class R>
-void grid_to_sphere(Ctx &c, int nf, CT<R> *P, double *Y, double scale, const double *Xd, const double *shift,
+void grid_to_sphere(Ctx &c, int nf, CT<R> *P, double *Y, long double scale, const double *Xd, const double *shift,
                     int period, double shift_const, CT<R> *colbuf) {
   using C = CT<R>;
   if (nf <= 0) return;
@@ -1220,7 +1230,7 @@ void sphere_h(Ctx &c, int nf, const double *X, double *HX, const double *shift) 
   const int nq = (nf + 1) / 2;
   set_attrs<C>();
   C *cb = colbuf_for<R>(c, nq);
-  const double s_in = 1.0 / std::sqrt(c.omega), s_out = std::sqrt(c.omega) / (double)c.nr;
+  const long double s_in = 1.0L / std::sqrt((long double)c.omega), s_out = std::sqrt((long double)c.omega) / c.nr;
   launch_z_inv<C>(c, nf, nq, X, s_in, cb);
   launch_xy<C, 2>(c, c.sfft, nq, cb, nullptr, c.grids<R>().vloc.get());
   launch_z_fwd<C>(c, nf, nq, cb, HX, s_out, X, shift, shift ? c.nocc : 1, 0.0);
@@ -1228,11 +1238,11 @@ void sphere_h(Ctx &c, int nf, const double *X, double *HX, const double *shift) 
 
 template bool sphere_fft_ok<double>(const Ctx &);
 template bool sphere_fft_ok<float>(const Ctx &);
-template void sphere_to_grid<double>(Ctx &, int, const double *, double2 *, double, double2 *);
-template void sphere_to_grid<float>(Ctx &, int, const double *, float2 *, double, float2 *);
-template void grid_to_sphere<double>(Ctx &, int, double2 *, double *, double, const double *, const double *, int,
+template void sphere_to_grid<double>(Ctx &, int, const double *, double2 *, long double, double2 *);
+template void sphere_to_grid<float>(Ctx &, int, const double *, float2 *, long double, float2 *);
+template void grid_to_sphere<double>(Ctx &, int, double2 *, double *, long double, const double *, const double *, int,
                                      double, double2 *);
-template void grid_to_sphere<float>(Ctx &, int, float2 *, double *, double, const double *, const double *, int,
+template void grid_to_sphere<float>(Ctx &, int, float2 *, double *, long double, const double *, const double *, int,
                                     double, float2 *);
 template void sphere_h<double>(Ctx &, int, const double *, double *, const double *);
 template void sphere_h<float>(Ctx &, int, const double *, double *, const double *);

@@ -441,6 +441,11 @@ void run(char ta, char tb, int M, int N, int K, double alpha, const double *A, i
 
 }  // namespace
 
+size_t digit_scratch(int M, int N, int K) {
+  const size_t slices = ((size_t)K + kMaxSlice - 1) / kMaxSlice;
+  return ((size_t)M + N + 1) / 2 + (slices > 1 ? slices * M * N : 0);
+}
+
 void digit_gemm(int digits, char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda,
                 const double *B, int ldb, double beta, double *C, int ldc, cudaStream_t s, DevBuf<double> &scratch,
                 bool fixed, int split_pct) {

@@ -1,6 +1,7 @@
-// FP64 dense linear algebra for the plain path: tiled SIMT GEMM (occupied overlaps of
-// P_c, PDEP projection and back-projection of Eq. 3, Davidson subspace products),
-// deterministic row reductions, and the host eigensolver for Rayleigh-Ritz matrices.
+// Dense linear algebra: the choice of a GEMM form (occupied overlaps of P_c, PDEP projection and
+// back-projection of Eq. 3, Davidson subspace products; FP64 by digit products, digit_gemm.cu, but for long
+// or thin shapes), the tiled FP32 SIMT GEMM, deterministic row reductions, and the host eigensolver for
+// Rayleigh-Ritz matrices.
 #include <unistd.h>
 
 #include <algorithm>
@@ -298,7 +299,7 @@ DevBuf<float> &splitk_buf32() {
 }
 
 // Number of K slices for a tiled product with `tiles` output tiles.  One 256-thread CTA already
-// saturates an SM's FP64 pipe, so the time of a launch is about the largest number of CTAs that
+// saturates an SM's arithmetic, so the time of a launch is about the largest number of CTAs that
 // any of the 152 SMs receives times (the K length of one CTA + a fixed per-CTA cost of about
 // 8 K steps for the prologue and the partial-tile store); the split minimises that.
 int split_for(long tiles, int K) {
@@ -321,7 +322,7 @@ int split_for(long tiles, int K) {
   return best;
 }
 
-// tiled path shared by the FP64 and FP32 GEMMs (split-K when the output has few tiles)
+// the tiled FP32 GEMM (split-K when the output has few tiles)
 // fixed: `scratch` keeps its size (its address is recorded in captured graphs); the split is
 // clamped to what fits, down to no split at all
 template <class T>
@@ -461,7 +462,20 @@ void dgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A,
   // latency): N T 80 x 216 x 6859 72 us (383 before), 200 x 216 x 922 34 (121), 128 x 128 x 6859 56 (205),
   // 16 x 16 x 500 15 (86); N N 128 x 6859 x 128 71 (210), 128 x 373248 x 128 3.0 ms (10.0), 4 x 4 x 8 7 us
   // (18); no shape of 1..512 x 1..373248 x 1..200000 was found where they were faster
-  const bool fits = fixed && fixed->n >= ((size_t)M + N + 1) / 2;
+  // a fixed buffer too small for the whole product (millions of rows, or more than 2^19 k): in parts, so that a
+  // captured launch never holds the address of a buffer that can grow
+  if (fixed && fixed->n < digit_scratch(M, N, K) && M * (long)N > 1) {
+    const int m = N >= M ? M : M / 2, n = N >= M ? N / 2 : N;
+    dgemm(ta, tb, m, n, K, alpha, A, lda, B, ldb, beta, C, ldc, s, fixed, split_pct);
+    if (n < N)
+      dgemm(ta, tb, M, N - n, K, alpha, A, lda, B + (tb == 'T' ? (long)n * ldb : n), ldb, beta, C + n, ldc, s, fixed,
+            split_pct);
+    else
+      dgemm(ta, tb, M - m, N, K, alpha, A + (ta == 'N' ? (long)m * lda : m), lda, B, ldb, beta, C + (long)m * ldc, ldc,
+            s, fixed, split_pct);
+    return;
+  }
+  const bool fits = fixed && fixed->n >= digit_scratch(M, N, K);
   digit_gemm(8, ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, fits ? *fixed : splitk_buf(), fits, split_pct);
 }
 

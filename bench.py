@@ -34,21 +34,17 @@ MIXED_DAVIDSON_TOL = 1e-5
 ZVEC_TOL = 1e-10
 GS_TOL = 1e-10
 
-# DRAM traffic per launch of the fused K1d/combine kernel from one ncu capture, valid
-# only for the kernel source it was measured on (hash of kernels.cu).
 # DRAM traffic of the timed kernels, from one ncu capture each of a smaller case of the same
 # kernel (profiles/), keyed by a hash of the kernel's source text so that a changed kernel
 # reports null.  tau_factor: DRAM bytes read per algorithmic tau byte; the traffic of a full
 # launch is its algorithmic bytes with tau counted tau_factor times.
 NCU_TRAFFIC = {
-    # k1d_tma_kernel (column order, two-column register prefetch), N_occ = 64, 4-vector block:
-    # 3.59 GB read + 0.37 GB written against 3.97 GB algorithmic (tau 3.11 GB read once);
-    # profiles/k1d_tma_persistent_nocc64_mixed.md
-    "baa5281222e96203": {"tau_factor": 1.0},
-    # combine_tau_kernel (FP64), N_occ = 48, 2-vector block: 7.34 GB read + 0.28 GB written against
-    # 4.24 GB algorithmic (tau 3.51 GB, read about twice: by the two output tiles of each pair);
-    # profiles/combine_tau_nocc48_fp64.md
-    "a5f5b8bfb34f34ad": {"tau_factor": 1.96},
+    # k1d_tma_kernel, N_occ = 64, 4-vector block: 3.59 GB read + 0.37 GB written against 3.97 GB
+    # algorithmic (tau 3.11 GB read once); profiles/k1d_tma_persistent_nocc64_mixed.md
+    "43020757bf6c12d0": {"tau_factor": 1.0},
+    # k1d_fixed_kernel (FP64), N_occ = 64, 2-vector block: 7.02 GB read + 0.49 GB written against 7.18 GB
+    # algorithmic (tau 6.21 GB read once); profiles/k1d_fixed_nocc64_fp64.md
+    "426ae02a0244db73": {"tau_factor": 1.0},
 }
 
 
@@ -65,7 +61,7 @@ def kernel_text(path, name):
     return src[start:src.index("\n}\n", m.end()) + 3]
 
 
-def kernel_source_hash(fname="kernels.cu", name="combine_tau_kernel"):
+def kernel_source_hash(fname, name):
     txt = kernel_text(os.path.join(ROOT, "paper_2607_20728_gb300", "csrc", fname), name)
     return hashlib.sha256(txt.encode()).hexdigest()[:16]
 
@@ -241,7 +237,8 @@ def whole_job_rate(world, units_per_rank, t_max_s):
 # ---------------------------------------------------------------------------------------
 def measure_fp64_peak(n=8192, reps=3):
     """Dense FP64 rate of this GPU: torch.matmul (cuBLAS DGEMM) on n x n float64, best of reps,
-    CUDA events on the current stream.  The denominator of the FP64 ALU roofline."""
+    CUDA events on the current stream.  What the FP64 K1d's multiply-adds are set beside: they run as
+    integers, so the rate is no bound on them."""
     import torch
     a = torch.randn(n, n, dtype=torch.float64, device="cuda")
     b = torch.randn(n, n, dtype=torch.float64, device="cuda")
@@ -519,18 +516,19 @@ def run_ours(args, rank, world, local_rank):
     peaks, src = measured_peaks()
     launches = max(1, k1d["launches"])
     per_launch_ms = k1d["ms"] / launches
-    achieved = (k1d["alg_flops"] / launches) / (per_launch_ms / 1e3) / 1e12 if per_launch_ms > 0 else 0.0
-    traffic = traffic_per_launch(kernel_source_hash("kernels.cu", "combine_tau_kernel"), k1d["alg_bytes"] / launches,
+    achieved = (k1d["alg_bytes"] / launches) / (per_launch_ms / 1e3) / 1e9 if per_launch_ms > 0 else 0.0
+    hbm = peaks.get("hbm_gbs")
+    tflops = (k1d["alg_flops"] / launches) / (per_launch_ms / 1e3) / 1e12 if per_launch_ms > 0 else 0.0
+    traffic = traffic_per_launch(kernel_source_hash("k1d_fixed.cu", "k1d_fixed_kernel"), k1d["alg_bytes"] / launches,
                                  stats.get("bytes_tau", 0.0))
-    roofline = {"kernel": "combine_tau_kernel (fused V a + 2 v_H phi - sum tau a, Eq. 2)", "bound": "alu",
-                "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s", "frac": achieved / fp64_peak,
-                "traffic": traffic, "peak_source": "measured: cuBLAS DGEMM (torch.matmul float64 8192^3, best of 3, "
-                                                   "CUDA events) on this GPU before the timed region",
-                "peak_nominal": 1.25,
+    roofline = {"kernel": "k1d_fixed_kernel (fused V a + 2 v_H phi - sum tau a, Eq. 2, FP64 as fixed point)",
+                "bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
+                "traffic": traffic, "peak_source": src,
+                "fp64_tflops_equiv": tflops, "fp64_dgemm_tflops": fp64_peak,
+                "fp64_dgemm_source": "measured: cuBLAS DGEMM (torch.matmul float64 8192^3, best of 3, CUDA events) on "
+                                     "this GPU before the timed region",
                 "launches": k1d["launches"], "ms_per_launch": per_launch_ms,
                 "share_of_step": k1d["ms"] / t_ms if t_ms > 0 else None,
-                "achieved_gbs": (k1d["alg_bytes"] / launches) / (per_launch_ms / 1e3) / 1e9 if per_launch_ms else 0.0,
-                "hbm_peak_gbs": peaks.get("hbm_gbs"), "hbm_peak_source": src,
                 "fft_ms_per_launch": fft["ms"] / max(1, fft["launches"]), "fft_launches": fft["launches"],
                 "fft_share_of_step": fft["ms"] / t_ms if t_ms > 0 else None,
                 "sphere_fft_ms_per_launch": sfft["ms"] / max(1, sfft["launches"]),
@@ -890,7 +888,7 @@ def run_batched(pkg, bse_inputs, workers=8):
         if st is None:
             continue
         key = (f"fft={'full' if st['tuned_full_grid_fft'] else 'sphere'} k1d_nb={st['tuned_k1d_nb']} "
-               f"xy_threads={st['tuned_xy_threads'] or 512} gemm_split={st['tuned_gemm_split_pct']}%")
+               f"xy_threads={st['tuned_xy_threads'] or 'default'} gemm_split={st['tuned_gemm_split_pct']}%")
         choices[key] = choices.get(key, 0) + 1
         graphed += st["zvector_graphed"]
     b.close()

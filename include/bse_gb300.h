@@ -329,6 +329,13 @@ bse_status bse_selftest_bounded_wait(void *stream);
  * context without that pipeline, BSE_ERR_CUDA otherwise. */
 bse_status bse_selftest_k1d_stall(bse_ctx *ctx);
 
+/* Failure-detection self-test of the FP64 K1d pipeline inside the U vector of `root` (after
+ * bse_davidson, FP64, n_occ >= 16): its producer warps issue no copies, every consumer's bounded wait
+ * gives up after one second, and the U vector must report it.  Nothing of the context changes.  Returns
+ * BSE_ERR_TIMEOUT when that happened (expected; the context stays usable), BSE_ERR_STATE for a context
+ * without that pipeline or without roots, BSE_ERR_CUDA otherwise. */
+bse_status bse_selftest_uvector_stall(bse_ctx *ctx, int root);
+
 /* Host-only utility: all eigenvalues w[n] (ascending) of the symmetric A[n][n] and the
  * eigenvectors of the k lowest (columns 0..k-1 of V[n][n]; the other columns are left as
  * they are): Householder tridiagonalisation, eigenvalues by implicit QR without vectors,

@@ -130,6 +130,7 @@ def load_library():
         "bse_host_sym_eig": (ctypes.c_int, [ctypes.c_int, _dp, _dp, _dp]),
         "bse_selftest_bounded_wait": (ctypes.c_int, [vp]),
         "bse_selftest_k1d_stall": (ctypes.c_int, [vp]),
+        "bse_selftest_uvector_stall": (ctypes.c_int, [vp, ctypes.c_int]),
         "bse_sphere_to_grid": (ctypes.c_int, [vp, ctypes.c_int, vp, vp]),
         "bse_batch_timing": (ctypes.c_int, [vp, _dp, _dp]),
         "bse_grid_to_sphere": (ctypes.c_int, [vp, ctypes.c_int, vp, vp]),

@@ -2618,13 +2618,11 @@ void uvector_t(Ctx &c, int root, double *U) {
   sync(c);
 }
 
+// U of one root; its apply goes past apply_liouville, so the flag of the streamed K1d kernels is read here
 void uvector_impl(Ctx &c, int root, double *U) {
-  if (c.prec == 0) {
-    uvector_t<double>(c, root, U);
-  } else {
-    uvector_t<float>(c, root, U);
-    check_device_flag(c);
-  }
+  if (c.prec == 0) uvector_t<double>(c, root, U);
+  else uvector_t<float>(c, root, U);
+  check_device_flag(c);
 }
 
 // Batched preconditioned CG for P_c (H - eps_v) x_v = b_v on P_c, all orbitals at once, with the
@@ -3663,6 +3661,28 @@ bse_status bse_selftest_k1d_stall(bse_ctx *ctx) {
   bse::sync(c);
   bse::check_device_flag(c);  // BSE_ERR_TIMEOUT when the waits gave up
   throw bse::Error(BSE_ERR_CUDA, "the K1d pipeline's bounded waits did not give up");
+  BSE_API_END(ctx)
+}
+
+bse_status bse_selftest_uvector_stall(bse_ctx *ctx, int root) {
+  BSE_API_BEGIN
+  BSE_REQUIRE(ctx, "ctx is required");
+  bse::Ctx &c = ctx->c;
+  if (!c.have_gs || !c.k1x.ready)
+    throw bse::Error(BSE_ERR_STATE, "no fixed-point K1d pipeline (FP64, n_occ from 16 up to what its tiles hold)");
+  if (c.nroots == 0) throw bse::Error(BSE_ERR_STATE, "no excitation");
+  BSE_REQUIRE(root >= 0 && root < c.nroots, "root out of range");
+  bse::DevBuf<double> U;
+  U.alloc((size_t)c.nocc * c.npw);
+  c.k1x.hold = 1;
+  try {
+    bse::uvector_impl(c, root, U.get());
+  } catch (...) {
+    c.k1x.hold = 0;
+    throw;
+  }
+  c.k1x.hold = 0;
+  throw bse::Error(BSE_ERR_CUDA, "the U vector did not report the waits that gave up");
   BSE_API_END(ctx)
 }
 

@@ -194,6 +194,7 @@ struct K1dFixed {
   long npairs = 0;
   int *err = nullptr;                  // device flag set when a bounded wait gives up
   bool ready = false;
+  int hold = 0;                        // failure-detection self-test only: the producer issues no copies
 };
 // position (in pairs) of the pair (v', v), v' <= v, inside one 32-point tile of that layout
 __host__ __device__ inline long k1d_tile_slot(int vp, int v, int nocc) {

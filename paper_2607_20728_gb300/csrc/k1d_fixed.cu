@@ -19,7 +19,9 @@
 // into a ring of 32 KB stages.  Warps 0-3 accumulate Y_c += tau^T a_I in registers over the column
 // ("role A", two orbitals each), warps 4-7 add tau a_c to the rows of Y_I chunk by chunk ("role B").
 // Within a column no two warps write the same rows of Y; a named barrier separates columns.  One more warp
-// is the producer and runs ahead over tile boundaries.  (Warp numbers for 8 consumer warps.)
+// is the producer and runs ahead over tile boundaries.  (Warp numbers for 8 consumer warps.)  Waits are
+// bounded: a consumer whose wait runs out sets the device flag and the CTA's, every warp still passes the
+// same barriers up to the next tile's first one, and all leave there; hold != 0 (self-test) makes them run out.
 //
 // Time of one launch, FP64 kernel before -> this one (tau at the measured copy rate): N_occ = 128, 72^3: one
 // vector 10.41 -> 4.87 ms (3.64), two 20.28 -> 7.82; N_occ = 63, 72^3: 2.64 -> 1.38 (0.89), two 5.13 -> 2.63;
@@ -107,7 +109,7 @@ __global__ void __launch_bounds__(W * 32 + 32, 16 / W) k1d_fixed_kernel(
     const int2 *__restrict__ tau, const double *__restrict__ tscale, long npairs, long nr, int nocc, int nb_total,
     int b0, int stages, const double *__restrict__ phir, const double *__restrict__ vloc,
     const double *__restrict__ Pa, const double *__restrict__ Pvh, double *__restrict__ Py, int use_vloc, int use_k1e,
-    int *__restrict__ err) {
+    int *__restrict__ err, int hold) {
   extern __shared__ __align__(128) unsigned char smem[];
   int2 *tau_s = reinterpret_cast<int2 *>(smem);                                     // [stages][128][32]
   int2 *a_s = tau_s + (size_t)stages * kStageElems;                                 // [NB][nocc][32]
@@ -133,7 +135,7 @@ __global__ void __launch_bounds__(W * 32 + 32, 16 / W) k1d_fixed_kernel(
   __syncthreads();
   if (warp == W) {
     // ---- producer ----
-    if (lane == 0) {
+    if (lane == 0 && !hold) {
       long g = 0;
       int st = 0;
       unsigned round = 0;  // completed trips around the ring
@@ -386,7 +388,7 @@ void launch(const Ctx &c, const K1dFixed &t, int stages, int nb, int b0, const d
   const unsigned grid = (unsigned)std::min<long>((c.nr + kR - 1) / kR, std::max(1, nsm) * (16 / W));
   k1d_fixed_kernel<NB, W><<<grid, W * 32 + 32, smem, c.stream>>>(
       t.tau, t.scale, t.npairs, c.nr, c.nocc, nb, b0, stages, phir, vloc, reinterpret_cast<const double *>(Pa),
-      reinterpret_cast<const double *>(Pvh), reinterpret_cast<double *>(Py), use_vloc, use_k1e, t.err);
+      reinterpret_cast<const double *>(Pvh), reinterpret_cast<double *>(Py), use_vloc, use_k1e, t.err, t.hold);
   BSE_CHECK_LAUNCH();
 }
 

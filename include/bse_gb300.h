@@ -272,8 +272,11 @@ bse_status bse_fft3d_noalloc(int n1, int n2, int n3, int batch, double *data_dev
 
 /* Utility: the library's FP64 GEMM, C = alpha op(A) op(B) + beta C on device arrays,
  * row-major: ta 'N' op(A) = A [M][lda], 'T' op(A) = A^T with A [K][lda]; tb 'N' op(B) = B [K][ldb],
- * 'T' op(B) = B^T with B [N][ldb]; C [M][ldc].  It carries the occupied-space projector
- * (S = Phi^T Y, Y -= Phi S) and the Davidson / PDEP products.  Ordered on `stream`,
+ * 'T' op(B) = B^T with B [N][ldb]; C [M][ldc].  Every output is within an FP64 sum's bound,
+ * (K + 8) 2^-53 sum_k |A_ik| |B_kj| for alpha = 1 and beta = 0, whatever the range of the entries.  The same
+ * kernels carry the occupied-space projector (S = Phi^T Y, Y -= Phi S) and the Davidson / PDEP
+ * products inside the library, where the bound holds relative to the largest entries of row and
+ * column instead (max_k |A_ik| max_k |B_kj| in place of each product).  Ordered on `stream`,
  * synchronised before returning. */
 bse_status bse_gemm(char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda,
                     const double *B, int ldb, double beta, double *C, int ldc, void *stream);

@@ -3586,7 +3586,7 @@ bse_status bse_gemm(char ta, char tb, int M, int N, int K, double alpha, const d
   BSE_REQUIRE((ta == 'N' || ta == 'T') && (tb == 'N' || tb == 'T'), "ta and tb must be 'N' or 'T'");
   BSE_REQUIRE(M >= 0 && N >= 0 && K >= 0 && C, "bad sizes");
   BSE_REQUIRE(K == 0 || (A && B), "A and B are required");
-  bse::dgemm(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, (cudaStream_t)stream);
+  bse::dgemm(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, (cudaStream_t)stream, nullptr, 100, true);
   BSE_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
   BSE_API_END(ctx)
 }

@@ -13,11 +13,24 @@
 // the rounding of X.  What comes here instead of to the streaming kernels, with times, stands
 // at dgemm in linalg.cu.
 //
+// The operands' rounding is relative to the largest entry of the row or column, so an output that collects only
+// products far below (max of the row) (max of the column) has fewer correct digits than an FP64 sum: with
+// S_ij = sum_k |A_ik| |B_kj|, sA_i = sum_k |A_ik| / 2^eA, sB_j likewise (2^e just above the largest entry), the
+// error is at most 2^-56 (sA + sB) + 6 K 2^-63 in units of 2^(eA + eB), an FP64 sum's K 2^-53 S.  The products
+// of the library's solvers are norms, overlaps and rotations of whole vectors, where only the former matters.
+// With CHECK (bse_gemm) every output for which the bound is above half of an FP64 sum's is summed anew in FP64,
+// and the result is an FP64 product entry by entry, whatever the grading of rows and columns: row_exponents
+// also returns sA and sB, the kernel estimates S by one more product per tile and 16 k, of the first two digits'
+// magnitudes rounded to BF16, and the outputs it finds weak are dealt to whole warps, or summed together when a tile
+// has many.  Kernel time with CHECK (without): N T 80 x 216 x 6859 72 us (67), N N 80 x 2400 x 64 23 (20), T N
+// 200 x 6859 x 128 114 (115); with every output weak 302, 54 and 419 (as tiled FP64 kernels 384, 69 and 391).
+//
 // With ND = 4 digits (28 bits, groups s + t <= 4) the same kernel serves the products whose contract is
 // FP32 arithmetic on FP64 operands: finer operands than FP32's 24 bits and exact sums, 13 products
 // instead of 43.
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include <cuda_bf16.h>
 
@@ -29,12 +42,15 @@ namespace {
 constexpr int kKC = 16;             // k per staged chunk
 constexpr int kRawStride = kKC + 2;  // doubles per staged row (16-byte aligned, rows off the same banks)
 constexpr int kDigStride = kKC + 8;  // bf16 per digit row: ldmatrix reads 8 rows without bank conflicts
-constexpr int kMaxStrips = 9;       // 16-row strips of A and B per CTA
-constexpr int kRows = 16 * kMaxStrips;
+// 16-row strips of A and B per CTA (with CHECK the sums of S take the place of the ninth)
+template <bool CHECK>
+constexpr int kMaxStrips = CHECK ? 8 : 9;
 constexpr int kWarps = 16;
 constexpr int kFlush = 8;           // chunks between reads of the FP32 accumulators (128 k)
 constexpr int kBadExp = 1 << 28;    // row holds a non-finite value
 constexpr int kMaxSlice = 1 << 19;  // longest K slice
+constexpr int kFewWeak = 64;        // weak outputs of a tile that go to one warp each
+constexpr int kStageK = 64;         // k at a time for more
 
 // |x| < 2^e  ->  round(x 2^(kBits - e)), kBits = 7 ND - 1
 template <int ND>
@@ -83,19 +99,56 @@ __device__ __forceinline__ int exponent_of(unsigned long long m) {
   return E ? E - 1022 : m ? 64 - __clzll(m) - 1074 : 0;
 }
 
+// Running sum of |x| from above: sum 2^(E - 1043), E the largest biased exponent so far, every term rounded up to
+// its leading 21 bits below that (integers: the FP64 pipe would take longer than the loads)
+struct AbsSum {
+  unsigned long long sum;
+  int E;
+  __device__ __forceinline__ void rescale(int to) {
+    if (to > E) {
+      const int d = to - E;
+      sum = sum ? (d > 63 ? 0 : sum >> d) + 1 : 0;
+      E = to;
+    }
+  }
+  __device__ __forceinline__ void add(unsigned long long bits) {  // of |x|
+    const unsigned h = (unsigned)(bits >> 32);
+    const int e = max((int)(h >> 20), 1);
+    rescale(e);
+    const unsigned m = (h & 0xfffffu) | (h >> 20 ? 0x100000u : 0u);
+    sum += bits ? (E - e > 31 ? 0u : m >> (E - e)) + 1u : 0u;
+  }
+  __device__ __forceinline__ void add(AbsSum o) {
+    const int to = max(E, o.E);
+    rescale(to);
+    o.rescale(to);
+    sum += o.sum;
+  }
+};
+
 // Exponents of the rows of op(A) and the columns of op(B): the smallest e with |x| < 2^e over the row,
-// kBadExp when a value is not finite.  Rows that are contiguous in k take one CTA each; rows that lie
-// across the memory (k strides by ld) go 32 to a CTA, 8 k at a time, coalesced over the rows.
+// kBadExp when a value is not finite; with CHECK also sum |x| / 2^e from above, 0 for a row of zeros.  Rows that
+// are contiguous in k take one CTA each; rows that lie across the memory (k strides by ld) go 32 to a CTA, 8 k
+// at a time, coalesced over the rows.
+template <bool CHECK>
 __global__ void __launch_bounds__(256) row_exponents(int M, int N, int K, bool a_across, const double *__restrict__ A,
                                                      int lda, bool b_across, const double *__restrict__ B, int ldb,
-                                                     int nblk_a, int *__restrict__ ex) {
+                                                     int nblk_a, int *__restrict__ ex, float *__restrict__ sums) {
   __shared__ unsigned long long red[8][32];
+  __shared__ AbsSum sred[CHECK ? 8 : 1][32];
   const bool isb = (int)blockIdx.x >= nblk_a;
   const int blk = isb ? blockIdx.x - nblk_a : blockIdx.x;
   const bool across = isb ? b_across : a_across;
   const double *X = isb ? B : A;
   const int ld = isb ? ldb : lda, rows = isb ? N : M;
   int *out = ex + (isb ? M : 0);
+  float *sout = sums + (isb ? M : 0);
+  AbsSum t{0, 1};
+  auto sum_of = [](AbsSum a, unsigned long long top) {
+    const int e = exponent_of(top);
+    if (top == 0 || e == kBadExp) return 0.f;
+    return fmaxf(0.5f, (float)ldexp((double)a.sum, a.E - 1043 - e));
+  };
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned long long m = 0;
   auto bits = [](double x) { return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull; };
@@ -103,31 +156,79 @@ __global__ void __launch_bounds__(256) row_exponents(int M, int N, int K, bool a
     const int row = blk * 32 + lane;
     if (row < rows)
 #pragma unroll 8
-      for (int k = warp; k < K; k += 8) m = max(m, bits(__ldg(&X[(long)k * ld + row])));
+      for (int k = warp; k < K; k += 8) {
+        const unsigned long long x = bits(__ldg(&X[(long)k * ld + row]));
+        m = max(m, x);
+        if (CHECK) t.add(x);
+      }
     red[warp][lane] = m;
+    if (CHECK) sred[warp][lane] = t;
     __syncthreads();
     if (warp == 0 && row < rows) {
       for (int w = 1; w < 8; ++w) m = max(m, red[w][lane]);
       out[row] = exponent_of(m);
+      if (CHECK) {
+        for (int w = 1; w < 8; ++w) t.add(sred[w][lane]);
+        sout[row] = sum_of(t, m);
+      }
     }
   } else {
     const double *x = X + (long)blk * ld;
 #pragma unroll 8
-    for (int k = threadIdx.x; k < K; k += 256) m = max(m, bits(__ldg(&x[k])));
-    for (int w = 16; w > 0; w >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, w));
-    if (lane == 0) red[0][warp] = m;
+    for (int k = threadIdx.x; k < K; k += 256) {
+      const unsigned long long v = bits(__ldg(&x[k]));
+      m = max(m, v);
+      if (CHECK) t.add(v);
+    }
+    for (int w = 16; w > 0; w >>= 1) {
+      m = max(m, __shfl_xor_sync(0xffffffffu, m, w));
+      if (CHECK) {
+        AbsSum o;
+        o.sum = __shfl_xor_sync(0xffffffffu, t.sum, w);
+        o.E = __shfl_xor_sync(0xffffffffu, t.E, w);
+        t.add(o);
+      }
+    }
+    if (lane == 0) {
+      red[0][warp] = m;
+      if (CHECK) sred[0][warp] = t;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
       for (int w = 1; w < 8; ++w) m = max(m, red[0][w]);
       out[blk] = exponent_of(m);
+      if (CHECK) {
+        for (int w = 1; w < 8; ++w) t.add(sred[0][w]);
+        sout[blk] = sum_of(t, m);
+      }
     }
   }
 }
 
-template <int ND>
+// Whether an output needs the FP64 sum: a row or column is not finite, or the bound above exceeds half of an FP64
+// sum's.  S is overestimated by less than a tenth plus 2^-13 (sA + sB) (the digits left out), so an output that
+// passes does meet it; the other half is for the roundings of up to K/64 slices, alpha and beta.
+__device__ __forceinline__ bool weak(int ea, int eb, float sa, float sb, int K, float S) {
+  if (ea == kBadExp || eb == kBadExp) return true;
+  if (sa == 0.f || sb == 0.f) return false;
+  const float k = (float)K, s = sa + sb;
+  return !(S >= 1.1f * (0.125f * s + 0.006f * k) / (0.5f * k + 4.f) + 1.25e-4f * s);
+}
+// sum_k a[k sa] b[k sb] by a warp, the result in every lane
+__device__ __forceinline__ double warp_dot(const double *__restrict__ a, long sa, const double *__restrict__ b, long sb,
+                                           int K) {
+  double s = 0.0;
+#pragma unroll 8
+  for (int k = threadIdx.x & 31; k < K; k += 32) s = fma(__ldg(a + k * sa), __ldg(b + k * sb), s);
+  for (int w = 16; w > 0; w >>= 1) s += __shfl_xor_sync(0xffffffffu, s, w);
+  return s;
+}
+
+template <int ND, bool CHECK>
 constexpr size_t digit_smem() {
-  return (size_t)2 * kRows * kRawStride * 8 + (size_t)2 * ND * kRows * kDigStride * 2 +
-         (ND == 8 ? (size_t)kWarps * 32 * 8 * 16 : 0) + kRows * 12;
+  constexpr int rows = 16 * kMaxStrips<CHECK>;
+  return (size_t)2 * rows * kRawStride * 8 + (size_t)2 * ND * rows * kDigStride * 2 +
+         (ND == 8 ? (size_t)kWarps * 32 * 8 * 16 : 0) + (CHECK ? (size_t)kWarps * 32 * 8 * 4 : 0) + rows * 12;
 }
 
 // One CTA: SM x SN warps (at most 16), each a 16 x 16 block of C over k in its K slice; the SM strips of
@@ -139,24 +240,27 @@ constexpr size_t digit_smem() {
 // tensor pipe alone (86 mma.sync of two clocks per warp and 16 k) would take 69: with four warps per
 // scheduler and a barrier per 16 k, neither phase fills its pipe.  Strips past the end of C skip their
 // products.
-template <bool TA, bool TB, int ND>
+template <bool TA, bool TB, int ND, bool CHECK>
 __global__ void __launch_bounds__(kWarps * 32, 1)
     digit_gemm_kernel(int M, int N, int K, int kslice, int SM, int SN, const double *__restrict__ A, int lda,
-                      const double *__restrict__ B, int ldb, const int *__restrict__ ex, double alpha, double beta,
-                      double *__restrict__ C, int ldc, double *__restrict__ part) {
+                      const double *__restrict__ B, int ldb, const int *__restrict__ ex,
+                      const float *__restrict__ rsum, double alpha, double beta, double *__restrict__ C, int ldc,
+                      double *__restrict__ part, float *__restrict__ part_s) {
+  constexpr int kRows = 16 * kMaxStrips<CHECK>;
   extern __shared__ __align__(16) unsigned char smem[];
   double *raw = reinterpret_cast<double *>(smem);                                  // [2][rows][kRawStride]
   __nv_bfloat16 *dig = reinterpret_cast<__nv_bfloat16 *>(raw + 2 * kRows * kRawStride);  // [2][ND][rows][kDigStride]
   longlong2 *sums = reinterpret_cast<longlong2 *>(dig + (size_t)2 * ND * kRows * kDigStride);  // [8][512] (ND = 8)
-  double *rscale = reinterpret_cast<double *>(reinterpret_cast<unsigned char *>(sums) +
-                                              (ND == 8 ? (size_t)kWarps * 32 * 8 * 16 : 0));
+  float4 *mags = reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(sums) +
+                                            (ND == 8 ? (size_t)kWarps * 32 * 8 * 16 : 0));  // [2][512] (CHECK): S
+  double *rscale = reinterpret_cast<double *>(mags + (CHECK ? 2 * kWarps * 32 : 0));
   int *rexp = reinterpret_cast<int *>(rscale + kRows);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rows_a = 16 * SM, rows = 16 * (SM + SN);
   const int m0 = blockIdx.y * rows_a, n0 = blockIdx.x * 16 * SN;
   const int kbeg = blockIdx.z * kslice, kend = min(K, kbeg + kslice);
-  __shared__ int tiny;
-  if (tid == 0) tiny = 0;
+  __shared__ int tiny, nweak;
+  if (tid == 0) tiny = nweak = 0;
   __syncthreads();
   for (int r = tid; r < rows; r += blockDim.x) {
     const bool a = r < rows_a;
@@ -210,6 +314,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1)
 #pragma unroll
     for (int o = 0; o < 8; ++o) one[o] = 0;
   }
+  if constexpr (CHECK) mags[tid] = mags[kWarps * 32 + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
   constexpr unsigned kBuffer = ND * kPlane;
   // FP64 -> digits, two k per thread and step
   auto rewrite = [&](int buf) {
@@ -251,6 +356,31 @@ __global__ void __launch_bounds__(kWarps * 32, 1)
       for (int s = 0; s < ND && s + t < NG; ++s) {
         mma16816(acc[s + t][0], a[s], b[0], b[1]);
         mma16816(acc[s + t][1], a[s], b[2], b[3]);
+      }
+    }
+    if constexpr (CHECK) {
+      // |x| as BF16 from the first two digits, in units of the leading one
+      auto magnitude = [](unsigned (&r)[4], unsigned addr) {
+        unsigned d[4];
+        ldmatrix4(r, addr);
+        ldmatrix4(d, addr + kPlane);
+        const __nv_bfloat162 w = __float2bfloat162_rn(0.0078125f);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const __nv_bfloat162 x = __hfma2(*reinterpret_cast<const __nv_bfloat162 *>(&d[i]), w,
+                                           *reinterpret_cast<const __nv_bfloat162 *>(&r[i]));
+          r[i] = *reinterpret_cast<const unsigned *>(&x) & 0x7fff7fffu;
+        }
+      };
+      unsigned am[4], bm[4];
+      magnitude(am, a_addr + buf * kBuffer);
+      magnitude(bm, b_addr + buf * kBuffer);
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        float4 &m = mags[t * (kWarps * 32) + tid];
+        float d[4] = {m.x, m.y, m.z, m.w};
+        mma16816(d, am, bm[2 * t], bm[2 * t + 1]);
+        m = make_float4(d[0], d[1], d[2], d[3]);
       }
     }
   };
@@ -301,18 +431,22 @@ __global__ void __launch_bounds__(kWarps * 32, 1)
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
   }
-  if (!active) return;
+  if constexpr (!CHECK)
+    if (!active) return;
   if (part) part += (long)blockIdx.z * M * N;
+  if (CHECK && part) part_s += (long)blockIdx.z * M * N;
+  int *list = reinterpret_cast<int *>(raw);  // (CHECK) outputs of the tile to be summed in FP64
 #pragma unroll
   for (int t = 0; t < 2; ++t)
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
+      if (CHECK && !active) continue;
       const int m = m0 + 16 * wm + (lane >> 2) + (i >> 1) * 8;
       const int n = n0 + 16 * wn + t * 8 + (lane & 3) * 2 + (i & 1);
       if (m >= M || n >= N) continue;
       const int ea = ex[m], eb = ex[M + n];
       double v;
-      if (ea == kBadExp || eb == kBadExp) {
+      if (!CHECK && (ea == kBadExp || eb == kBadExp)) {
         // infinities and NaN follow the plain FP64 sum
         v = 0.0;
         for (int k = kbeg; k < kend; ++k)
@@ -325,20 +459,95 @@ __global__ void __launch_bounds__(kWarps * 32, 1)
         // group g weighs 128^(6 - g) of 2^(ea + eb - 54)
         v = ldexp((double)one[t * 4 + i], ea + eb - 54 + 14);
       }
+      float S = 0.f;
+      if constexpr (CHECK) {
+        const float4 q = mags[t * (kWarps * 32) + tid];
+        S = (i == 0 ? q.x : i == 1 ? q.y : i == 2 ? q.z : q.w) * 0x1p-12f;  // leading digits weigh 2^-6
+      }
       if (part) {
         part[(long)m * N + n] = v;
+        if (CHECK) part_s[(long)m * N + n] = S;
+      } else if (CHECK && weak(ea, eb, rsum[m], rsum[M + n], K, S)) {
+        list[atomicAdd(&nweak, 1)] = (m - m0) << 16 | (n - n0);
       } else {
         double *c = C + (long)m * ldc + n;
         *c = beta == 0.0 ? alpha * v : alpha * v + beta * (*c);
       }
     }
+  if constexpr (CHECK) {
+    if (part) return;
+    __syncthreads();
+    if (nweak > kFewWeak) {
+      // rows and columns of the tile through shared memory, up to eight listed outputs per thread
+      double *stage = raw + kWarps * 32 * 8 / 2;  // after the list: [rows][kStageK + 1]
+      auto fill = [&](const double *X, bool across, int ld, int x0, int rows_x, int n_x, double *dst, int k0) {
+        for (int e = tid; e < rows_x * kStageK; e += kWarps * 32) {
+          const int r = across ? e % rows_x : e / kStageK, k = across ? e / rows_x : e % kStageK;
+          const bool ok = x0 + r < n_x && k0 + k < K;
+          dst[r * (kStageK + 1) + k] =
+              ok ? __ldg(X + (across ? (long)(k0 + k) * ld + x0 + r : (long)(x0 + r) * ld + k0 + k)) : 0.0;
+        }
+      };
+      double v[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = 0.0;
+      for (int k0 = 0; k0 < K; k0 += kStageK) {
+        fill(A, TA, lda, m0, rows_a, M, stage, k0);
+        fill(B, !TB, ldb, n0, rows - rows_a, N, stage + rows_a * (kStageK + 1), k0);
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int q = tid + j * kWarps * 32;
+          if (q < nweak) {
+            const double *x = stage + (list[q] >> 16) * (kStageK + 1);
+            const double *y = stage + (rows_a + (list[q] & 0xffff)) * (kStageK + 1);
+#pragma unroll 8
+            for (int k = 0; k < kStageK; ++k) v[j] = fma(x[k], y[k], v[j]);
+          }
+        }
+        __syncthreads();
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int q = tid + j * kWarps * 32;
+        if (q < nweak) {
+          double *c = C + (long)(m0 + (list[q] >> 16)) * ldc + n0 + (list[q] & 0xffff);
+          *c = beta == 0.0 ? alpha * v[j] : alpha * v[j] + beta * (*c);
+        }
+      }
+      return;
+    }
+    for (int q = warp; q < nweak; q += kWarps) {
+      const int m = m0 + (list[q] >> 16), n = n0 + (list[q] & 0xffff);
+      const double v = warp_dot(TA ? A + m : A + (long)m * lda, TA ? lda : 1, TB ? B + (long)n * ldb : B + n,
+                                TB ? 1 : ldb, K);
+      if (lane == 0) {
+        double *c = C + (long)m * ldc + n;
+        *c = beta == 0.0 ? alpha * v : alpha * v + beta * (*c);
+      }
+    }
+  }
 }
 
+// op(A) and op(B) of a CHECK launch as strided rows: element (m, k) at A[m am + k ak], (k, n) at B[n bn + k bk]
+struct Operands {
+  const double *A, *B;
+  long am, ak, bn, bk;
+  const int *ex;
+  const float *rsum, *part_s;
+  int K;
+};
+
 // C = alpha sum_z part[z] + beta C: 32 outputs per CTA, the slices dealt to eight warps and their sums added
-// in order (as one thread per output, 44 x 216 outputs of 30 slices took 9 us, now 3)
+// in order (as one thread per output, 44 x 216 outputs of 30 slices took 9 us, now 3).  CHECK: S is added
+// likewise, and the weak outputs are dealt to the warps for an FP64 sum.
+template <bool CHECK>
 __global__ void __launch_bounds__(256) digit_reduce(int M, int N, int nsplit, const double *__restrict__ part,
-                                                    double alpha, double beta, double *__restrict__ C, int ldc) {
+                                                    double alpha, double beta, double *__restrict__ C, int ldc,
+                                                    Operands op) {
   __shared__ double red[8][33];
+  __shared__ float sred[CHECK ? 8 : 1][33];
+  __shared__ unsigned todo;
   const long total = (long)M * N;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long i = blockIdx.x * 32L + lane;
@@ -347,11 +556,43 @@ __global__ void __launch_bounds__(256) digit_reduce(int M, int N, int nsplit, co
 #pragma unroll 4
     for (int z = warp; z < nsplit; z += 8) s += __ldg(&part[(long)z * total + i]);
   red[warp][lane] = s;
+  float S = 0.f;
+  if constexpr (CHECK) {
+    if (i < total)
+#pragma unroll 4
+      for (int z = warp; z < nsplit; z += 8) S += __ldg(&op.part_s[(long)z * total + i]);
+    sred[warp][lane] = S;
+  }
   __syncthreads();
-  if (warp == 0 && i < total) {
-    for (int w = 1; w < 8; ++w) s += red[w][lane];
-    double *c = C + (i / N) * ldc + (i % N);
-    *c = beta == 0.0 ? alpha * s : alpha * s + beta * (*c);
+  if (warp == 0) {
+    bool again = false;
+    if (CHECK && i < total) {
+      for (int w = 1; w < 8; ++w) S += sred[w][lane];
+      const int m = (int)(i / N), n = M + (int)(i % N);
+      again = weak(op.ex[m], op.ex[n], op.rsum[m], op.rsum[n], op.K, S);
+    }
+    if (CHECK) {
+      const unsigned all = __ballot_sync(0xffffffffu, again);
+      if (lane == 0) todo = all;
+    }
+    if (i < total && !again) {
+      for (int w = 1; w < 8; ++w) s += red[w][lane];
+      double *c = C + (i / N) * ldc + (i % N);
+      *c = beta == 0.0 ? alpha * s : alpha * s + beta * (*c);
+    }
+  }
+  if constexpr (CHECK) {
+    __syncthreads();
+    int q = 0;
+    for (unsigned left = todo; left; left &= left - 1, ++q) {
+      if ((q & 7) != warp) continue;
+      const long o = blockIdx.x * 32L + __ffs(left) - 1, m = o / N, n = o % N;
+      const double v = warp_dot(op.A + m * op.am, op.ak, op.B + n * op.bn, op.bk, op.K);
+      if (lane == 0) {
+        double *c = C + m * ldc + n;
+        *c = beta == 0.0 ? alpha * v : alpha * v + beta * (*c);
+      }
+    }
   }
 }
 
@@ -361,7 +602,7 @@ __global__ void __launch_bounds__(256) digit_reduce(int M, int N, int nsplit, co
 struct Shape {
   int sm, sn, kslice, nsplit;
 };
-Shape choose(int M, int N, int K, int nd, size_t part_cap) {
+Shape choose(int M, int N, int K, int nd, size_t part_cap, int strips) {
   static const int opts[][2] = {{4, 4}, {5, 3}, {3, 5}, {2, 7}, {7, 2}, {6, 2}, {2, 6}, {3, 3}, {2, 4}, {4, 2}, {2, 2},
                                 {1, 8}, {8, 1}, {1, 4}, {4, 1}, {1, 1}};
   const int ms = (M + 15) / 16, ns = (N + 15) / 16;
@@ -370,7 +611,7 @@ Shape choose(int M, int N, int K, int nd, size_t part_cap) {
   double bc = 1e300;
   for (auto &o : opts) {
     const int sm = o[0], sn = o[1];
-    if (sm > ms + 1 || sn > ns + 1) continue;
+    if (sm > ms + 1 || sn > ns + 1 || sm + sn > strips) continue;
     const long tiles = (long)((ms + sm - 1) / sm) * ((ns + sn - 1) / sn);
     const double load = std::max(240.0 * (sm + sn), per_warp * std::min(sm, ms) * std::min(sn, ns)) + 500.0;
     // a slice of at most kMaxSlice k keeps the 64-bit sums in range (2^50 per 128 k)
@@ -393,22 +634,25 @@ Shape choose(int M, int N, int K, int nd, size_t part_cap) {
   return best;
 }
 
-template <bool TA, bool TB, int ND>
+template <bool TA, bool TB, int ND, bool CHECK>
 void go(dim3 grid, cudaStream_t s, int M, int N, int K, const Shape &h, const double *A, int lda, const double *B,
-        int ldb, const int *ex, double alpha, double beta, double *C, int ldc, double *part) {
-  BSE_CUDA(cudaFuncSetAttribute(digit_gemm_kernel<TA, TB, ND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)digit_smem<ND>()));
-  digit_gemm_kernel<TA, TB, ND><<<grid, kWarps * 32, digit_smem<ND>(), s>>>(M, N, K, h.kslice, h.sm, h.sn, A, lda, B,
-                                                                           ldb, ex, alpha, beta, C, ldc, part);
+        int ldb, const int *ex, const float *rsum, double alpha, double beta, double *C, int ldc, double *part,
+        float *part_s) {
+  constexpr size_t smem = digit_smem<ND, CHECK>();
+  auto kernel = digit_gemm_kernel<TA, TB, ND, CHECK>;
+  BSE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  kernel<<<grid, kWarps * 32, smem, s>>>(M, N, K, h.kslice, h.sm, h.sn, A, lda, B, ldb, ex, rsum, alpha, beta, C, ldc,
+                                         part, part_s);
   BSE_CHECK_LAUNCH();
 }
 
-template <int ND>
+template <int ND, bool CHECK>
 void run(char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda, const double *B, int ldb,
          double beta, double *C, int ldc, cudaStream_t s, DevBuf<double> &scratch, bool fixed, int split_pct) {
-  const size_t nex = ((size_t)M + N + 1) / 2;  // exponents, in doubles, ahead of the partial sums
+  // exponents (and the row sums of CHECK, at one float each) in doubles, ahead of the partial sums
+  const size_t nex = CHECK ? (size_t)M + N : ((size_t)M + N + 1) / 2;
   const size_t cap = fixed ? (scratch.n > nex ? scratch.n - nex : 0) : (size_t)1 << 26;
-  Shape h = choose(M, N, K, ND, cap);
+  Shape h = choose(M, N, K, ND, cap, kMaxStrips<CHECK>);
   if (split_pct != 100) {
     // the autotuner's variation of the number of K slices
     const int chunks = (K + kKC - 1) / kKC;
@@ -419,22 +663,30 @@ void run(char ta, char tb, int M, int N, int K, double alpha, const double *A, i
     h.kslice = per * kKC;
     h.nsplit = (chunks + per - 1) / per;
   }
-  if (!fixed) scratch.alloc(nex + (h.nsplit > 1 ? (size_t)h.nsplit * M * N : 0));
+  const long total = (long)M * N;
+  const size_t npart = h.nsplit > 1 ? (size_t)h.nsplit * total : 0;
+  if (!fixed) scratch.alloc(nex + npart + (CHECK ? (npart + 1) / 2 : 0));
   int *ex = reinterpret_cast<int *>(scratch.get());
-  double *part = h.nsplit > 1 ? scratch.get() + nex : nullptr;
+  float *rsum = CHECK ? reinterpret_cast<float *>(ex + M + N) : nullptr;
+  double *part = npart ? scratch.get() + nex : nullptr;
+  float *part_s = CHECK && npart ? reinterpret_cast<float *>(part + npart) : nullptr;
   const bool TA = ta == 'T', TB = tb == 'T';
   const int ba = TA ? (M + 31) / 32 : M, bb = TB ? N : (N + 31) / 32;
-  row_exponents<<<ba + bb, 256, 0, s>>>(M, N, K, TA, A, lda, !TB, B, ldb, ba, ex);
+  row_exponents<CHECK><<<ba + bb, 256, 0, s>>>(M, N, K, TA, A, lda, !TB, B, ldb, ba, ex, rsum);
   BSE_CHECK_LAUNCH();
   const dim3 grid((unsigned)((N + 16 * h.sn - 1) / (16 * h.sn)), (unsigned)((M + 16 * h.sm - 1) / (16 * h.sm)),
                   (unsigned)h.nsplit);
-  if (!TA && !TB) go<false, false, ND>(grid, s, M, N, K, h, A, lda, B, ldb, ex, alpha, beta, C, ldc, part);
-  else if (!TA && TB) go<false, true, ND>(grid, s, M, N, K, h, A, lda, B, ldb, ex, alpha, beta, C, ldc, part);
-  else if (TA && !TB) go<true, false, ND>(grid, s, M, N, K, h, A, lda, B, ldb, ex, alpha, beta, C, ldc, part);
-  else go<true, true, ND>(grid, s, M, N, K, h, A, lda, B, ldb, ex, alpha, beta, C, ldc, part);
+  auto launch = [&](auto a, auto b) {
+    go<decltype(a)::value, decltype(b)::value, ND, CHECK>(grid, s, M, N, K, h, A, lda, B, ldb, ex, rsum, alpha, beta, C,
+                                                          ldc, part, part_s);
+  };
+  if (!TA && !TB) launch(std::false_type(), std::false_type());
+  else if (!TA && TB) launch(std::false_type(), std::true_type());
+  else if (TA && !TB) launch(std::true_type(), std::false_type());
+  else launch(std::true_type(), std::true_type());
   if (part) {
-    const long total = (long)M * N;
-    digit_reduce<<<(unsigned)((total + 31) / 32), 256, 0, s>>>(M, N, h.nsplit, part, alpha, beta, C, ldc);
+    const Operands op{A, B, TA ? 1 : lda, TA ? lda : 1, TB ? ldb : 1, TB ? 1 : ldb, ex, rsum, part_s, K};
+    digit_reduce<CHECK><<<(unsigned)((total + 31) / 32), 256, 0, s>>>(M, N, h.nsplit, part, alpha, beta, C, ldc, op);
     BSE_CHECK_LAUNCH();
   }
 }
@@ -448,9 +700,11 @@ size_t digit_scratch(int M, int N, int K) {
 
 void digit_gemm(int digits, char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda,
                 const double *B, int ldb, double beta, double *C, int ldc, cudaStream_t s, DevBuf<double> &scratch,
-                bool fixed, int split_pct) {
-  if (digits == 8) run<8>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, scratch, fixed, split_pct);
-  else run<4>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, scratch, fixed, split_pct);
+                bool fixed, int split_pct, bool entrywise) {
+  if (digits != 8) run<4, false>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, scratch, fixed, split_pct);
+  else if (entrywise)
+    run<8, true>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, scratch, fixed, split_pct);
+  else run<8, false>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, scratch, fixed, split_pct);
 }
 
 }  // namespace bse

@@ -114,10 +114,12 @@ void fft3d_noalloc(int n1, int n2, int n3, int batch, double2 *data, int dir, cu
 //   'N' op(B) = B [K][N]; 'T' op(B) = B^T with B stored [N][K]
 // fixed: split-K partials go to this buffer, which is never resized (the split is clamped to
 // it); the default is a per-thread buffer that grows on demand.  split_pct scales the number of
-// K slices the heuristic picks (a tunable of the autotuner; 100 = the heuristic)
+// K slices the heuristic picks (a tunable of the autotuner; 100 = the heuristic).  Errors are those of an FP64
+// sum for whole rows and columns (relative to max |row of A| max |column of B|); with entrywise (not with fixed)
+// for every output on its own, whatever the grading of rows and columns (digit_gemm.cu)
 void dgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda,
            const double *B, int ldb, double beta, double *C, int ldc, cudaStream_t s,
-           DevBuf<double> *fixed = nullptr, int split_pct = 100);
+           DevBuf<double> *fixed = nullptr, int split_pct = 100, bool entrywise = false);
 // FP32 SIMT GEMM with FP32 accumulation (same conventions)
 void sgemm(char ta, char tb, int M, int N, int K, float alpha, const float *A, int lda,
            const float *B, int ldb, float beta, float *C, int ldc, cudaStream_t s,
@@ -128,10 +130,10 @@ void mgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A,
            double beta, double *C, int ldc, cudaStream_t s, int split_pct = 100);
 // the same product from exact BF16 digit products on the tensor pipe (digit_gemm.cu): digits = 8 for
 // FP64 results, 4 where dgemm's callers ask for FP32 arithmetic.  scratch: row exponents and split-K
-// partial sums, grown on demand unless fixed
+// partial sums, grown on demand unless fixed (not fixed with entrywise, digits = 8: see dgemm)
 void digit_gemm(int digits, char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda,
                 const double *B, int ldb, double beta, double *C, int ldc, cudaStream_t s, DevBuf<double> &scratch,
-                bool fixed, int split_pct = 100);
+                bool fixed, int split_pct = 100, bool entrywise = false);
 size_t digit_scratch(int M, int N, int K);  // the least scratch, in doubles
 // out[i] = sum_j X[i][j] * Y[i][j] for i < rows (part: scratch of the partial sums; the default is
 // a per-thread buffer)

@@ -402,7 +402,7 @@ void skinny_launch(int N, int K, const double *A, int lda, const double *B, int 
 
 void dgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda,
            const double *B, int ldb, double beta, double *C, int ldc, cudaStream_t s, DevBuf<double> *fixed,
-           int split_pct) {
+           int split_pct, bool entrywise) {
   if (M <= 0 || N <= 0) return;
   if (K <= 0) {
     if (beta != 1.0) {
@@ -476,7 +476,8 @@ void dgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A,
     return;
   }
   const bool fits = fixed && fixed->n >= digit_scratch(M, N, K);
-  digit_gemm(8, ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, fits ? *fixed : splitk_buf(), fits, split_pct);
+  digit_gemm(8, ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, fits ? *fixed : splitk_buf(), fits, split_pct,
+             entrywise);
 }
 
 void mgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda, const double *B, int ldb,

@@ -257,8 +257,9 @@ __global__ void __launch_bounds__(kWarps * 32, 1)
   int *rexp = reinterpret_cast<int *>(rscale + kRows);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rows_a = 16 * SM, rows = 16 * (SM + SN);
-  const int m0 = blockIdx.y * rows_a, n0 = blockIdx.x * 16 * SN;
-  const int kbeg = blockIdx.z * kslice, kend = min(K, kbeg + kslice);
+  const int ntx = (N + 16 * SN - 1) / (16 * SN);
+  const int m0 = blockIdx.x / ntx * rows_a, n0 = blockIdx.x % ntx * 16 * SN;
+  const int kbeg = blockIdx.y * kslice, kend = min(K, kbeg + kslice);
   __shared__ int tiny, nweak;
   if (tid == 0) tiny = nweak = 0;
   __syncthreads();
@@ -433,8 +434,8 @@ __global__ void __launch_bounds__(kWarps * 32, 1)
   }
   if constexpr (!CHECK)
     if (!active) return;
-  if (part) part += (long)blockIdx.z * M * N;
-  if (CHECK && part) part_s += (long)blockIdx.z * M * N;
+  if (part) part += (long)blockIdx.y * M * N;
+  if (CHECK && part) part_s += (long)blockIdx.y * M * N;
   int *list = reinterpret_cast<int *>(raw);  // (CHECK) outputs of the tile to be summed in FP64
 #pragma unroll
   for (int t = 0; t < 2; ++t)
@@ -674,8 +675,9 @@ void run(char ta, char tb, int M, int N, int K, double alpha, const double *A, i
   const int ba = TA ? (M + 31) / 32 : M, bb = TB ? N : (N + 31) / 32;
   row_exponents<CHECK><<<ba + bb, 256, 0, s>>>(M, N, K, TA, A, lda, !TB, B, ldb, ba, ex, rsum);
   BSE_CHECK_LAUNCH();
-  const dim3 grid((unsigned)((N + 16 * h.sn - 1) / (16 * h.sn)), (unsigned)((M + 16 * h.sm - 1) / (16 * h.sm)),
-                  (unsigned)h.nsplit);
+  // tiles along x: y and z end at 65535, which tiles of 32 to 48 rows pass at two to three million rows
+  const long tiles = (long)((N + 16 * h.sn - 1) / (16 * h.sn)) * ((M + 16 * h.sm - 1) / (16 * h.sm));
+  const dim3 grid((unsigned)tiles, (unsigned)h.nsplit);
   auto launch = [&](auto a, auto b) {
     go<decltype(a)::value, decltype(b)::value, ND, CHECK>(grid, s, M, N, K, h, A, lda, B, ldb, ex, rsum, alpha, beta, C,
                                                           ldc, part, part_s);

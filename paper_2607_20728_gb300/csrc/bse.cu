@@ -1011,7 +1011,7 @@ struct DavSpec {
   std::function<void(int, const double *, double *)> apply;
   std::function<void(int, double *, const double *)> precond;  // (k, T in/out, theta_dev)
   std::function<void(int, double *)> project;
-  bool fp32 = false;  // subspace products in FP32 (FP32-level tolerances only)
+  bool fp32 = false;  // FP32-grid operator: rank thresholds of FP32-level tolerances
   int keep = 0;       // Ritz vectors kept at a restart (0: block)
 };
 struct DavOut {
@@ -1020,16 +1020,12 @@ struct DavOut {
   bool converged = false;
 };
 
-// C = alpha op(A) op(B) + beta C.  With fp32 the product is taken in FP32 (operands rounded,
-// FP32 accumulation) and only the update is FP64: the subspace arithmetic of the ground-state
-// chunks that are converged with the FP32-grid Hamiltonian to FP32-level tolerances.
-void gemm_p(Ctx &c, bool fp32, char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda,
-            const double *B, int ldb, double beta, double *C, int ldc) {
-  if (!fp32 || M <= 0 || N <= 0 || K <= 0) {
-    dgemm(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, c.stream);
-    return;
-  }
-  mgemm(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, c.stream);
+// C = alpha op(A) op(B) + beta C on the context's stream.  The mixed form takes its subspace products in FP64
+// too: four digits (28 bits below a row's largest entry) instead of eight saved 0.7% of a mixed force evaluation
+// (63-well Hartree cell) and held entries below 2^-4 of the largest with less than FP32's 24 bits.
+void gemm_c(Ctx &c, char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda, const double *B,
+            int ldb, double beta, double *C, int ldc) {
+  dgemm(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, c.stream);
 }
 
 // W = L^-1 for the Cholesky factor G = L L^T of a symmetric positive definite n x n matrix
@@ -1087,17 +1083,17 @@ int orthonormalize(Ctx &c, long n, double *T, int kk, const double *V, int m, co
     // projection and through the Cholesky pivots (its loss of orthogonality is then a small
     // multiple of the rounding unit)
     if (m > 0) {
-      gemm_p(c, fp32, 'N', 'T', kk, m, (int)n, 1.0, T, (int)n, V, (int)n, 0.0, C.get(), m);
-      gemm_p(c, fp32, 'N', 'N', kk, (int)n, m, -1.0, C.get(), m, V, (int)n, 1.0, T, (int)n);
+      gemm_c(c, 'N', 'T', kk, m, (int)n, 1.0, T, (int)n, V, (int)n, 0.0, C.get(), m);
+      gemm_c(c, 'N', 'N', kk, (int)n, m, -1.0, C.get(), m, V, (int)n, 1.0, T, (int)n);
     }
     if (nq > 0) {
-      gemm_p(c, fp32, 'N', 'T', kk, nq, (int)n, 1.0, T, (int)n, Q, (int)n, 0.0, C.get(), nq);
-      gemm_p(c, fp32, 'N', 'N', kk, (int)n, nq, -1.0, C.get(), nq, Q, (int)n, 1.0, T, (int)n);
+      gemm_c(c, 'N', 'T', kk, nq, (int)n, 1.0, T, (int)n, Q, (int)n, 0.0, C.get(), nq);
+      gemm_c(c, 'N', 'N', kk, (int)n, nq, -1.0, C.get(), nq, Q, (int)n, 1.0, T, (int)n);
     }
     // symmetric orthonormalisation, dropping directions with relative norm below 1e-9 (1e-5 when
     // the Gram matrix is FP32: below that its eigenvectors are rounding noise)
     std::vector<double> G((size_t)kk * kk), w(kk), U((size_t)kk * kk);
-    gemm_p(c, fp32, 'N', 'T', kk, kk, (int)n, 1.0, T, (int)n, T, (int)n, 0.0, C.get(), kk);
+    gemm_c(c, 'N', 'T', kk, kk, (int)n, 1.0, T, (int)n, T, (int)n, 0.0, C.get(), kk);
     d2h(G.data(), C.get(), G.size() * sizeof(double), c);
     std::vector<double> Wm;
     int kept = 0;
@@ -1129,7 +1125,7 @@ int orthonormalize(Ctx &c, long n, double *T, int kk, const double *V, int m, co
     }
     if (kept == 0) return 0;
     h2d(C.get(), Wm.data(), Wm.size() * sizeof(double), c);
-    gemm_p(c, fp32, 'N', 'N', kept, (int)n, kk, 1.0, C.get(), kk, T, (int)n, 0.0, tmp.get(), (int)n);
+    gemm_c(c, 'N', 'N', kept, (int)n, kk, 1.0, C.get(), kk, T, (int)n, 0.0, tmp.get(), (int)n);
     d2d(T, tmp.get(), (size_t)kept * n * sizeof(double), c);
     kk = kept;
     ref = 1.0;
@@ -1167,7 +1163,7 @@ DavOut davidson(Ctx &c, const DavSpec &sp, const double *X0, int k0, double *Xou
   // symmetric on the P_c space), the new-new block is symmetrised
   auto grow = [&](int m0, int m1) {
     const int k = m1 - m0;
-    gemm_p(c, sp.fp32, 'N', 'T', k, m1, (int)n, 1.0, V.get() + (size_t)m0 * n, (int)n, AV.get(), (int)n, 0.0,
+    gemm_c(c, 'N', 'T', k, m1, (int)n, 1.0, V.get() + (size_t)m0 * n, (int)n, AV.get(), (int)n, 0.0,
            small.get(), m1);
     Hn.resize((size_t)k * m1);
     d2h(Hn.data(), small.get(), Hn.size() * sizeof(double), c);
@@ -1208,8 +1204,8 @@ DavOut davidson(Ctx &c, const DavSpec &sp, const double *X0, int k0, double *Xou
     for (int j = 0; j < m; ++j)
       for (int r = 0; r < nb; ++r) Yb[(size_t)j * nb + r] = Y[(size_t)j * m + r];
     h2d(small.get(), Yb.data(), Yb.size() * sizeof(double), c);
-    gemm_p(c, sp.fp32, 'T', 'N', nb, (int)n, m, 1.0, small.get(), nb, V.get(), (int)n, 0.0, X.get(), (int)n);
-    gemm_p(c, sp.fp32, 'T', 'N', nb, (int)n, m, 1.0, small.get(), nb, AV.get(), (int)n, 0.0, AX.get(), (int)n);
+    gemm_c(c, 'T', 'N', nb, (int)n, m, 1.0, small.get(), nb, V.get(), (int)n, 0.0, X.get(), (int)n);
+    gemm_c(c, 'T', 'N', nb, (int)n, m, 1.0, small.get(), nb, AV.get(), (int)n, 0.0, AX.get(), (int)n);
     h2d(th.get(), w.data(), nb * sizeof(double), c);
     k::residual(nb, n, AX.get(), X.get(), th.get(), T.get(), c.stream);
     rowdot(nb, n, T.get(), T.get(), rn.get(), c.stream);
@@ -1256,8 +1252,8 @@ DavOut davidson(Ctx &c, const DavSpec &sp, const double *X0, int k0, double *Xou
         for (int j = 0; j < m; ++j)
           for (int r = 0; r < nk; ++r) Yb[(size_t)j * nk + r] = Y[(size_t)j * m + r];
         h2d(small.get(), Yb.data(), Yb.size() * sizeof(double), c);
-        gemm_p(c, sp.fp32, 'T', 'N', nk, (int)n, m, 1.0, small.get(), nk, V.get(), (int)n, 0.0, Xk.get(), (int)n);
-        gemm_p(c, sp.fp32, 'T', 'N', nk, (int)n, m, 1.0, small.get(), nk, AV.get(), (int)n, 0.0, AXk.get(),
+        gemm_c(c, 'T', 'N', nk, (int)n, m, 1.0, small.get(), nk, V.get(), (int)n, 0.0, Xk.get(), (int)n);
+        gemm_c(c, 'T', 'N', nk, (int)n, m, 1.0, small.get(), nk, AV.get(), (int)n, 0.0, AXk.get(),
                (int)n);
         d2d(V.get(), Xk.get(), (size_t)nk * n * sizeof(double), c);
         d2d(AV.get(), AXk.get(), (size_t)nk * n * sizeof(double), c);
@@ -2084,21 +2080,17 @@ struct PairPrecond {
     one.alloc(c.nocc);
     h2d(one.get(), v.data(), c.nocc * sizeof(double), c);
   }
-  // the products with the empty states run in FP32 in the mixed form (a preconditioner only
-  // changes the convergence rate, not the converged root; its FP64 products cost a quarter of a
-  // mixed Davidson iteration)
   void operator()(int kk, double *T, const double *th) {
     const long n = (long)c.nocc * c.npw;
     const int rows = kk * c.nocc;
-    const bool fp32 = c.prec == 1;
     if (ne > 0)
-      gemm_p(c, fp32, 'N', 'T', rows, ne, c.npw, 1.0, T, c.npw, c.empty.get(), c.npw, 0.0, Cb.get(), ne);
+      gemm_c(c, 'N', 'T', rows, ne, c.npw, 1.0, T, c.npw, c.empty.get(), c.npw, 0.0, Cb.get(), ne);
     k::precond_diag(kk, n, T, c.kin.get(), c.npw, one.get(), 0.0, th, 1e-3, T, c.stream);
     if (ne > 0) {
-      gemm_p(c, fp32, 'N', 'T', rows, ne, c.npw, 1.0, T, c.npw, c.empty.get(), c.npw, 0.0, Ckb.get(), ne);
+      gemm_c(c, 'N', 'T', rows, ne, c.npw, 1.0, T, c.npw, c.empty.get(), c.npw, 0.0, Ckb.get(), ne);
       k::subspace_den(rows, ne, c.nocc, Cb.get(), Ckb.get(), c.eps_empty_d.get(), c.eps.get(), c.scissor, th,
                       1e-6, Cb.get(), c.stream);
-      gemm_p(c, fp32, 'N', 'N', rows, c.npw, ne, 1.0, Cb.get(), ne, c.empty.get(), c.npw, 1.0, T, c.npw);
+      gemm_c(c, 'N', 'N', rows, c.npw, ne, 1.0, Cb.get(), ne, c.empty.get(), c.npw, 1.0, T, c.npw);
     }
   }
 };

@@ -24,10 +24,6 @@
 // magnitudes rounded to BF16, and the outputs it finds weak are dealt to whole warps, or summed together when a tile
 // has many.  Kernel time with CHECK (without): N T 80 x 216 x 6859 72 us (67), N N 80 x 2400 x 64 23 (20), T N
 // 200 x 6859 x 128 114 (115); with every output weak 302, 54 and 419 (as tiled FP64 kernels 384, 69 and 391).
-//
-// With ND = 4 digits (28 bits, groups s + t <= 4) the same kernel serves the products whose contract is
-// FP32 arithmetic on FP64 operands: finer operands than FP32's 24 bits and exact sums, 13 products
-// instead of 43.
 #include <algorithm>
 #include <cstdint>
 #include <type_traits>
@@ -39,6 +35,7 @@
 namespace bse {
 namespace {
 
+constexpr int kND = 8;              // digits
 constexpr int kKC = 16;             // k per staged chunk
 constexpr int kRawStride = kKC + 2;  // doubles per staged row (16-byte aligned, rows off the same banks)
 constexpr int kDigStride = kKC + 8;  // bf16 per digit row: ldmatrix reads 8 rows without bank conflicts
@@ -52,24 +49,22 @@ constexpr int kMaxSlice = 1 << 19;  // longest K slice
 constexpr int kFewWeak = 64;        // weak outputs of a tile that go to one warp each
 constexpr int kStageK = 64;         // k at a time for more
 
-// |x| < 2^e  ->  round(x 2^(kBits - e)), kBits = 7 ND - 1
-template <int ND>
+// |x| < 2^e  ->  round(x 2^(55 - e))
 __device__ __forceinline__ long long to_fixed(double x, int e) {
   const long long b = __double_as_longlong(x);
   const int E = (int)((b >> 52) & 0x7ff);
   unsigned long long m = (unsigned long long)b & 0xfffffffffffffull;
   if (E) m |= 1ull << 52;
-  const int s = max(E, 1) - 1075 + (7 * ND - 1) - e;  // at most 2 for ND = 8
+  const int s = max(E, 1) - 1075 + (7 * kND - 1) - e;  // at most 2
   const int l = min(max(s, 0), 63), r = min(max(-s, 0), 63);  // (above 2: rows of denormals, or with infinities)
   m <<= l;
   m = (m + ((1ull << r) >> 1)) >> r;
   return b < 0 ? -(long long)m : (long long)m;
 }
 // sum over all digits of 64 * 128^j: makes every balanced digit a plain 7-bit field
-template <int ND>
 __device__ __forceinline__ constexpr unsigned long long digit_bias() {
   unsigned long long c = 0;
-  for (int j = 0; j < ND; ++j) c = c * 128 + 64;
+  for (int j = 0; j < kND; ++j) c = c * 128 + 64;
   return c;
 }
 
@@ -224,11 +219,11 @@ __device__ __forceinline__ double warp_dot(const double *__restrict__ a, long sa
   return s;
 }
 
-template <int ND, bool CHECK>
+template <bool CHECK>
 constexpr size_t digit_smem() {
   constexpr int rows = 16 * kMaxStrips<CHECK>;
-  return (size_t)2 * rows * kRawStride * 8 + (size_t)2 * ND * rows * kDigStride * 2 +
-         (ND == 8 ? (size_t)kWarps * 32 * 8 * 16 : 0) + (CHECK ? (size_t)kWarps * 32 * 8 * 4 : 0) + rows * 12;
+  return (size_t)2 * rows * kRawStride * 8 + (size_t)2 * kND * rows * kDigStride * 2 +
+         (size_t)kWarps * 32 * 8 * 16 + (CHECK ? (size_t)kWarps * 32 * 8 * 4 : 0) + rows * 12;
 }
 
 // One CTA: SM x SN warps (at most 16), each a 16 x 16 block of C over k in its K slice; the SM strips of
@@ -240,7 +235,7 @@ constexpr size_t digit_smem() {
 // tensor pipe alone (86 mma.sync of two clocks per warp and 16 k) would take 69: with four warps per
 // scheduler and a barrier per 16 k, neither phase fills its pipe.  Strips past the end of C skip their
 // products.
-template <bool TA, bool TB, int ND, bool CHECK>
+template <bool TA, bool TB, bool CHECK>
 __global__ void __launch_bounds__(kWarps * 32, 1)
     digit_gemm_kernel(int M, int N, int K, int kslice, int SM, int SN, const double *__restrict__ A, int lda,
                       const double *__restrict__ B, int ldb, const int *__restrict__ ex,
@@ -249,10 +244,9 @@ __global__ void __launch_bounds__(kWarps * 32, 1)
   constexpr int kRows = 16 * kMaxStrips<CHECK>;
   extern __shared__ __align__(16) unsigned char smem[];
   double *raw = reinterpret_cast<double *>(smem);                                  // [2][rows][kRawStride]
-  __nv_bfloat16 *dig = reinterpret_cast<__nv_bfloat16 *>(raw + 2 * kRows * kRawStride);  // [2][ND][rows][kDigStride]
-  longlong2 *sums = reinterpret_cast<longlong2 *>(dig + (size_t)2 * ND * kRows * kDigStride);  // [8][512] (ND = 8)
-  float4 *mags = reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(sums) +
-                                            (ND == 8 ? (size_t)kWarps * 32 * 8 * 16 : 0));  // [2][512] (CHECK): S
+  __nv_bfloat16 *dig = reinterpret_cast<__nv_bfloat16 *>(raw + 2 * kRows * kRawStride);  // [2][kND][rows][kDigStride]
+  longlong2 *sums = reinterpret_cast<longlong2 *>(dig + (size_t)2 * kND * kRows * kDigStride);  // [8][512]
+  float4 *mags = reinterpret_cast<float4 *>(sums + kWarps * 32 * 8);                       // [2][512] (CHECK): S
   double *rscale = reinterpret_cast<double *>(mags + (CHECK ? 2 * kWarps * 32 : 0));
   int *rexp = reinterpret_cast<int *>(rscale + kRows);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -269,7 +263,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1)
     if (g < (a ? M : N)) e = ex[a ? g : M + g];
     rexp[r] = e = e == kBadExp ? 0 : e;
     // 2^(kBits - e), rows of very small numbers (where that could overflow) converted by to_fixed
-    if (e > -900) rscale[r] = __longlong_as_double((long long)(1023 + 7 * ND - 1 - e) << 52);
+    if (e > -900) rscale[r] = __longlong_as_double((long long)(1023 + 7 * kND - 1 - e) << 52);
     else atomicOr(&tiny, 1);
   }
   // 8-byte copies of 32-row groups of each operand, consecutive threads along its contiguous direction: a
@@ -298,7 +292,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1)
   const unsigned b_addr =
       smem_addr(dig + (rows_a + 16 * wn + ((lane >> 4) << 3) + (lane & 7)) * kDigStride + ((lane >> 3) & 1) * 8);
   constexpr unsigned kPlane = kRows * kDigStride * 2;
-  constexpr int NG = ND + 1;  // digit-pair groups s + t = 0 .. ND
+  constexpr int NG = kND + 1;  // digit-pair groups s + t = 0 .. kND
   float acc[NG][2][4];
 #pragma unroll
   for (int g = 0; g < NG; ++g)
@@ -306,16 +300,10 @@ __global__ void __launch_bounds__(kWarps * 32, 1)
     for (int t = 0; t < 2; ++t)
 #pragma unroll
       for (int i = 0; i < 4; ++i) acc[g][t][i] = 0.f;
-  long long one[ND == 8 ? 1 : 8];  // ND = 4: a single 64-bit sum per output, in registers
-  if constexpr (ND == 8) {
 #pragma unroll
-    for (int o = 0; o < 8; ++o) sums[o * (kWarps * 32) + tid] = make_longlong2(0, 0);
-  } else {
-#pragma unroll
-    for (int o = 0; o < 8; ++o) one[o] = 0;
-  }
+  for (int o = 0; o < 8; ++o) sums[o * (kWarps * 32) + tid] = make_longlong2(0, 0);
   if constexpr (CHECK) mags[tid] = mags[kWarps * 32 + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
-  constexpr unsigned kBuffer = ND * kPlane;
+  constexpr unsigned kBuffer = kND * kPlane;
   // FP64 -> digits, two k per thread and step
   auto rewrite = [&](int buf) {
     for (int i = tid; i < rows * (kKC / 2); i += kWarps * 32) {
@@ -325,16 +313,16 @@ __global__ void __launch_bounds__(kWarps * 32, 1)
       if (!tiny) {
         // the scaling is exact and the conversion rounds to nearest: the FP64 pipe is free here
         const double sc = rscale[r];
-        y0 = (unsigned long long)__double2ll_rn(x.x * sc) + digit_bias<ND>();
-        y1 = (unsigned long long)__double2ll_rn(x.y * sc) + digit_bias<ND>();
+        y0 = (unsigned long long)__double2ll_rn(x.x * sc) + digit_bias();
+        y1 = (unsigned long long)__double2ll_rn(x.y * sc) + digit_bias();
       } else {
-        y0 = (unsigned long long)to_fixed<ND>(x.x, rexp[r]) + digit_bias<ND>();
-        y1 = (unsigned long long)to_fixed<ND>(x.y, rexp[r]) + digit_bias<ND>();
+        y0 = (unsigned long long)to_fixed(x.x, rexp[r]) + digit_bias();
+        y1 = (unsigned long long)to_fixed(x.y, rexp[r]) + digit_bias();
       }
       unsigned *d = reinterpret_cast<unsigned *>(dig + (size_t)buf * (kBuffer / 2) + r * kDigStride + 2 * kp);
 #pragma unroll
-      for (int s = 0; s < ND; ++s) {
-        const int sh = 7 * (ND - 1 - s);
+      for (int s = 0; s < kND; ++s) {
+        const int sh = 7 * (kND - 1 - s);
         // the leading field reaches 128; a 7-bit field u next to the BF16 bits of 128 reads 128 + u
         const unsigned msk = s == 0 ? 0xffu : 0x7fu;
         const unsigned hi = sh >= 16 ? (unsigned)(y1 >> (sh >= 16 ? sh - 16 : 0)) : (unsigned)(y1 << (sh < 16 ? 16 - sh : 0));
@@ -345,15 +333,15 @@ __global__ void __launch_bounds__(kWarps * 32, 1)
     }
   };
   auto multiply = [&](int buf) {
-    unsigned a[ND][4];
+    unsigned a[kND][4];
 #pragma unroll
-    for (int s = 0; s < ND; ++s) ldmatrix4(a[s], a_addr + buf * kBuffer + s * kPlane);
+    for (int s = 0; s < kND; ++s) ldmatrix4(a[s], a_addr + buf * kBuffer + s * kPlane);
 #pragma unroll
-    for (int t = 0; t < ND; ++t) {
+    for (int t = 0; t < kND; ++t) {
       unsigned b[4];
       ldmatrix4(b, b_addr + buf * kBuffer + t * kPlane);
 #pragma unroll
-      for (int s = 0; s < ND && s + t < NG; ++s) {
+      for (int s = 0; s < kND && s + t < NG; ++s) {
         mma16816(acc[s + t][0], a[s], b[0], b[1]);
         mma16816(acc[s + t][1], a[s], b[2], b[3]);
       }
@@ -417,15 +405,11 @@ __global__ void __launch_bounds__(kWarps * 32, 1)
             v[g] = __float_as_int(acc[g][t][i] + 12582912.f) - 0x4B400000;
             acc[g][t][i] = 0.f;
           }
-          if constexpr (ND == 8) {
-            longlong2 &s = sums[(t * 4 + i) * (kWarps * 32) + tid];
-            longlong2 x = s;
-            x.x += (((long long)v[0] * 128 + v[1]) * 128 + v[2]) * 128 + v[3];
-            x.y += ((((long long)v[4] * 128 + v[5]) * 128 + v[6]) * 128 + v[7]) * 128 + v[8];
-            s = x;
-          } else {
-            one[t * 4 + i] += ((((long long)v[0] * 128 + v[1]) * 128 + v[2]) * 128 + v[3]) * 128 + v[4];
-          }
+          longlong2 &s = sums[(t * 4 + i) * (kWarps * 32) + tid];
+          longlong2 x = s;
+          x.x += (((long long)v[0] * 128 + v[1]) * 128 + v[2]) * 128 + v[3];
+          x.y += ((((long long)v[4] * 128 + v[5]) * 128 + v[6]) * 128 + v[7]) * 128 + v[8];
+          s = x;
         }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -451,13 +435,10 @@ __global__ void __launch_bounds__(kWarps * 32, 1)
         v = 0.0;
         for (int k = kbeg; k < kend; ++k)
           v = fma(TA ? A[(long)k * lda + m] : A[(long)m * lda + k], TB ? B[(long)n * ldb + k] : B[(long)k * ldb + n], v);
-      } else if constexpr (ND == 8) {
+      } else {
         // group g weighs 128^(14 - g) of 2^(ea + eb - 110)
         const longlong2 s = sums[(t * 4 + i) * (kWarps * 32) + tid];
         v = ldexp(fma((double)s.x, 34359738368.0, (double)s.y), ea + eb - 110 + 42);
-      } else {
-        // group g weighs 128^(6 - g) of 2^(ea + eb - 54)
-        v = ldexp((double)one[t * 4 + i], ea + eb - 54 + 14);
       }
       float S = 0.f;
       if constexpr (CHECK) {
@@ -597,23 +578,21 @@ __global__ void __launch_bounds__(256) digit_reduce(int M, int N, int nsplit, co
 }
 
 // Strips per CTA and K slices: the fewest clocks by a model of one CTA per SM, a chunk of 16 k costing the
-// larger of its rewriting (240 clocks per strip) and its products (172 per active warp with ND = 8, 52 with
-// ND = 4) plus 500, a CTA 8000 more.
+// larger of its rewriting (240 clocks per strip) and its products (172 per active warp) plus 500, a CTA 8000 more.
 struct Shape {
   int sm, sn, kslice, nsplit;
 };
-Shape choose(int M, int N, int K, int nd, size_t part_cap, int strips) {
+Shape choose(int M, int N, int K, size_t part_cap, int strips) {
   static const int opts[][2] = {{4, 4}, {5, 3}, {3, 5}, {2, 7}, {7, 2}, {6, 2}, {2, 6}, {3, 3}, {2, 4}, {4, 2}, {2, 2},
                                 {1, 8}, {8, 1}, {1, 4}, {4, 1}, {1, 1}};
   const int ms = (M + 15) / 16, ns = (N + 15) / 16;
-  const double per_warp = nd == 8 ? 172.0 : 52.0;
   Shape best{4, 4, K, 1};
   double bc = 1e300;
   for (auto &o : opts) {
     const int sm = o[0], sn = o[1];
     if (sm > ms + 1 || sn > ns + 1 || sm + sn > strips) continue;
     const long tiles = (long)((ms + sm - 1) / sm) * ((ns + sn - 1) / sn);
-    const double load = std::max(240.0 * (sm + sn), per_warp * std::min(sm, ms) * std::min(sn, ns)) + 500.0;
+    const double load = std::max(240.0 * (sm + sn), 172.0 * std::min(sm, ms) * std::min(sn, ns)) + 500.0;
     // a slice of at most kMaxSlice k keeps the 64-bit sums in range (2^50 per 128 k)
     const int mins = (K + kMaxSlice - 1) / kMaxSlice;
     const int maxs = (int)std::max(mins, std::min(K / 64, 128));
@@ -634,25 +613,25 @@ Shape choose(int M, int N, int K, int nd, size_t part_cap, int strips) {
   return best;
 }
 
-template <bool TA, bool TB, int ND, bool CHECK>
+template <bool TA, bool TB, bool CHECK>
 void go(dim3 grid, cudaStream_t s, int M, int N, int K, const Shape &h, const double *A, int lda, const double *B,
         int ldb, const int *ex, const float *rsum, double alpha, double beta, double *C, int ldc, double *part,
         float *part_s) {
-  constexpr size_t smem = digit_smem<ND, CHECK>();
-  auto kernel = digit_gemm_kernel<TA, TB, ND, CHECK>;
+  constexpr size_t smem = digit_smem<CHECK>();
+  auto kernel = digit_gemm_kernel<TA, TB, CHECK>;
   BSE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   kernel<<<grid, kWarps * 32, smem, s>>>(M, N, K, h.kslice, h.sm, h.sn, A, lda, B, ldb, ex, rsum, alpha, beta, C, ldc,
                                          part, part_s);
   BSE_CHECK_LAUNCH();
 }
 
-template <int ND, bool CHECK>
+template <bool CHECK>
 void run(char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda, const double *B, int ldb,
          double beta, double *C, int ldc, cudaStream_t s, DevBuf<double> &scratch, bool fixed, int split_pct) {
   // exponents (and the row sums of CHECK, at one float each) in doubles, ahead of the partial sums
   const size_t nex = CHECK ? (size_t)M + N : ((size_t)M + N + 1) / 2;
   const size_t cap = fixed ? (scratch.n > nex ? scratch.n - nex : 0) : (size_t)1 << 26;
-  Shape h = choose(M, N, K, ND, cap, kMaxStrips<CHECK>);
+  Shape h = choose(M, N, K, cap, kMaxStrips<CHECK>);
   if (split_pct != 100) {
     // the autotuner's variation of the number of K slices
     const int chunks = (K + kKC - 1) / kKC;
@@ -667,8 +646,8 @@ void run(char ta, char tb, int M, int N, int K, double alpha, const double *A, i
     // row tiles lie along y, which ends there (with 32 or 48 rows at two to three million): in two halves.
     // Numbering all tiles along x made m0 and n0 the results of a division and every product 8% slower.
     const int m = M / 2;
-    run<ND, CHECK>(ta, tb, m, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, scratch, fixed, split_pct);
-    run<ND, CHECK>(ta, tb, M - m, N, K, alpha, A + (ta == 'T' ? m : (long)m * lda), lda, B, ldb, beta,
+    run<CHECK>(ta, tb, m, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, scratch, fixed, split_pct);
+    run<CHECK>(ta, tb, M - m, N, K, alpha, A + (ta == 'T' ? m : (long)m * lda), lda, B, ldb, beta,
                    C + (long)m * ldc, ldc, s, scratch, fixed, split_pct);
     return;
   }
@@ -686,7 +665,7 @@ void run(char ta, char tb, int M, int N, int K, double alpha, const double *A, i
   const dim3 grid((unsigned)((N + 16 * h.sn - 1) / (16 * h.sn)), (unsigned)((M + 16 * h.sm - 1) / (16 * h.sm)),
                   (unsigned)h.nsplit);
   auto launch = [&](auto a, auto b) {
-    go<decltype(a)::value, decltype(b)::value, ND, CHECK>(grid, s, M, N, K, h, A, lda, B, ldb, ex, rsum, alpha, beta, C,
+    go<decltype(a)::value, decltype(b)::value, CHECK>(grid, s, M, N, K, h, A, lda, B, ldb, ex, rsum, alpha, beta, C,
                                                           ldc, part, part_s);
   };
   if (!TA && !TB) launch(std::false_type(), std::false_type());
@@ -707,13 +686,11 @@ size_t digit_scratch(int M, int N, int K) {
   return ((size_t)M + N + 1) / 2 + (slices > 1 ? slices * M * N : 0);
 }
 
-void digit_gemm(int digits, char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda,
+void digit_gemm(char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda,
                 const double *B, int ldb, double beta, double *C, int ldc, cudaStream_t s, DevBuf<double> &scratch,
                 bool fixed, int split_pct, bool entrywise) {
-  if (digits != 8) run<4, false>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, scratch, fixed, split_pct);
-  else if (entrywise)
-    run<8, true>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, scratch, fixed, split_pct);
-  else run<8, false>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, scratch, fixed, split_pct);
+  if (entrywise) run<true>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, scratch, fixed, split_pct);
+  else run<false>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, scratch, fixed, split_pct);
 }
 
 }  // namespace bse

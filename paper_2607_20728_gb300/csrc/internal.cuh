@@ -124,14 +124,9 @@ void dgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A,
 void sgemm(char ta, char tb, int M, int N, int K, float alpha, const float *A, int lda,
            const float *B, int ldb, float beta, float *C, int ldc, cudaStream_t s,
            DevBuf<float> *fixed = nullptr, int split_pct = 100);
-// FP64 operands and output with products and sums no less exact than FP32's (same conventions as dgemm): four
-// BF16 digits of each operand, alpha, beta and the sum over K slices in FP64
-void mgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda, const double *B, int ldb,
-           double beta, double *C, int ldc, cudaStream_t s, int split_pct = 100);
-// the same product from exact BF16 digit products on the tensor pipe (digit_gemm.cu): digits = 8 for
-// FP64 results, 4 where dgemm's callers ask for FP32 arithmetic.  scratch: row exponents and split-K
-// partial sums, grown on demand unless fixed (not fixed with entrywise, digits = 8: see dgemm)
-void digit_gemm(int digits, char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda,
+// the same product from exact BF16 digit products on the tensor pipe (digit_gemm.cu).  scratch: row exponents
+// and split-K partial sums, grown on demand unless fixed (not fixed with entrywise: see dgemm)
+void digit_gemm(char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda,
                 const double *B, int ldb, double beta, double *C, int ldc, cudaStream_t s, DevBuf<double> &scratch,
                 bool fixed, int split_pct = 100, bool entrywise = false);
 size_t digit_scratch(int M, int N, int K);  // the least scratch, in doubles

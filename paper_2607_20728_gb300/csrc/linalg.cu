@@ -476,18 +476,8 @@ void dgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A,
     return;
   }
   const bool fits = fixed && fixed->n >= digit_scratch(M, N, K);
-  digit_gemm(8, ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, fits ? *fixed : splitk_buf(), fits, split_pct,
+  digit_gemm(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, fits ? *fixed : splitk_buf(), fits, split_pct,
              entrywise);
-}
-
-void mgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda, const double *B, int ldb,
-           double beta, double *C, int ldc, cudaStream_t s, int split_pct) {
-  if (M <= 0 || N <= 0) return;
-  if (K <= 0) {
-    dgemm(ta, tb, M, N, 0, alpha, A, lda, B, ldb, beta, C, ldc, s);
-    return;
-  }
-  digit_gemm(4, ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, s, splitk_buf(), false, split_pct);
 }
 
 void sgemm(char ta, char tb, int M, int N, int K, float alpha, const float *A, int lda, const float *B, int ldb,

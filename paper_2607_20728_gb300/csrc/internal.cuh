@@ -183,11 +183,11 @@ struct K1dTma {
   int *err = nullptr;                  // device flag set when a bounded wait gives up
   bool ready = false;
 };
-// FP64 K1d contraction in fixed point (k1d_fixed.cu): tau as integer limbs, tile-major, and the value of
-// one unit of it at every point
+// FP64 K1d contraction in fixed point (k1d_fixed.cu): tau as integer limbs, tile-major, and the scale of
+// every point
 struct K1dFixed {
   const int2 *tau = nullptr;
-  const double *scale = nullptr;       // [nr]
+  const double2 *scale = nullptr;      // [nr] (unit of the sums, bits of a)
   long npairs = 0;
   int *err = nullptr;                  // device flag set when a bounded wait gives up
   bool ready = false;
@@ -349,7 +349,7 @@ struct Ctx {
 
   K1dTma k1d;                  // FP32 K1d with TMA staging (mixed precision)
   K1dFixed k1x;                // FP64 K1d in fixed point (FP64 contexts)
-  DevBuf<double> tau_scale;    // [nr] its units
+  DevBuf<double2> tau_scale;   // [nr] its scales
   DevBuf<unsigned> tau_top;    // [nr] largest |tau| of each point (high word), while tau is built
   SplitBF16 pdep_split;        // PDEP rows x v_c^{1/2} (projection operand, mixed precision)
   SplitBF16 pdepT_split;       // their transpose (back-projection operand)
@@ -386,9 +386,9 @@ struct Ctx {
 bool k1d_fixed_supported(int nocc);
 size_t k1d_tiled_size(long npairs, long nr);  // elements of a tile-major tau
 // packed grids of np pair products -> tile-major doubles and the points' largest values (top, zeroed
-// before the first batch); after the last batch, doubles -> limbs in place and the units
+// before the first batch); after the last batch, doubles -> limbs in place and the scales
 void k1d_fixed_tile(const Ctx &c, int np, const int2 *pairs, const double2 *P, double *tau, unsigned *top);
-void k1d_fixed_finish(const Ctx &c, double *tau, const unsigned *top, double *scale);
+void k1d_fixed_finish(const Ctx &c, double *tau, const unsigned *top, double2 *scale);
 void k1d_fixed(const Ctx &c, const K1dFixed &t, int nb, const double *phir, const double *vloc, const double2 *Pa,
                const double2 *Pvh, double2 *Py, bool use_vloc, bool use_k1e);
 bool k1d_tma_supported(int nocc, long nr);

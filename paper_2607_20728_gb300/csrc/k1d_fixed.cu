@@ -7,11 +7,13 @@
 // tau is stored once per unordered pair as a 57-bit fixed-point number relative to the power of two
 // above max_pairs |tau(r)| of its point r, as two signed limbs of 27 bits below: t = th 2^27 + tl,
 // |th| <= 2^29, |tl| <= 2^26 (8 bytes, like the double it replaces).  a_v(r) is rounded the same way to
-// 54 bits below max_v |a_v(r)|, so the three products th ah, th al + tl ah (tl al is below 2^-57 of the
-// largest product) are integers whose sums over up to 128 orbitals stay below 2^63 and are exact; tau
-// has one bit less for up to 256 orbitals and two less for up to 512.  The sums are rounded to 2^-55 of
-// max|tau| max|a| as they are added to Y and to FP64 once at the end.  Against the FP64 sum (an error
-// of about 2^-53 of the running sum per term) the result is the more accurate one.
+// 53 + s bits below max_v |a_v(r)|, so the three products th ah, th al + tl ah (tl al is a quarter of the last
+// unit at most) are integers; s is a property of the point, as large as the 64-bit sums allow: with
+// C = max_v sum_v' |tau_v'v|, |sum| <= C max|a|, and C is far below N_occ max|tau| where the diagonal dominates.
+// The sums are rounded to 2^-(55 + s) of max|tau| max|a| as they are added to Y and to FP64 once at the end.
+// Error over a point's orbitals (2-norm, emulated), s = 0 and all N_occ terms at the maximum assumed -> this ->
+// an FP64 sum: 128 flat 1.6e-16 -> 0.3e-16 (3.6e-16), 128 with a dominant diagonal 6.3e-16 -> 2.1e-16 (3.8e-16),
+// 200 likewise 13e-16 -> 2.6e-16 (3.9e-16), orbitals of very different size 3.3e-16 -> 0.6e-16 (3.0e-16).
 //
 // Every tau element is read from memory once: a CTA owns 32 points (one per lane) and walks the columns
 // c of 8 orbitals; column c holds blocks of 16 rows x 8 orbitals below it (one of 8 rows when c is odd)
@@ -44,6 +46,7 @@ constexpr unsigned kStageBytes = kStageElems * 8;
 constexpr size_t kSmemCap = 227 * 1024;
 constexpr size_t kSmemHalf = 113 * 1024;  // two CTAs per SM
 constexpr int kMaxStages = 6;
+constexpr int kTauBits = 56;      // of tau below its point's power of two
 
 template <int W>
 __device__ __forceinline__ void consumers_sync() {
@@ -106,7 +109,7 @@ __device__ __forceinline__ int chunks_of(int c) { return c / 2 + (c & 1) + 1; }
 
 template <int NB, int W>
 __global__ void __launch_bounds__(W * 32 + 32, 16 / W) k1d_fixed_kernel(
-    const int2 *__restrict__ tau, const double *__restrict__ tscale, long npairs, long nr, int nocc, int nb_total,
+    const int2 *__restrict__ tau, const double2 *__restrict__ tscale, long npairs, long nr, int nocc, int nb_total,
     int b0, int stages, const double *__restrict__ phir, const double *__restrict__ vloc,
     const double *__restrict__ Pa, const double *__restrict__ Pvh, double *__restrict__ Py, int use_vloc, int use_k1e,
     int *__restrict__ err, int hold) {
@@ -183,8 +186,13 @@ __global__ void __launch_bounds__(W * 32 + 32, 16 / W) k1d_fixed_kernel(
   double x[NB][kKeep > 0 ? kKeep : 1];
   auto row = [&](int b, int v, long rr) { return b0 + b < nb_total ? __ldg(&Pa[at(b, v, rr)]) : 0.0; };
   auto point = [&](long t) { return min(t * kR + lane, nr - 1); };
+  // bits of a at the tile's point: with the rows for one vector and 16 warps (4.92 -> 4.82 ms at 128 orbitals), at
+  // the top of the tile otherwise (with the rows 48 orbitals take 125 and 192 us, so 124 and 186)
+  constexpr bool kAhead = NB == 1 && W == 16;
+  double abits = 0;
   auto fetch = [&](long t) {
     const long rr = point(t);
+    if (kAhead) abits = __ldg(&tscale[rr].y);
 #pragma unroll
     for (int b = 0; b < NB; ++b)
 #pragma unroll
@@ -197,6 +205,7 @@ __global__ void __launch_bounds__(W * 32 + 32, 16 / W) k1d_fixed_kernel(
   for (long t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const bool live = t * kR + lane < nr;
     const long rr = point(t);
+    if (!kAhead) abits = __ldg(&tscale[rr].y);
     // largest |a_v| of every point, then a as limbs
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
@@ -213,9 +222,9 @@ __global__ void __launch_bounds__(W * 32 + 32, 16 / W) k1d_fixed_kernel(
     for (int b = 0; b < NB; ++b) {
       const unsigned m = top[b * kR + lane];
       const int e = exp_above(m);
-      ascale[b] = scale_of(m, e - 53 + 54);  // unit of a times the 2^54 of `rounded`
+      ascale[b] = scale_of(m, e);
       auto put = [&](int v, double xv) {
-        a_s[((size_t)b * nocc + v) * kR + lane] = limbs(to_fixed(xv, e, 53));
+        a_s[((size_t)b * nocc + v) * kR + lane] = limbs(to_fixed(xv, e, (int)abits));
         y_s[((size_t)b * nocc + v) * kR + lane] = 0;
       };
 #pragma unroll
@@ -339,7 +348,7 @@ __global__ void __launch_bounds__(W * 32 + 32, 16 / W) k1d_fixed_kernel(
       consumers_sync<W>();  // the rows of column c are complete up to here for role B of later columns
     }
     if (!ok || !live) continue;
-    const double ts = tscale[rr], V = use_vloc ? vloc[rr] : 0.0;
+    const double ts = tscale[rr].x, V = use_vloc ? vloc[rr] : 0.0;
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
       if (b0 + b >= nb_total) break;
@@ -416,29 +425,67 @@ __global__ void __launch_bounds__(256) tile_kernel(long nr, int np, int nocc, lo
   if (r < nr) atomicMax(&top[r], m);
 }
 
-// doubles -> limbs in place, relative to the power of two above the point's largest pair
-__global__ void __launch_bounds__(256) fix_kernel(long nr, long npairs, int bits, const unsigned *__restrict__ top,
-                                                  double *__restrict__ tau) {
-  const long per = npairs * kR, total = (nr + kR - 1) / kR * per;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
-    const long r = i / per * kR + i % kR;
-    const int2 l = r < nr ? limbs(to_fixed(tau[i], exp_above(top[r]), bits)) : make_int2(0, 0);
-    *reinterpret_cast<int2 *>(&tau[i]) = l;
+// Doubles -> limbs in place, relative to the power of two above the point's largest pair, and the point's scale:
+// (unit of the sums for max|a| < 1, bits of a).  One CTA per tile; a warp takes whole columns v (sum over
+// v' <= v in a register, the mirror terms by shared-memory integer atomics), in units of 2^36 rounded up.
+//   th ah: C 2^36 2^(53 + s) / 2^54 <= 1.25 2^62;   th al + tl ah: C 2^36 / 2 + N_occ 2^(52 + s) < 2^63,
+// the latter by s <= 4, 3 or 2 for up to 64, 128 or more orbitals; C <= N_occ (2^20 + 1), so s >= -1 up to 261.
+// Bound by the read and write of tau (63-well cell 24.6 GB each).
+__global__ void __launch_bounds__(256) fix_kernel(long nr, int nocc, long npairs, const unsigned *__restrict__ top,
+                                                  double *__restrict__ tau, double2 *__restrict__ scale) {
+  extern __shared__ unsigned csum[];  // [nocc][32]
+  __shared__ unsigned cmax[kR];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long ntiles = (nr + kR - 1) / kR;
+  const int smax = nocc <= 64 ? 4 : nocc <= 128 ? 3 : 2;
+  for (long t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const long r = t * kR + lane;
+    const bool live = r < nr;
+    const unsigned hi = live ? top[r] : 0;
+    const int e = exp_above(hi);
+    double *tile = tau + (size_t)t * npairs * kR + lane;
+    for (int v = warp; v < nocc; v += 8) csum[v * kR + lane] = 0;
+    if (warp == 0) cmax[lane] = 0;
+    __syncthreads();
+    for (int v = warp; v < nocc; v += 8) {
+      unsigned col = 0;
+      for (int v0 = 0; v0 <= v; v0 += 8) {  // eight loads in flight
+        double x[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = v0 + i <= v && live ? tile[fixed_slot(v0 + i, v, nocc) * kR] : 0.0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int vp = v0 + i;
+          if (vp > v) break;
+          const long long f = to_fixed(x[i], e, kTauBits);
+          *reinterpret_cast<int2 *>(&tile[fixed_slot(vp, v, nocc) * kR]) = limbs(f);
+          const unsigned m = (unsigned)((f < 0 ? -f : f) >> 36) + 1;
+          col += m;
+          if (vp != v) atomicAdd(&csum[vp * kR + lane], m);
+        }
+      }
+      atomicAdd(&csum[v * kR + lane], col);
+    }
+    __syncthreads();
+    unsigned c = 0;
+    for (int v = warp; v < nocc; v += 8) c = max(c, csum[v * kR + lane]);
+    atomicMax(&cmax[lane], c);
+    __syncthreads();
+    if (warp == 0 && live) {
+      int s = smax;
+      while (s > -1 && ((unsigned long long)cmax[lane] << (s + 1)) > (5ull << 26)) --s;  // C 2^s <= 1.25 2^27
+      scale[r] = make_double2(scale_of(hi, e - kTauBits + 1 - s), 53 + s);
+    }
+    __syncthreads();
   }
 }
-__global__ void scale_kernel(long nr, int bits, const unsigned *__restrict__ top, double *__restrict__ scale) {
-  const long r = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  if (r < nr) scale[r] = scale_of(top[r], exp_above(top[r]) - bits);
-}
-
-int tau_bits(int nocc) { return nocc <= 128 ? 56 : nocc <= 256 ? 55 : 54; }
 
 }  // namespace
 
 // From 16 orbitals on, as long as the limbs and sums of one vector fit beside the stages.  With 16 orbitals on
 // 24^3 one vector takes 13.5 us (FP64 kernel 22.7); with 8 it would take 9.0 (12.2) and with 4 7.9 (7.1),
 // which the read of the error flag after the call (about 8 us) outweighs.
-bool k1d_fixed_supported(int nocc) { return nocc >= 16 && nocc <= 512 && shape_for(1, nocc).stages > 0; }
+bool k1d_fixed_supported(int nocc) { return nocc >= 16 && shape_for(1, nocc).stages > 0; }
 
 size_t k1d_tiled_size(long npairs, long nr) { return (size_t)npairs * ((nr + kR - 1) / kR * kR); }
 
@@ -449,13 +496,10 @@ void k1d_fixed_tile(const Ctx &c, int np, const int2 *pairs, const double2 *P, d
   BSE_CHECK_LAUNCH();
 }
 
-void k1d_fixed_finish(const Ctx &c, double *tau, const unsigned *top, double *scale) {
-  const long npairs = (long)c.nocc * (c.nocc + 1) / 2;
-  const int bits = tau_bits(c.nocc);
-  const long total = (c.nr + kR - 1) / kR * kR * npairs;
-  fix_kernel<<<(int)std::min<long>(152L * 64, (total + 255) / 256), 256, 0, c.stream>>>(c.nr, npairs, bits, top, tau);
-  BSE_CHECK_LAUNCH();
-  scale_kernel<<<(unsigned)((c.nr + 255) / 256), 256, 0, c.stream>>>(c.nr, bits, top, scale);
+void k1d_fixed_finish(const Ctx &c, double *tau, const unsigned *top, double2 *scale) {
+  const long npairs = (long)c.nocc * (c.nocc + 1) / 2, ntiles = (c.nr + kR - 1) / kR;
+  fix_kernel<<<(unsigned)std::min<long>(ntiles, 152L * 8), 256, (size_t)c.nocc * kR * 4, c.stream>>>(
+      c.nr, c.nocc, npairs, top, tau, scale);
   BSE_CHECK_LAUNCH();
 }
 

@@ -431,9 +431,15 @@ void dgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A,
     return;
   }
   // few output rows, short K, long N: one column per thread, a stream over B.  Against the digit form
-  // (exponent pass and rewriting of B), N = 200000: M = 2 K = 8 10 us (120), M = 2 K = 100 82 (343),
-  // M = 8 K = 8 64 (122), M = 8 K = 100 686 (347); N = 6859: M = 4 K = 64 19 (14), M = 8 K = 8 13 (11)
-  if (tb == 'N' && M <= kSmallM && K <= 1024 && N >= 4096 && (M <= 4 || M * K <= 96)) {
+  // (exponent pass and rewriting of B), us.  N = 200000: M = 2 K = 8 10 (90), M = 4 K = 256 390 (592), M = 8
+  // K = 8 60 (90), M = 8 K = 16 124 (93); N = 20000: M = 4 K = 256 67 (92), M = 8 K = 8 11 (16), M = 8 K = 16 20
+  // (17).  Below 16384 columns there are few threads and a column's chain shows, N = 6859: M = 2 K = 100 15 (21),
+  // M = 2 K = 256 35 (34), M = 3 K = 64 14.2 (14.6), M = 4 K = 32 10.1 (10.4), M = 4 K = 64 18 (15), M = 8 K = 4
+  // 6.9 (8.0), M = 8 K = 8 11 (8), M = 16 K = 4 7.3 (9.3); entrywise, with the checked digit form, M = 2 K = 256 35
+  // (39), M = 3 K = 100 21 (25), M = 4 K = 64 18 (18)
+  const bool few =
+      N >= 16384 ? M <= 4 || M * K <= 96 : M <= 4 ? M * M * K <= (entrywise ? 1100 : 600) : K <= 4;
+  if (tb == 'N' && M <= kSmallM && K <= 1024 && N >= 4096 && few) {
     const size_t smem = (size_t)M * K * sizeof(double);
     const int grid = (N + 255) / 256;
     auto go = [&](auto ta_c, auto mt_c) {

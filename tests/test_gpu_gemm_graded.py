@@ -3,7 +3,7 @@
 
 Data: A diag(s) and diag(1/s) B with s between 10^-r and 10^r, disjoint supports (the bound is 0), rotations close
 to the identity, a huge entry per row that meets a zero.  Shapes with one K slice and with many, every
-orientation, sizes that 16-row strips do not divide."""
+orientation, sizes that 16-row strips do not divide, and few rows on both sides of the streaming kernel's rule."""
 import numpy as np
 import pytest
 
@@ -43,6 +43,7 @@ def _operands(kind, M, N, K, rng):
                                   "spike"])
 @pytest.mark.parametrize("ta,tb,M,N,K", [
     ("N", "T", 1, 1, 2), ("N", "T", 5, 5, 31), ("N", "N", 40, 301, 48), ("T", "N", 33, 130, 257), ("T", "T", 65, 20, 500),
+    ("N", "N", 4, 4100, 68), ("N", "N", 4, 4100, 69), ("T", "N", 2, 4111, 276), ("N", "N", 9, 5000, 5),
     ("N", "N", 60, 1500, 130), ("N", "T", 17, 33, 900), ("N", "T", 80, 70, 3001)])
 def test_entrywise_bound(pkg, kind, ta, tb, M, N, K):
     rng = np.random.default_rng(M + 10 * N + 100 * K)

@@ -191,9 +191,9 @@ def mid48(**kw):
     N_occ = 48, N_pdep = 96, lambda_i = -0.6 exp(-i/40).  Each well binds one s-like and three
     p-like states, so the 48 occupied states are bound and the HOMO-LUMO gap is 0.45 Ha.  Sized
     for element-wise parity of the multi-block kernel paths against the oracle: three 16-orbital
-    blocks (off-diagonal blocks of the tiled contraction), 1176 pairs (several pair batches of
-    the tau build), 46656 grid points (a ragged last tile of 128 points, 1458 tiles of 32 points
-    spread unevenly over the SMs)."""
+    blocks (off-diagonal blocks of the FP32 contraction) or six 8-orbital columns (FP64), 1176 pairs
+    (several pair batches of the tau build), 46656 grid points (1458 tiles of 32 points spread
+    unevenly over the SMs)."""
     return _wells("wells12-36^3-nocc48", 12.0, 12, 10.0, (36, 36, 36), 8.0, 0.8, 48, SEED_BASE + 48 + 1000, 3.0,
                   **kw)
 
@@ -201,8 +201,8 @@ def mid48(**kw):
 def mid40(**kw):
     """Cubic L = 11 bohr, 10 wells (Z = 8, sigma = 0.8, at least 3 bohr apart), 10 Ry, 30^3,
     N_occ = 40, N_pdep = 80, lambda_i = -0.6 exp(-i/40); HOMO-LUMO gap 0.46 Ha.  The shapes the
-    16-orbital tiling does not divide: 40 orbitals (a half-filled last orbital tile) and 27000 grid
-    points (not a whole number of 32- or 128-point tiles), 820 pairs."""
+    FP32 contraction's tiling does not divide: 40 orbitals (a half-filled last 16-orbital block) and
+    27000 grid points (a ragged last tile of 32), 820 pairs."""
     return _wells("wells10-30^3-nocc40", 11.0, 10, 10.0, (30, 30, 30), 8.0, 0.8, 40, SEED_BASE + 40, 3.0, **kw)
 
 

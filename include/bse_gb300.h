@@ -107,7 +107,11 @@ typedef struct {
   int pdep_on_device;
   double scissor;             /* Ha: H^QP = H^KS + P_c scissor (Table S1, "BSE-Scissor") */
   int spin;                   /* 0 singlet D + 2K1e - K1d; 1 triplet D - K1d */
-  int precision;              /* 0 = FP64 throughout */
+  int precision;              /* 0: FP64 data; inside the operators matrix products, transforms and the
+                                 K1d sum run in integers of 52 to 62 bits relative to the largest entry
+                                 of a matrix row, of a plane of a grid (or of 32 columns of one) and of
+                                 a grid point, with errors relative to that entry no larger than FP64
+                                 arithmetic's; 1: FP32 grids, tau and PDEP products, FP64 solvers */
   int flags;                  /* BSE_FLAG_* */
   void *stream;               /* cudaStream_t to order all work on; NULL = context-owned stream */
   double gs_tol;              /* ground-state residual-norm target ||H phi - eps phi||; 0 = 1e-11 */
@@ -144,7 +148,7 @@ typedef struct {
   int wannier_pairs;          /* K1d pairs kept under BSE_FLAG_WANNIER_PRUNE (of n_occ (n_occ + 1)/2) */
   int wannier_sweeps;         /* Jacobi sweeps of the localisation */
   int tuned_xy_threads;       /* its choice: threads per plane-pass CTA of the sphere-pruned transforms
-                                 (0: the default, 512) */
+                                 (0: the default, by the planes that share an SM) */
   int tuned_gemm_split_pct;   /* its choice: split-K of the occupied-projection GEMMs, percent of the
                                  library's heuristic (100: the heuristic) */
   int zvector_graphed;        /* 1 when the last Z-vector conjugate-gradient solve ran as one captured

@@ -246,8 +246,9 @@ __global__ void __launch_bounds__(256) drho_kernel(long nr, int nocc, int nb, in
   }
 }
 
-// Y_{b,v}(r) = V(r) a_{b,v} + 2 vH_b phi_v - sum_v' tau_{v'v} a_{b,v'}  (Eqs. 2a-2c on the grid), for fewer than 16
-// orbitals and without K1d (k1d_tma.cu and k1d_fixed.cu stream tau for the others)
+// Y_{b,v}(r) = V(r) a_{b,v} + 2 vH_b phi_v - sum_v' tau_{v'v} a_{b,v'}  (Eqs. 2a-2c on the grid), without K1d, for
+// fewer than 16 orbitals and for more than the tiles of the kernels that stream tau hold (k1d_fixed.cu: 261;
+// k1d_tma.cu: 640)
 template <class R, int NB, int TV>
 __global__ void __launch_bounds__(128) combine_tau_kernel(
     long nr, int nocc, int nb_total, int b0, const R *__restrict__ phir,

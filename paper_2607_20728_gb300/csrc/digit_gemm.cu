@@ -686,6 +686,12 @@ size_t digit_scratch(int M, int N, int K) {
   return ((size_t)M + N + 1) / 2 + (slices > 1 ? slices * M * N : 0);
 }
 
+void splitk_sum(int M, int N, int nsplit, const double *part, double alpha, double beta, double *C, int ldc,
+                cudaStream_t s) {
+  digit_reduce<false><<<(unsigned)(((long)M * N + 31) / 32), 256, 0, s>>>(M, N, nsplit, part, alpha, beta, C, ldc, {});
+  BSE_CHECK_LAUNCH();
+}
+
 void digit_gemm(char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda,
                 const double *B, int ldb, double beta, double *C, int ldc, cudaStream_t s, DevBuf<double> &scratch,
                 bool fixed, int split_pct, bool entrywise) {

@@ -129,6 +129,9 @@ void sgemm(char ta, char tb, int M, int N, int K, float alpha, const float *A, i
 void digit_gemm(char ta, char tb, int M, int N, int K, double alpha, const double *A, int lda,
                 const double *B, int ldb, double beta, double *C, int ldc, cudaStream_t s, DevBuf<double> &scratch,
                 bool fixed, int split_pct = 100, bool entrywise = false);
+// C = alpha sum_z part[z][M][N] + beta C
+void splitk_sum(int M, int N, int nsplit, const double *part, double alpha, double beta, double *C, int ldc,
+                cudaStream_t s);
 size_t digit_scratch(int M, int N, int K);  // the least scratch, in doubles
 // out[i] = sum_j X[i][j] * Y[i][j] for i < rows (part: scratch of the partial sums; the default is
 // a per-thread buffer)

@@ -95,19 +95,23 @@ __global__ void __launch_bounds__(256) sgemm_kernel(int M, int N, int K, int kch
   }
 }
 
-// Skinny inner products for at most four rows of A: part[z][i][j] = sum over the z-th K slice of
-// A[i][k] B[j][k] for i < MM and the kSkinnyRows rows j of B this block takes.  Threads stream
+// Inner products of few rows over a long K: part[z][i][j] = sum over the z-th K slice of A[i][k] B[j][k]
+// for the MM rows i of A (blockIdx.z: groups of MM, the last one clamped) and the kSkinnyRows rows j of B
+// that this block takes.  Threads stream
 // consecutive k (coalesced loads of every row; VEC: pairs of k as one 16-byte load, rows and slices
 // 16-byte aligned), keep the MM x kSkinnyRows products in registers, and reduce them through warp
 // shuffles and shared memory at the end: every element of B is read once, and the FP64 pipe bounds
 // the launch.
 constexpr int kSkinnyRows = 8;
 template <int MM, bool VEC>
-__global__ void __launch_bounds__(256) gemm_nt_skinny_kernel(int N, int K, int kchunk, const double *__restrict__ A,
+__global__ void __launch_bounds__(256) gemm_nt_skinny_kernel(int M, int N, int K, int kchunk, const double *__restrict__ A,
                                                              int lda, const double *__restrict__ B, int ldb,
                                                              double *__restrict__ part) {
   __shared__ double red[8][MM * kSkinnyRows];
-  const int j0 = blockIdx.x * kSkinnyRows;
+  const int j0 = blockIdx.x * kSkinnyRows, i0 = blockIdx.z * MM;
+  const double *Ar[MM];
+#pragma unroll
+  for (int i = 0; i < MM; ++i) Ar[i] = A + (long)min(i0 + i, M - 1) * lda;
   const int nj = min(kSkinnyRows, N - j0);
   const long k0 = (long)blockIdx.y * kchunk;
   const long k1 = min((long)K, k0 + kchunk);
@@ -119,7 +123,7 @@ __global__ void __launch_bounds__(256) gemm_nt_skinny_kernel(int N, int K, int k
   auto step = [&](long k) {
     double a[MM];
 #pragma unroll
-    for (int i = 0; i < MM; ++i) a[i] = __ldg(&A[(long)i * lda + k]);
+    for (int i = 0; i < MM; ++i) a[i] = __ldg(&Ar[i][k]);
 #pragma unroll
     for (int r = 0; r < kSkinnyRows; ++r) {
       if (r < nj) {
@@ -134,7 +138,7 @@ __global__ void __launch_bounds__(256) gemm_nt_skinny_kernel(int N, int K, int k
     for (long k = k0 + 2 * threadIdx.x; k + 1 < k1; k += 2 * blockDim.x) {
       double2 a[MM];
 #pragma unroll
-      for (int i = 0; i < MM; ++i) a[i] = __ldg(reinterpret_cast<const double2 *>(&A[(long)i * lda + k]));
+      for (int i = 0; i < MM; ++i) a[i] = __ldg(reinterpret_cast<const double2 *>(&Ar[i][k]));
 #pragma unroll
       for (int r = 0; r < kSkinnyRows; ++r) {
         if (r < nj) {
@@ -163,7 +167,7 @@ __global__ void __launch_bounds__(256) gemm_nt_skinny_kernel(int N, int K, int k
     const int i = threadIdx.x / kSkinnyRows, r = threadIdx.x % kSkinnyRows;
     double v = 0.0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[w][threadIdx.x];
-    if (r < nj) part[((long)blockIdx.y * MM + i) * N + j0 + r] = v;
+    if (r < nj && i0 + i < M) part[((long)blockIdx.y * M + i0 + i) * N + j0 + r] = v;
   }
 }
 
@@ -378,24 +382,29 @@ int skinny_slots() {
   return slots;
 }
 
+// 16-byte loads of every row
+bool rows_aligned(const double *A, int lda, const double *B, int ldb) {
+  return ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) == 0 && lda % 2 == 0 && ldb % 2 == 0;
+}
+
 template <int MM, bool VEC>
-void skinny_launch(int N, int K, const double *A, int lda, const double *B, int ldb, double alpha, double beta,
-                   double *C, int ldc, cudaStream_t s, DevBuf<double> *fixed, DevBuf<double> &scratch) {
-  const int nb = (N + kSkinnyRows - 1) / kSkinnyRows;
-  int nsplit = std::max(1, std::min(K / 2048, skinny_slots<MM, VEC>() / nb));
-  if (fixed) nsplit = (int)std::max<size_t>(1, std::min<size_t>(nsplit, fixed->n / ((size_t)MM * N)));
+void skinny_launch(int M, int N, int K, const double *A, int lda, const double *B, int ldb, double alpha, double beta,
+                   double *C, int ldc, cudaStream_t s, DevBuf<double> *fixed, DevBuf<double> &scratch,
+                   bool column = false) {
+  const int nb = (N + kSkinnyRows - 1) / kSkinnyRows, ng = (M + MM - 1) / MM;
+  int nsplit = std::max(1, std::min(K / 2048, skinny_slots<MM, VEC>() / (nb * ng)));
+  if (fixed) nsplit = (int)std::max<size_t>(1, std::min<size_t>(nsplit, fixed->n / ((size_t)M * N)));
   int kchunk = (K + nsplit - 1) / nsplit;
   kchunk += kchunk & 1;  // even slice starts keep the 16-byte loads aligned
   nsplit = (K + kchunk - 1) / kchunk;
   DevBuf<double> &p = fixed ? *fixed : scratch;
-  if (!fixed) p.alloc((size_t)nsplit * MM * N);
-  gemm_nt_skinny_kernel<MM, VEC><<<dim3((unsigned)nb, (unsigned)nsplit), 256, 0, s>>>(N, K, kchunk, A, lda, B, ldb,
-                                                                                    p.get());
+  if (!fixed) p.alloc((size_t)nsplit * M * N);
+  gemm_nt_skinny_kernel<MM, VEC><<<dim3((unsigned)nb, (unsigned)nsplit, (unsigned)ng), 256, 0, s>>>(
+      M, N, K, kchunk, A, lda, B, ldb, p.get());
   BSE_CHECK_LAUNCH();
-  const long total = (long)MM * N;
-  splitk_reduce<double><<<(int)std::min<long>(4096, (total + 255) / 256), 256, 0, s>>>(MM, N, nsplit, p.get(), alpha,
-                                                                                        beta, C, ldc);
-  BSE_CHECK_LAUNCH();
+  // column: the one row of outputs is the column C[0..N)[0] of the caller
+  if (column) splitk_sum(N, 1, nsplit, p.get(), alpha, beta, C, ldc, s);
+  else splitk_sum(M, N, nsplit, p.get(), alpha, beta, C, ldc, s);
 }
 
 }  // namespace
@@ -412,15 +421,27 @@ void dgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A,
     }
     return;
   }
-  // at most four rows of A against any number of rows of B over a very long K (the Davidson
-  // subspace products of trial vectors): register-blocked streaming, split over K
-  if (ta == 'N' && tb == 'T' && M <= 4 && K >= 65536 && (!fixed || fixed->n >= (size_t)M * N * 8)) {
-    const bool vec = ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) == 0 &&
-                     (lda % 2) == 0 && (ldb % 2) == 0;
+  // few outputs over a very long K (the Davidson subspace products of trial vectors, the Gram rows of the density
+  // mixing): register-blocked FP64 streaming in groups of four rows, split over K, while the digit form's exponent
+  // pass and rewriting cost a microsecond per 1000 k whatever the outputs.  Time against the digit form, us:
+  // K = 878000: 3 x 16 95 (1115), 5 x 40 488 (1362), 16 x 16 392 (1147), 8 x 96 1173 (1707), 30 x 30 1682 (1315);
+  // K = 65536: 4 x 64 61 (88), 16 x 16 61 (73), 20 x 20 86 (85), 30 x 30 153 (86); K = 32768: 1 x 1 12 (39), 4 x 64
+  // 33 (49), 16 x 16 33 (42), 5 x 40 61 (49); K = 16384: 3 x 16 25 (25), 16 x 16 33 (26).  A single row of B takes
+  // the place of A (8 x 1 x 373248 74 -> 21; digit form 360).
+  if (ta == 'N' && tb == 'T' && N == 1 && M > 4 && K >= 32768 && (!fixed || fixed->n >= (size_t)M * 8)) {
+    const bool vec = rows_aligned(A, lda, B, ldb);
+    if (vec) skinny_launch<1, true>(1, M, K, B, ldb, A, lda, alpha, beta, C, ldc, s, fixed, splitk_buf(), true);
+    else skinny_launch<1, false>(1, M, K, B, ldb, A, lda, alpha, beta, C, ldc, s, fixed, splitk_buf(), true);
+    return;
+  }
+  const long padded = M <= 4 ? 0 : (M + 3L) / 4 * 4 * N;  // outputs of whole groups
+  const bool stream = K >= 65536 ? padded <= 768 : K >= 32768 && padded <= 256;
+  if (ta == 'N' && tb == 'T' && stream && (!fixed || fixed->n >= (size_t)M * N * 8)) {
+    const bool vec = rows_aligned(A, lda, B, ldb);
     auto go = [&](auto mm_c) {
       constexpr int MM = decltype(mm_c)::value;
-      if (vec) skinny_launch<MM, true>(N, K, A, lda, B, ldb, alpha, beta, C, ldc, s, fixed, splitk_buf());
-      else skinny_launch<MM, false>(N, K, A, lda, B, ldb, alpha, beta, C, ldc, s, fixed, splitk_buf());
+      if (vec) skinny_launch<MM, true>(M, N, K, A, lda, B, ldb, alpha, beta, C, ldc, s, fixed, splitk_buf());
+      else skinny_launch<MM, false>(M, N, K, A, lda, B, ldb, alpha, beta, C, ldc, s, fixed, splitk_buf());
     };
     switch (M) {
       case 1: go(std::integral_constant<int, 1>()); break;
@@ -467,7 +488,7 @@ void dgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A,
   // kernels that stood here (64 x 64 tiles, bound by the FP64 pipe or, below about 20 Mflop, by its
   // latency): N T 80 x 216 x 6859 72 us (383 before), 200 x 216 x 922 34 (121), 128 x 128 x 6859 56 (205),
   // 16 x 16 x 500 15 (86); N N 128 x 6859 x 128 71 (210), 128 x 373248 x 128 3.0 ms (10.0), 4 x 4 x 8 7 us
-  // (18); no shape of 1..512 x 1..373248 x 1..200000 was found where they were faster
+  // (18); a few outputs over a long K, where they were faster, go to the streaming kernel above
   // a fixed buffer too small for the whole product (millions of rows, or more than 2^19 k): in parts, so that a
   // captured launch never holds the address of a buffer that can grow
   if (fixed && fixed->n < digit_scratch(M, N, K) && M * (long)N > 1) {

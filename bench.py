@@ -44,7 +44,7 @@ NCU_TRAFFIC = {
     "43020757bf6c12d0": {"tau_factor": 1.0},
     # k1d_fixed_kernel (FP64), N_occ = 64, 2-vector block: 7.02 GB read + 0.49 GB written against 7.18 GB
     # algorithmic (tau 6.21 GB read once); profiles/k1d_fixed_nocc64_fp64.md
-    "426ae02a0244db73": {"tau_factor": 1.0},
+    "35ebeef3a54e430a": {"tau_factor": 1.0},
 }
 
 

@@ -333,9 +333,10 @@ __global__ void __launch_bounds__(kXYThreads) sph_xy(SphArgs<C> a, C *__restrict
 // Each is an upper bound taken from the leading 21 bits.  Rounding is at 2^-61 of those sums: against extended
 // precision (flat data, 24^3 to 72^3) the relative error of a transform is 1.0-2.1e-16, as FP64 3.1-4.1e-16.
 // 64 packed grids of the 63-well cell (72^3, 4608 planes), FP64 pass -> this one: inverse 1490 -> 502 us,
-// forward 1595 -> 669, H product 2710 -> 1017.  Bound by instruction issue (57 thousand warp instructions a
-// plane, 42% of the issue slots used: few warps and a barrier per stage).  Measured and not kept: radices
-// 8 3 3 for 72 (566 and 685 us), the plane in chunks of rows so that two CTAs share an SM (679 and 659).
+// forward 1595 -> 669, H product 2710 -> 1017.  Bound by instruction issue (61 and 70 thousand warp
+// instructions a plane, 46% and 42% of the issue slots used: few warps and a barrier per stage).  Measured
+// and not kept: radices 8 3 3 for 72 (566 and 685 us), the plane in chunks of rows so that two CTAs share an
+// SM (679 and 659).
 struct FxArgs {
   int N1, N2, N3, ncols_pad, nxs;
   long nr;

@@ -22,9 +22,10 @@
 // and the result is an FP64 product entry by entry, whatever the grading of rows and columns: row_exponents
 // also returns sA and sB, the kernel estimates S by one more product per tile and 16 k, of the first two digits'
 // magnitudes rounded to BF16, and the outputs it finds weak are dealt to whole warps, or summed together when a tile
-// has many.  Kernel time with CHECK (without): N T 80 x 216 x 6859 72 us (67), N N 80 x 2400 x 64 23 (20), T N
-// 200 x 6859 x 128 114 (115); with every output weak 302, 54 and 419 (as tiled FP64 kernels 384, 69 and 391).
+// has many.  Kernel time with CHECK (without): N T 80 x 216 x 6859 69 us (66), N N 80 x 2400 x 64 20.5 (19.5), T N
+// 200 x 6859 x 128 111 (114); with every output weak 298, 53 and 417 (as tiled FP64 kernels 384, 69 and 391).
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 #include <type_traits>
 
@@ -87,128 +88,160 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const unsigned (&a)[4], 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// smallest e with |x| < 2^e for a row whose largest |x| has the bits m (0: any e)
-__device__ __forceinline__ int exponent_of(unsigned long long m) {
-  const int E = (int)(m >> 52);
-  if (E == 0x7ff) return kBadExp;
-  return E ? E - 1022 : m ? 64 - __clzll(m) - 1074 : 0;
-}
-
-// Running sum of |x| from above: sum 2^(E - 1043), E the largest biased exponent so far, every term rounded up to
-// its leading 21 bits below that (integers: the FP64 pipe would take longer than the loads)
-struct AbsSum {
+// Largest |x| of a row or of a slice of it, as the high word, with the low words or'ed; sums: also sum |x| from
+// above, every term as its leading 21 bits below the largest so far, in units of 2^(its biased exponent - 1043) and
+// rounded up (integers: the FP64 pipe would take longer than the loads)
+struct RowPart {
+  unsigned hi, lo;
   unsigned long long sum;
-  int E;
-  __device__ __forceinline__ void rescale(int to) {
-    if (to > E) {
-      const int d = to - E;
-      sum = sum ? (d > 63 ? 0 : sum >> d) + 1 : 0;
-      E = to;
+  __device__ __forceinline__ void raise(unsigned h) {
+    const unsigned d = (h >> 20) - (hi >> 20);
+    if (h > hi && d) sum = (d > 63 ? 0 : sum >> d) + 1;
+    hi = max(hi, h);
+  }
+  // eight values; zeros count for next to nothing, denormals as if normal
+  template <bool SUMS>
+  __device__ __forceinline__ void take(const double (&x)[8]) {
+    unsigned h[8], m = hi;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      h[i] = (unsigned)__double2hiint(x[i]) & 0x7fffffffu;
+      lo |= (unsigned)__double2loint(x[i]);
+      m = max(m, h[i]);
     }
+    if (SUMS) {
+      raise(m);
+      unsigned t = 8;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) t += ((h[i] & 0xfffffu) | 0x100000u) >> min((m >> 20) - (h[i] >> 20), 31u);
+      sum += t;
+    }
+    hi = m;
   }
-  __device__ __forceinline__ void add(unsigned long long bits) {  // of |x|
-    const unsigned h = (unsigned)(bits >> 32);
-    const int e = max((int)(h >> 20), 1);
-    rescale(e);
-    const unsigned m = (h & 0xfffffu) | (h >> 20 ? 0x100000u : 0u);
-    sum += bits ? (E - e > 31 ? 0u : m >> (E - e)) + 1u : 0u;
-  }
-  __device__ __forceinline__ void add(AbsSum o) {
-    const int to = max(E, o.E);
-    rescale(to);
-    o.rescale(to);
+  __device__ __forceinline__ void add(RowPart o) {
+    const unsigned h = max(hi, o.hi);
+    raise(h);
+    o.raise(h);
+    lo |= o.lo;
     sum += o.sum;
   }
+  // smallest e with |x| < 2^e (0 for a row of zeros, -1021 for denormals), and sum |x| / 2^e
+  __device__ __forceinline__ void store(int *ex, float *rsum) const {
+    const bool zero = (hi | lo) == 0;
+    *ex = hi >= 0x7ff00000u ? kBadExp : zero ? 0 : max((int)(hi >> 20), 1) - 1022;
+    if (rsum) *rsum = zero ? 0.f : fmaxf(0.5f, (float)sum * 0x1p-21f);
+  }
 };
+// how the rows of an operand are read: contiguous ones by a CTA or a warp each, those across the memory 32 by a CTA
+enum RowMode { kRowCta, kRowWarp, kRowAcross };
+constexpr int kSliceRow = 8192;   // k per CTA when rows are cut: contiguous ones
+constexpr int kSliceAcross = 512;  // and those across the memory
 
 // Exponents of the rows of op(A) and the columns of op(B): the smallest e with |x| < 2^e over the row,
 // kBadExp when a value is not finite; with CHECK also sum |x| / 2^e from above, 0 for a row of zeros.  Rows that
-// are contiguous in k take one CTA each; rows that lie across the memory (k strides by ld) go 32 to a CTA, 8 k
-// at a time, coalesced over the rows.
+// are contiguous in k take one CTA each, eight short or many ones share one; rows that lie across the memory (k
+// strides by ld) go 32 to a CTA, 8 k at a time, coalesced over the rows.  Few long rows are cut into sa (sb) slices of k,
+// whose parts combine_rows adds: with one CTA per 32 columns, 64 x 40 x 120000 (N N) took 3.6 ms a call, 0.93 as a
+// tiled FP64 product and 0.31 now, 8 x 64 x 6859 133 us, 115 and 54; as one CTA per row of one element 33 x 100000 x
+// 1 (N T) 218 us, now 192.
 template <bool CHECK>
-__global__ void __launch_bounds__(256) row_exponents(int M, int N, int K, bool a_across, const double *__restrict__ A,
-                                                     int lda, bool b_across, const double *__restrict__ B, int ldb,
-                                                     int nblk_a, int *__restrict__ ex, float *__restrict__ sums) {
-  __shared__ unsigned long long red[8][32];
-  __shared__ AbsSum sred[CHECK ? 8 : 1][32];
+__global__ void __launch_bounds__(256) row_exponents(int M, int N, int K, RowMode a_mode, const double *__restrict__ A,
+                                                     int lda, RowMode b_mode, const double *__restrict__ B, int ldb,
+                                                     int nblk_a, int sa, int sb, int *__restrict__ ex,
+                                                     float *__restrict__ rsum, RowPart *__restrict__ parts) {
+  __shared__ RowPart red[8][32];
   const bool isb = (int)blockIdx.x >= nblk_a;
-  const int blk = isb ? blockIdx.x - nblk_a : blockIdx.x;
-  const bool across = isb ? b_across : a_across;
+  const int ns = isb ? sb : sa, idx = isb ? blockIdx.x - nblk_a : blockIdx.x;
+  int blk = idx, slice = 0, kbeg = 0, kend = K;
+  if (ns > 1) {
+    blk = idx / ns;
+    slice = idx - blk * ns;
+    kbeg = (int)((long)K * slice / ns);
+    kend = (int)((long)K * (slice + 1) / ns);
+  }
+  const RowMode mode = isb ? b_mode : a_mode;
   const double *X = isb ? B : A;
-  const int ld = isb ? ldb : lda, rows = isb ? N : M;
-  int *out = ex + (isb ? M : 0);
-  float *sout = sums + (isb ? M : 0);
-  AbsSum t{0, 1};
-  auto sum_of = [](AbsSum a, unsigned long long top) {
-    const int e = exponent_of(top);
-    if (top == 0 || e == kBadExp) return 0.f;
-    return fmaxf(0.5f, (float)ldexp((double)a.sum, a.E - 1043 - e));
-  };
+  const int ld = isb ? ldb : lda, rows = isb ? N : M, out = isb ? M : 0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned long long m = 0;
-  auto bits = [](double x) { return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull; };
-  if (across) {
+  RowPart p{0, 0, 0};
+  // x[k stride] for k = k0, k0 + step, ... below kend, eight loads in flight
+  auto scan = [&](const double *x, long stride, int k0, int step) {
+    for (long k = k0; k < kend; k += 8 * step) {
+      double v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = k + i * step < kend ? __ldg(&x[(k + i * step) * stride]) : 0.0;
+      p.take<CHECK>(v);
+    }
+  };
+  auto emit = [&](int row) {
+    if (ns == 1) p.store(ex + out + row, CHECK ? rsum + out + row : nullptr);
+    else parts[(isb && sa > 1 ? (long)M * sa : 0) + (long)row * ns + slice] = p;
+  };
+  auto over_warp = [&] {
+    for (int w = 16; w > 0; w >>= 1) {
+      RowPart o;
+      o.hi = __shfl_xor_sync(0xffffffffu, p.hi, w);
+      o.lo = __shfl_xor_sync(0xffffffffu, p.lo, w);
+      o.sum = CHECK ? __shfl_xor_sync(0xffffffffu, p.sum, w) : 0;
+      p.add(o);
+    }
+  };
+  if (mode == kRowAcross) {
     const int row = blk * 32 + lane;
-    if (row < rows)
-#pragma unroll 8
-      for (int k = warp; k < K; k += 8) {
-        const unsigned long long x = bits(__ldg(&X[(long)k * ld + row]));
-        m = max(m, x);
-        if (CHECK) t.add(x);
-      }
-    red[warp][lane] = m;
-    if (CHECK) sred[warp][lane] = t;
+    if (row < rows) scan(X + row, ld, kbeg + warp, 8);
+    red[warp][lane] = p;
     __syncthreads();
     if (warp == 0 && row < rows) {
-      for (int w = 1; w < 8; ++w) m = max(m, red[w][lane]);
-      out[row] = exponent_of(m);
-      if (CHECK) {
-        for (int w = 1; w < 8; ++w) t.add(sred[w][lane]);
-        sout[row] = sum_of(t, m);
-      }
+      for (int w = 1; w < 8; ++w) p.add(red[w][lane]);
+      emit(row);
     }
+  } else if (mode == kRowWarp) {
+    const int row = blk * 8 + warp;
+    if (row >= rows) return;
+    scan(X + (long)row * ld, 1, lane, 32);
+    over_warp();
+    if (lane == 0) emit(row);
   } else {
-    const double *x = X + (long)blk * ld;
-#pragma unroll 8
-    for (int k = threadIdx.x; k < K; k += 256) {
-      const unsigned long long v = bits(__ldg(&x[k]));
-      m = max(m, v);
-      if (CHECK) t.add(v);
-    }
-    for (int w = 16; w > 0; w >>= 1) {
-      m = max(m, __shfl_xor_sync(0xffffffffu, m, w));
-      if (CHECK) {
-        AbsSum o;
-        o.sum = __shfl_xor_sync(0xffffffffu, t.sum, w);
-        o.E = __shfl_xor_sync(0xffffffffu, t.E, w);
-        t.add(o);
-      }
-    }
-    if (lane == 0) {
-      red[0][warp] = m;
-      if (CHECK) sred[0][warp] = t;
-    }
+    scan(X + (long)blk * ld, 1, kbeg + threadIdx.x, 256);
+    over_warp();
+    if (lane == 0) red[0][warp] = p;
     __syncthreads();
     if (threadIdx.x == 0) {
-      for (int w = 1; w < 8; ++w) m = max(m, red[0][w]);
-      out[blk] = exponent_of(m);
-      if (CHECK) {
-        for (int w = 1; w < 8; ++w) t.add(sred[0][w]);
-        sout[blk] = sum_of(t, m);
-      }
+      for (int w = 1; w < 8; ++w) p.add(red[0][w]);
+      emit(blk);
     }
   }
+}
+
+// the slices of the rows that were cut: one thread per row
+__global__ void __launch_bounds__(256) combine_rows(int M, int N, int sa, int sb, const RowPart *__restrict__ parts,
+                                                    int *__restrict__ ex, float *__restrict__ rsum) {
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= M + N) return;
+  const int ns = i < M ? sa : sb, row = i < M ? i : i - M;
+  if (ns == 1) return;
+  parts += (i >= M && sa > 1 ? (long)M * sa : 0) + (long)row * ns;
+  RowPart p = parts[0];
+#pragma unroll 8
+  for (int s = 1; s < ns; ++s) p.add(parts[s]);
+  p.store(ex + i, rsum ? rsum + i : nullptr);
 }
 
 // Whether an output needs the FP64 sum: a row or column is not finite, or the bound above exceeds half of an FP64
 // sum's.  S is overestimated by less than a tenth plus 2^-13 (sA + sB) (the digits left out), so an output that
 // passes does meet it; the other half is for the roundings of up to K/64 slices, alpha and beta.
-__device__ __forceinline__ bool weak(int ea, int eb, float sa, float sb, int K, float S) {
-  if (ea == kBadExp || eb == kBadExp) return true;
-  if (sa == 0.f || sb == 0.f) return false;
-  const float k = (float)K, s = sa + sb;
-  return !(S >= 1.1f * (0.125f * s + 0.006f * k) / (0.5f * k + 4.f) + 1.25e-4f * s);
-}
+struct Bound {
+  float c0, c1;  // S >= c0 + c1 (sA + sB)
+  explicit Bound(int K) {
+    const double per = 1.1 / (0.5 * K + 4.0);
+    c0 = (float)(0.006 * K * per);
+    c1 = (float)(0.125 * per + 1.25e-4);
+  }
+  __device__ __forceinline__ bool weak(int ea, int eb, float sa, float sb, float S) const {
+    if (ea == kBadExp || eb == kBadExp) return true;
+    return sa != 0.f && sb != 0.f && !(S >= c0 + c1 * (sa + sb));
+  }
+};
 // sum_k a[k sa] b[k sb] by a warp, the result in every lane
 __device__ __forceinline__ double warp_dot(const double *__restrict__ a, long sa, const double *__restrict__ b, long sb,
                                            int K) {
@@ -239,8 +272,8 @@ template <bool TA, bool TB, bool CHECK>
 __global__ void __launch_bounds__(kWarps * 32, 1)
     digit_gemm_kernel(int M, int N, int K, int kslice, int SM, int SN, const double *__restrict__ A, int lda,
                       const double *__restrict__ B, int ldb, const int *__restrict__ ex,
-                      const float *__restrict__ rsum, double alpha, double beta, double *__restrict__ C, int ldc,
-                      double *__restrict__ part, float *__restrict__ part_s) {
+                      const float *__restrict__ rsum, Bound bound, double alpha, double beta, double *__restrict__ C,
+                      int ldc, double *__restrict__ part, float *__restrict__ part_s) {
   constexpr int kRows = 16 * kMaxStrips<CHECK>;
   extern __shared__ __align__(16) unsigned char smem[];
   double *raw = reinterpret_cast<double *>(smem);                                  // [2][rows][kRawStride]
@@ -448,7 +481,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1)
       if (part) {
         part[(long)m * N + n] = v;
         if (CHECK) part_s[(long)m * N + n] = S;
-      } else if (CHECK && weak(ea, eb, rsum[m], rsum[M + n], K, S)) {
+      } else if (CHECK && bound.weak(ea, eb, rsum[m], rsum[M + n], S)) {
         list[atomicAdd(&nweak, 1)] = (m - m0) << 16 | (n - n0);
       } else {
         double *c = C + (long)m * ldc + n;
@@ -517,6 +550,7 @@ struct Operands {
   const int *ex;
   const float *rsum, *part_s;
   int K;
+  Bound bound;
 };
 
 // C = alpha sum_z part[z] + beta C: 32 outputs per CTA, the slices dealt to eight warps and their sums added
@@ -550,7 +584,7 @@ __global__ void __launch_bounds__(256) digit_reduce(int M, int N, int nsplit, co
     if (CHECK && i < total) {
       for (int w = 1; w < 8; ++w) S += sred[w][lane];
       const int m = (int)(i / N), n = M + (int)(i % N);
-      again = weak(op.ex[m], op.ex[n], op.rsum[m], op.rsum[n], op.K, S);
+      again = op.bound.weak(op.ex[m], op.ex[n], op.rsum[m], op.rsum[n], S);
     }
     if (CHECK) {
       const unsigned all = __ballot_sync(0xffffffffu, again);
@@ -584,13 +618,14 @@ struct Shape {
 };
 Shape choose(int M, int N, int K, size_t part_cap, int strips) {
   static const int opts[][2] = {{4, 4}, {5, 3}, {3, 5}, {2, 7}, {7, 2}, {6, 2}, {2, 6}, {3, 3}, {2, 4}, {4, 2}, {2, 2},
-                                {1, 8}, {8, 1}, {1, 4}, {4, 1}, {1, 1}};
+                                {1, 8}, {8, 1}, {1, 7}, {7, 1}, {1, 4}, {4, 1}, {1, 1}};
   const int ms = (M + 15) / 16, ns = (N + 15) / 16;
   Shape best{4, 4, K, 1};
   double bc = 1e300;
   for (auto &o : opts) {
     const int sm = o[0], sn = o[1];
     if (sm > ms + 1 || sn > ns + 1 || sm + sn > strips) continue;
+    if (sm + sn == 8 && std::max(sm, sn) == 7 && strips > 8) continue;  // in the place of 1 + 8
     const long tiles = (long)((ms + sm - 1) / sm) * ((ns + sn - 1) / sn);
     const double load = std::max(240.0 * (sm + sn), 172.0 * std::min(sm, ms) * std::min(sn, ns)) + 500.0;
     // a slice of at most kMaxSlice k keeps the 64-bit sums in range (2^50 per 128 k)
@@ -619,9 +654,16 @@ void go(dim3 grid, cudaStream_t s, int M, int N, int K, const Shape &h, const do
         float *part_s) {
   constexpr size_t smem = digit_smem<CHECK>();
   auto kernel = digit_gemm_kernel<TA, TB, CHECK>;
-  BSE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kernel<<<grid, kWarps * 32, smem, s>>>(M, N, K, h.kslice, h.sm, h.sn, A, lda, B, ldb, ex, rsum, alpha, beta, C, ldc,
-                                         part, part_s);
+  // the limit is an attribute of the function on a device, the same at every launch: set once (a microsecond a call)
+  static std::atomic<unsigned long long> set{0};
+  int dev = 0;
+  BSE_CUDA(cudaGetDevice(&dev));
+  if (dev >= 64 || !(set.load() >> dev & 1)) {
+    BSE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (dev < 64) set.fetch_or(1ull << dev);
+  }
+  kernel<<<grid, kWarps * 32, smem, s>>>(M, N, K, h.kslice, h.sm, h.sn, A, lda, B, ldb, ex, rsum, Bound(K), alpha, beta,
+                                         C, ldc, part, part_s);
   BSE_CHECK_LAUNCH();
 }
 
@@ -653,15 +695,36 @@ void run(char ta, char tb, int M, int N, int K, double alpha, const double *A, i
   }
   const long total = (long)M * N;
   const size_t npart = h.nsplit > 1 ? (size_t)h.nsplit * total : 0;
-  if (!fixed) scratch.alloc(nex + npart + (CHECK ? (npart + 1) / 2 : 0));
+  // CTAs of the exponent pass, and slices of k where they would leave the chip empty; the slices' parts lie where
+  // the partial sums come later
+  const bool TA = ta == 'T', TB = tb == 'T';
+  // (a warp per row of 600 entries: 4096 of them 20 -> 6 us)
+  auto mode = [&](bool across, int rows) {
+    return across ? kRowAcross : K <= 256 || (K <= 4096 && rows >= 1216) ? kRowWarp : kRowCta;
+  };
+  auto blocks = [](RowMode m, int rows) { return m == kRowAcross ? (rows + 31) / 32 : m == kRowWarp ? (rows + 7) / 8 : rows; };
+  auto slices = [&](RowMode m, int nblk) {
+    if (m == kRowWarp) return 1;
+    return std::max(1, std::min(K / (m == kRowAcross ? kSliceAcross : kSliceRow), 1216 / nblk));
+  };
+  const RowMode am = mode(TA, M), bm = mode(!TB, N);
+  const int ba = blocks(am, M), bb = blocks(bm, N);
+  int sa = slices(am, ba), sb = slices(bm, bb);
+  size_t nrow = ((sa > 1 ? (size_t)M * sa : 0) + (sb > 1 ? (size_t)N * sb : 0)) * sizeof(RowPart) / sizeof(double);
+  if (fixed && nrow > cap) sa = sb = 1, nrow = 0;
+  if (!fixed) scratch.alloc(nex + std::max(nrow, npart + (CHECK ? (npart + 1) / 2 : 0)));
   int *ex = reinterpret_cast<int *>(scratch.get());
   float *rsum = CHECK ? reinterpret_cast<float *>(ex + M + N) : nullptr;
   double *part = npart ? scratch.get() + nex : nullptr;
   float *part_s = CHECK && npart ? reinterpret_cast<float *>(part + npart) : nullptr;
-  const bool TA = ta == 'T', TB = tb == 'T';
-  const int ba = TA ? (M + 31) / 32 : M, bb = TB ? N : (N + 31) / 32;
-  row_exponents<CHECK><<<ba + bb, 256, 0, s>>>(M, N, K, TA, A, lda, !TB, B, ldb, ba, ex, rsum);
+  RowPart *parts = nrow ? reinterpret_cast<RowPart *>(scratch.get() + nex) : nullptr;
+  row_exponents<CHECK><<<ba * sa + bb * sb, 256, 0, s>>>(M, N, K, am, A, lda, bm, B, ldb, ba * sa, sa, sb, ex, rsum,
+                                                         parts);
   BSE_CHECK_LAUNCH();
+  if (parts) {
+    combine_rows<<<(M + N + 255) / 256, 256, 0, s>>>(M, N, sa, sb, parts, ex, rsum);
+    BSE_CHECK_LAUNCH();
+  }
   const dim3 grid((unsigned)((N + 16 * h.sn - 1) / (16 * h.sn)), (unsigned)((M + 16 * h.sm - 1) / (16 * h.sm)),
                   (unsigned)h.nsplit);
   auto launch = [&](auto a, auto b) {
@@ -673,7 +736,7 @@ void run(char ta, char tb, int M, int N, int K, double alpha, const double *A, i
   else if (TA && !TB) launch(std::true_type(), std::false_type());
   else launch(std::true_type(), std::true_type());
   if (part) {
-    const Operands op{A, B, TA ? 1 : lda, TA ? lda : 1, TB ? ldb : 1, TB ? 1 : ldb, ex, rsum, part_s, K};
+    const Operands op{A, B, TA ? 1 : lda, TA ? lda : 1, TB ? ldb : 1, TB ? 1 : ldb, ex, rsum, part_s, K, Bound(K)};
     digit_reduce<CHECK><<<(unsigned)((total + 31) / 32), 256, 0, s>>>(M, N, h.nsplit, part, alpha, beta, C, ldc, op);
     BSE_CHECK_LAUNCH();
   }
@@ -688,7 +751,9 @@ size_t digit_scratch(int M, int N, int K) {
 
 void splitk_sum(int M, int N, int nsplit, const double *part, double alpha, double beta, double *C, int ldc,
                 cudaStream_t s) {
-  digit_reduce<false><<<(unsigned)(((long)M * N + 31) / 32), 256, 0, s>>>(M, N, nsplit, part, alpha, beta, C, ldc, {});
+  digit_reduce<false><<<(unsigned)(((long)M * N + 31) / 32), 256, 0, s>>>(M, N, nsplit, part, alpha, beta, C, ldc,
+                                                                             Operands{nullptr, nullptr, 0, 0, 0, 0, nullptr,
+                                                                                      nullptr, nullptr, 0, Bound(0)});
   BSE_CHECK_LAUNCH();
 }
 

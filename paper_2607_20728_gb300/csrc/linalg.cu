@@ -426,16 +426,19 @@ void dgemm(char ta, char tb, int M, int N, int K, double alpha, const double *A,
   // pass and rewriting cost a microsecond per 1000 k whatever the outputs.  Time against the digit form, us:
   // K = 878000: 3 x 16 95 (1115), 5 x 40 488 (1362), 16 x 16 392 (1147), 8 x 96 1173 (1707), 30 x 30 1682 (1315);
   // K = 65536: 4 x 64 61 (88), 16 x 16 61 (73), 20 x 20 86 (85), 30 x 30 153 (86); K = 32768: 1 x 1 12 (39), 4 x 64
-  // 33 (49), 16 x 16 33 (42), 5 x 40 61 (49); K = 16384: 3 x 16 25 (25), 16 x 16 33 (26).  A single row of B takes
-  // the place of A (8 x 1 x 373248 74 -> 21; digit form 360).
-  if (ta == 'N' && tb == 'T' && N == 1 && M > 4 && K >= 32768 && (!fixed || fixed->n >= (size_t)M * 8)) {
+  // 33 (49), 16 x 16 33 (42), 5 x 40 61 (49); K = 16384: 1 x 1 11 (23), 4 x 64 33 (30; checked 35), 16 x 16 33 (26;
+  // 32); K = 4096: 1 x 1 11 (13; 17).  A single row of B takes the place of A (8 x 1 x 373248 74 -> 21; 360).
+  if (ta == 'N' && tb == 'T' && N == 1 && M > 4 && K >= 4096 && (!fixed || fixed->n >= (size_t)M * 8)) {
     const bool vec = rows_aligned(A, lda, B, ldb);
     if (vec) skinny_launch<1, true>(1, M, K, B, ldb, A, lda, alpha, beta, C, ldc, s, fixed, splitk_buf(), true);
     else skinny_launch<1, false>(1, M, K, B, ldb, A, lda, alpha, beta, C, ldc, s, fixed, splitk_buf(), true);
     return;
   }
   const long padded = M <= 4 ? 0 : (M + 3L) / 4 * 4 * N;  // outputs of whole groups
-  const bool stream = K >= 65536 ? padded <= 768 : K >= 32768 && padded <= 256;
+  const bool stream = M == 1      ? K >= 4096
+                      : M <= 4    ? K >= 16384
+                      : K >= 65536 ? padded <= 768
+                                   : padded <= 256 && K >= (entrywise ? 16384 : 32768);
   if (ta == 'N' && tb == 'T' && stream && (!fixed || fixed->n >= (size_t)M * N * 8)) {
     const bool vec = rows_aligned(A, lda, B, ldb);
     auto go = [&](auto mm_c) {

@@ -3,7 +3,8 @@
 
 Data: A diag(s) and diag(1/s) B with s between 10^-r and 10^r, disjoint supports (the bound is 0), rotations close
 to the identity, a huge entry per row that meets a zero.  Shapes with one K slice and with many, every
-orientation, sizes that 16-row strips do not divide, and few rows on both sides of the streaming kernel's rule."""
+orientation, sizes that 16-row strips do not divide, few rows on both sides of the streaming kernel's rule, and
+long rows whose largest entry and sum are found in slices (1025 and more across the memory, 16384 along it)."""
 import numpy as np
 import pytest
 
@@ -44,7 +45,8 @@ def _operands(kind, M, N, K, rng):
 @pytest.mark.parametrize("ta,tb,M,N,K", [
     ("N", "T", 1, 1, 2), ("N", "T", 5, 5, 31), ("N", "N", 40, 301, 48), ("T", "N", 33, 130, 257), ("T", "T", 65, 20, 500),
     ("N", "N", 4, 4100, 68), ("N", "N", 4, 4100, 69), ("T", "N", 2, 4111, 276), ("N", "N", 9, 5000, 5),
-    ("N", "N", 60, 1500, 130), ("N", "T", 17, 33, 900), ("N", "T", 80, 70, 3001)])
+    ("N", "N", 60, 1500, 130), ("N", "T", 17, 33, 900), ("N", "T", 80, 70, 3001),
+    ("N", "N", 8, 33, 6859), ("T", "N", 5, 40, 5000), ("T", "T", 33, 7, 1025), ("N", "T", 5, 6, 20000)])
 def test_entrywise_bound(pkg, kind, ta, tb, M, N, K):
     rng = np.random.default_rng(M + 10 * N + 100 * K)
     A, B = _operands(kind, M, N, K, rng)
@@ -70,3 +72,24 @@ def test_alpha_and_beta(pkg):
         torch.cuda.synchronize()
         pkg.bse_gemm("N", "N", -3.0, torch.tensor(A, device="cuda"), torch.tensor(B, device="cuda"), 1.0, c)
         assert (np.abs((c.cpu().numpy() - E).astype(np.float64)) <= tol).all()
+
+
+def test_non_finite_long_rows(pkg):
+    """A NaN or infinity in any slice of a long row or column reaches its outputs and no others."""
+    rng = np.random.default_rng(2)
+    K = 20000
+    A, B = rng.standard_normal((6, K)), rng.standard_normal((K, 40))
+    A[1, 3], A[4, K - 1], B[K // 2, 7], B[K - 2, 33] = np.inf, np.nan, -np.inf, np.nan
+    with np.errstate(invalid="ignore"):
+        E = A @ B
+    for ta, tb in (("N", "N"), ("T", "T")):
+        c = torch.zeros(6, 40, dtype=torch.float64, device="cuda")
+        a, b = torch.tensor(A, device="cuda"), torch.tensor(B, device="cuda")
+        a, b = (a.T.contiguous(), b.T.contiguous()) if ta == "T" else (a, b)
+        torch.cuda.synchronize()
+        pkg.bse_gemm(ta, tb, 1.0, a, b, 0.0, c)
+        got = c.cpu().numpy()
+        assert np.array_equal(np.isnan(got), np.isnan(E))
+        assert np.array_equal(got[np.isinf(E)], E[np.isinf(E)])
+        ok = np.isfinite(E)
+        assert np.abs(got[ok] - E[ok]).max() < 1e-10

@@ -1194,7 +1194,7 @@ DavOut davidson(Ctx &c, const DavSpec &sp, const double *X0, int k0, double *Xou
       auto te = clk::now();
       // vectors only for the Ritz pairs this iteration can use: the corrected block, and the
       // `keep` lowest when the new directions could overflow the subspace (a thick restart)
-      const bool may_restart = m + std::min(sp.block, m) > S;
+      const bool may_restart = m + std::min(sp.block, m) > S && (S < n - sp.nq || m == S);
       sym_eig_lowest(m, Hs.data(), std::min(m, may_restart ? std::max(sp.block, keep) : sp.block), w.data(),
                      Y.data(), false);
       c.stats.ms_host_eig += ms_since(te);
@@ -1239,7 +1239,10 @@ DavOut davidson(Ctx &c, const DavSpec &sp, const double *X0, int k0, double *Xou
     h2d(th.get(), thsel.data(), nsel * sizeof(double), c);
     sp.precond(nsel, T.get(), th.get());
     if (sp.project) sp.project(nsel, T.get());
-    if (m + nsel > S) {
+    // A subspace that may grow to the whole deflated space needs no restart: the new directions' rank is at most
+    // what is left of it.  With a restart whenever a block might not fit, a block of more than half the space (the
+    // loose empty states of a cell with 123 plane waves) restarted in every iteration and now and then stood still.
+    if (m + nsel > S && (S < n - sp.nq || m == S)) {
       // thick restart on the `keep` lowest Ritz vectors
       const int nk = std::min(std::max(keep, nb), m);
       if (nk == nb) {
